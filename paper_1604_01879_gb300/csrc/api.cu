@@ -204,7 +204,8 @@ __global__ void k_list_runs(const int64_t* __restrict__ list_off, const int64_t*
   }
 }
 
-__global__ void k_cb_maxnorm(const float* __restrict__ half_sq, int K, float* __restrict__ out) {
+// out = raise * max_k ||b_k||
+__global__ void k_cb_maxnorm(const float* __restrict__ half_sq, int K, float* __restrict__ out, float raise) {
   float m = 0.f;
   for (int k = threadIdx.x; k < K; k += blockDim.x) m = fmaxf(m, half_sq[k]);
 #pragma unroll
@@ -215,13 +216,13 @@ __global__ void k_cb_maxnorm(const float* __restrict__ half_sq, int K, float* __
   if (threadIdx.x == 0) {
     float r = 0.f;
     for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r = fmaxf(r, w[i]);
-    out[0] = sqrtf(2.f * r);
+    out[0] = sqrtf(2.f * r) * raise;
   }
 }
 
 }  // namespace
 
-void prepare_codebook(Index& ix, cudaStream_t s) {
+const float* prepare_codebook_async(Index& ix, Scratch& sc, cudaStream_t s) {
   const int K = ix.prm.n_codewords, D = ix.prm.dim;
   if (!ix.cb_half_sq) {
     ix.cb_half_sq = ix.alloc<float>(K);
@@ -233,13 +234,10 @@ void prepare_codebook(Index& ix, cudaStream_t s) {
   }
   launch_half_sq_norm(ix.codebook, K, D, ix.cb_half_sq, s);
   split_rows_bf16(ix.codebook, K, D, ix.cb_hi, ix.cb_lo, s);
-  Scratch sc(s);
   float* d_cbmax = sc.get<float>(1);
-  k_cb_maxnorm<<<1, 1024, 0, s>>>(ix.cb_half_sq, K, d_cbmax);
+  k_cb_maxnorm<<<1, 1024, 0, s>>>(ix.cb_half_sq, K, d_cbmax, 1.0001f);
   GIFT_LAUNCHED("k_cb_maxnorm");
-  GIFT_CUDA(cudaMemcpyAsync(&ix.cb_max_norm, d_cbmax, 4, cudaMemcpyDeviceToHost, s));
-  GIFT_CUDA(cudaStreamSynchronize(s));
-  ix.cb_max_norm *= 1.0001f;
+  return d_cbmax;
 }
 
 namespace {
@@ -605,7 +603,7 @@ void build(const gift_index_params* prm, const float* db_feats, const float* cod
   GIFT_CUDA(cudaMemsetAsync(ix->cb_lo, 0, (size_t)ix->cb_rows_alloc * D * 2, s));
   split_rows_bf16(ix->codebook, K, D, ix->cb_hi, ix->cb_lo, s);
   float* d_cbmax = sc.get<float>(1);
-  k_cb_maxnorm<<<1, 1024, 0, s>>>(ix->cb_half_sq, K, d_cbmax);
+  k_cb_maxnorm<<<1, 1024, 0, s>>>(ix->cb_half_sq, K, d_cbmax, 1.f);
   GIFT_LAUNCHED("k_cb_maxnorm");
 
   // FP32 master (kept for the exact match and the rescore; otherwise scratch)
@@ -750,7 +748,7 @@ void stream_begin(const gift_index_params* prm, const float* codebook, cudaStrea
   GIFT_CUDA(cudaMemsetAsync(ix->cb_lo, 0, (size_t)ix->cb_rows_alloc * D * 2, s));
   split_rows_bf16(ix->codebook, K, D, ix->cb_hi, ix->cb_lo, s);
   float* d_cbmax = sc.get<float>(1);
-  k_cb_maxnorm<<<1, 1024, 0, s>>>(ix->cb_half_sq, K, d_cbmax);
+  k_cb_maxnorm<<<1, 1024, 0, s>>>(ix->cb_half_sq, K, d_cbmax, 1.f);
   GIFT_LAUNCHED("k_cb_maxnorm");
   GIFT_CUDA(cudaMemcpyAsync(&ix->cb_max_norm, d_cbmax, 4, cudaMemcpyDeviceToHost, s));
   ix->row_inv = ix->alloc<float>(n_rows);

@@ -175,14 +175,24 @@ void launch_fill_i32(int32_t* p, int64_t n, int32_t v, cudaStream_t s);
 // k_assign.cu
 // codes[v*ma + a] = a-th nearest codeword by (squared distance, index);
 // x_inv (optional) holds 1/||x|| of the rows.
+// parts (optional, n <= kAssignChunk): the rows' two-part copy, made before;
+// cb_max (optional): the device value of ix.cb_max_norm.
+constexpr int64_t kAssignChunk = 131072;  // rows per quantiser pass
+struct SplitRows {
+  __nv_bfloat16* hi = nullptr;  // [n + padding, D]
+  __nv_bfloat16* lo = nullptr;
+};
+SplitRows split_for_assign(const float* X, int64_t n, int D, Scratch& sc, cudaStream_t s);
 void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* codes,
-                  Scratch& sc, cudaStream_t s, const float* x_inv = nullptr, KernelClock* kc = nullptr);
+                  Scratch& sc, cudaStream_t s, const float* x_inv = nullptr, KernelClock* kc = nullptr,
+                  const SplitRows* parts = nullptr, const float* cb_max = nullptr);
 // hi = bf16(x), lo = bf16(x - hi) of a row-major [n, D] FP32 matrix
 void split_rows_bf16(const float* X, int64_t n, int D, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t s);
 
 // api.cu: the quantiser's derived codebook arrays (||b||^2 / 2, two-part BF16
-// rows padded by one TMA box, max ||b||) from ix.codebook; allocates them on first use
-void prepare_codebook(Index& ix, cudaStream_t s);
+// rows padded by one TMA box) from ix.codebook, allocated on first use; returns max ||b||
+// (slightly raised) in device memory of sc, so that nothing waits for it
+const float* prepare_codebook_async(Index& ix, Scratch& sc, cudaStream_t s);
 
 // k_kmeans.cu: Lloyd's k-means from the rows init_rows; C_out [K, D] (device or host)
 void kmeans(const float* X, int64_t n, int D, int K, const std::vector<int32_t>& init_rows, int iters, float* C_out,

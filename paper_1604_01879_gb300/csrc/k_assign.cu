@@ -248,7 +248,8 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
                                                        const float* __restrict__ cb, int K, int ma,
                                                        const float* __restrict__ cval,
                                                        const int32_t* __restrict__ cidx, int nch,
-                                                       const float* __restrict__ x_inv, float bmax,
+                                                       const float* __restrict__ x_inv, float bmax_host,
+                                                       const float* __restrict__ bmax_dev,
                                                        int32_t* __restrict__ codes) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * 8 + w;
@@ -269,6 +270,7 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
     tp = bp;
     ++found;
   }
+  const float bmax = bmax_dev ? *bmax_dev : bmax_host;
   const float xi = x_inv[r];
   const float xn = xi > 0.f ? 1.0001f / xi : 0.f;
   const float E = 2.44140625e-4f * (xn * bmax + 0.5f * bmax * bmax) + 1e-30f;
@@ -410,15 +412,25 @@ void split_rows_bf16(const float* X, int64_t n, int D, __nv_bfloat16* hi, __nv_b
   GIFT_LAUNCHED("k_split_rows");
 }
 
+SplitRows split_for_assign(const float* X, int64_t n, int D, Scratch& sc, cudaStream_t s) {
+  SplitRows r;
+  const int64_t rows_alloc = n + tc::kTM;  // one box of padding rows
+  r.hi = sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
+  r.lo = sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
+  split_rows_bf16(X, n, D, r.hi, r.lo, s);
+  return r;
+}
+
 void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* codes, Scratch& sc, cudaStream_t s,
-                  const float* x_inv, KernelClock* kc) {
+                  const float* x_inv, KernelClock* kc, const SplitRows* parts, const float* cb_max) {
   if (n <= 0) return;
   const int K = ix.prm.n_codewords, D = ix.prm.dim;
   GIFT_REQUIRE(ma >= 1 && ma <= GIFT_MAX_MA && ma <= K, "multiple assignment must be in [1, min(8, K)]");
-  const int64_t chunk = std::min<int64_t>(n, 131072);
+  const int64_t chunk = std::min<int64_t>(n, kAssignChunk);
   const int64_t rows_alloc = chunk + tc::kTM;  // one box of padding rows
-  __nv_bfloat16* hi = sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
-  __nv_bfloat16* lo = sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
+  GIFT_REQUIRE(!parts || n <= chunk, "a two-part copy made before covers one pass");
+  __nv_bfloat16* hi = parts ? parts->hi : sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
+  __nv_bfloat16* lo = parts ? parts->lo : sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
   const int nch = (int)cdiv(K, TNA);
   float* cval = sc.get<float>((size_t)chunk * nch * kT);
   int32_t* cidx = sc.get<int32_t>((size_t)chunk * nch * kT);
@@ -433,7 +445,7 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
   const int sms = device_sm_count();
   for (int64_t r0 = 0; r0 < n; r0 += chunk) {
     const int64_t m = std::min(chunk, n - r0);
-    split_rows_bf16(X + r0 * D, m, D, hi, lo, s);
+    if (!parts) split_rows_bf16(X + r0 * D, m, D, hi, lo, s);
     AssignPolicy p;
     p.n = m;
     p.K = K;
@@ -452,7 +464,7 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
       kc->assign_rows += m;
     }
     k_assign_refine<<<(unsigned)cdiv(m, 8), 256, 0, s>>>(X + r0 * D, m, D, ix.codebook, K, ma, cval, cidx, nch,
-                                                          x_inv + r0, ix.cb_max_norm, codes + r0 * ma);
+                                                          x_inv + r0, ix.cb_max_norm, cb_max, codes + r0 * ma);
     GIFT_LAUNCHED("k_assign_refine");
   }
 }

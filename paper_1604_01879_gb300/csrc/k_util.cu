@@ -39,6 +39,7 @@ __global__ void k_half_sq_norm(const float* __restrict__ X, int64_t n, int D, fl
   if (row >= n) return;
   const float* p = X + row * (int64_t)D;
   float hi = 0.f, lo = 0.f;
+#pragma unroll 8
   for (int i = lane; i < D; i += 32) {
     const float x = p[i];
     const float pr = x * x;
