@@ -420,12 +420,12 @@ void run_fif(Index& ix, const float* q, int64_t nv, const std::vector<int32_t>& 
 
   tm.mark(ST_TOPK);
   if (R <= 0) {
-    topk_rows_f32(S, B, N, topk, out_ids, out_scores, sc, s);
+    topk_rows_f32(S, B, N, topk, out_ids, out_scores, s);
     return;
   }
   const int Rr = std::min(R, N);
   int32_t* cand = sc.get<int32_t>((size_t)B * Rr);
-  topk_rows_f32(S, B, N, Rr, cand, nullptr, sc, s);
+  topk_rows_f32(S, B, N, Rr, cand, nullptr, s);
   int32_t* cand_sorted = sc.get<int32_t>((size_t)B * Rr);
   sort_ids_rows(cand, B, Rr, cand_sorted, s);
 
@@ -966,7 +966,7 @@ gift_status gift_query(gift_index* index, const float* q_feats, const int32_t* q
       else
         gift::exact_scores_lists(ix, q, q_inv, nv, d_qoff, h, B, S, sc, stream);
       tm.mark(gift::ST_TOPK);
-      gift::topk_rows_f32(S, B, ix.prm.n_shapes, topk, oid, osc, sc, stream);
+      gift::topk_rows_f32(S, B, ix.prm.n_shapes, topk, oid, osc, stream);
     } else if (mode == GIFT_MATCH_FIF) {
       if (ix.prm.rescore_r > 0 && topk > std::min(ix.prm.rescore_r, ix.prm.n_shapes) && ix.prm.n_shapes >= topk)
         gift::fail(GIFT_EUNSUPPORTED, "topk exceeds the rescore depth");
@@ -1213,7 +1213,7 @@ gift_status gift_merge_topk(const int32_t* ids, const float* scores, int32_t B, 
     const float* cs = gift::stage_in(scores, (size_t)B * n, sc, stream);
     int32_t* oid = gift::stage_out(out_ids, (size_t)B * k, sc, outs);
     float* osc = gift::stage_out(out_scores, (size_t)B * k, sc, outs);
-    gift::merge_topk_rows(ci, cs, B, n, k, oid, osc, sc, stream);
+    gift::merge_topk_rows(ci, cs, B, n, k, oid, osc, stream);
     gift::flush_out(outs, stream);
   });
 }

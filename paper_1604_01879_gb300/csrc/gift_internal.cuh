@@ -216,9 +216,9 @@ void exact_scores_lists(const Index& ix, const float* q, const float* q_inv, int
 // largest by (value desc, index asc). ids_out/val_out [B, k] (val_out may be
 // null). When n < k the tail gets id -1 and -INF.
 void topk_rows_f32(const float* scores, int32_t B, int64_t n, int32_t k, int32_t* ids_out,
-                   float* val_out, Scratch& sc, cudaStream_t s);
+                   float* val_out, cudaStream_t s);
 void topk_rows_u64(const uint64_t* keys, int32_t B, int64_t n, int32_t k, int32_t* ids_out,
-                   uint64_t* key_out, Scratch& sc, cudaStream_t s);
+                   uint64_t* key_out, cudaStream_t s);
 // Rows of (id, score) pairs of length r: sort by (score desc, id asc) and keep k.
 void sort_candidates(const int32_t* ids, const float* scores, int32_t B, int32_t r, int32_t k,
                      int32_t* ids_out, float* scores_out, cudaStream_t s);
@@ -227,7 +227,7 @@ void sort_ids_rows(const int32_t* ids, int32_t B, int32_t r, int32_t* out, cudaS
 // Rows of (id, score) pairs of any length n (ids distinct per row, id < 0 =
 // none): the k best by (score desc, id asc); missing entries id -1, -INF.
 void merge_topk_rows(const int32_t* ids, const float* scores, int32_t B, int64_t n, int32_t k, int32_t* ids_out,
-                     float* scores_out, Scratch& sc, cudaStream_t s);
+                     float* scores_out, cudaStream_t s);
 
 // k_sif.cu
 void sif_build(Index& ix, const int32_t* nbr_ids, const float* nbr_scores, Scratch& sc,

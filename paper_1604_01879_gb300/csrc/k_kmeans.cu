@@ -19,7 +19,7 @@ namespace {
 // takes one centre and 4 * kMeanT columns, one float4 of them per thread, and keeps
 // kMeanRows row loads in flight per thread: the kernel is bound by reading X once
 // (16,384 x 4096 FP32, 1,024 centres: 268 MB), and a loop with one dependent
-// 4-byte load per row and thread left that read latency-bound (1,174 us against 51).
+// 4-byte load per row and thread left that read latency-bound (1,174 us against 75).
 // Every column still adds its rows in ascending order, so the sums are the same.
 constexpr int kMeanT = 128, kMeanRows = 8;
 __global__ __launch_bounds__(kMeanT) void k_km_mean(const float* __restrict__ X, int D,
@@ -140,7 +140,7 @@ void kmeans(const float* X, int64_t n, int D, int K, const std::vector<int32_t>&
       k_km_dist<<<(unsigned)cdiv(n, 8), 256, 0, s>>>(X, n, D, tmp.codebook, lab, dist);
       GIFT_LAUNCHED("k_km_dist");
       int32_t* far = isc.get<int32_t>(E);
-      topk_rows_f32(dist, 1, n, E, far, nullptr, isc, s);  // distance desc, index asc
+      topk_rows_f32(dist, 1, n, E, far, nullptr, s);  // distance desc, index asc
       std::vector<int32_t> h_far(E);
       GIFT_CUDA(cudaMemcpyAsync(h_far.data(), far, (size_t)E * 4, cudaMemcpyDeviceToHost, s));
       GIFT_CUDA(cudaStreamSynchronize(s));

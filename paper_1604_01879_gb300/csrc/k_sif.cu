@@ -9,10 +9,12 @@
 //
 // Re-rank: F_q comes from the first k1 candidates of the query. For each
 // non-zero F_q[i] the entry i is walked and min(F_q[i], F_p[i]) is added to
-// p's numerator (Eq. 13, uint64 atomics: exact and order-free). Then
+// p's numerator (Eq. 13, integer atomics: exact and order-free). Then
 // S' = num / (||F_q||_1 + ||F_p||_1 - num) (Eq. 14) in FP32, and the final
 // order (S' desc, S desc, id asc) is a top-k over 64-bit keys
-// (key(S') << 32 | key(S)) with ties to the lower id.
+// (key(S') << 32 | key(S)) with ties to the lower id. One block per query does it
+// all in shared memory (k_rerank_reach); the re-rank on caller-provided scratch
+// keeps dense rows.
 //
 // Two measures (Sec. 2.4, Eqs. 9-11): a block per shape (database or query)
 // gathers the activations that make up its two contextual activations — its
@@ -24,6 +26,7 @@
 // inverted file of their own; a query's activation is walked through it as in
 // the one-measure re-rank.
 #include "gift_internal.cuh"
+#include "select.cuh"
 
 namespace gift {
 
@@ -127,91 +130,349 @@ __global__ void k_rerank_keys(const unsigned long long* __restrict__ num,
   keys[idx] = ((unsigned long long)f2key(sp) << 32) | (unsigned long long)f2key(Srow[idx]);
 }
 
-// The shapes a query reaches -- through the S-IF walk (numerator > 0) or as a
-// candidate (finite S) -- in ascending id order, with their ranking keys (as
-// k_rerank_keys); every other shape has the same key, S' = 0 and S = -inf,
-// below all of these, so the top-k of the dense row is the top-k of this
-// compact row, followed (when fewer than min(topk, N) shapes are reached) by the
-// unreached shapes in ascending id order. One block per query, rows of `cap`
-// (padding: key 0, id -1).
-constexpr int kCompactT = 1024;
-__global__ __launch_bounds__(kCompactT) void k_rerank_compact(
-    const unsigned long long* __restrict__ num, const unsigned long long* __restrict__ fq_norm,
-    const unsigned long long* __restrict__ card, const float* __restrict__ Srow, int32_t N, int64_t cap, int need,
-    int32_t* __restrict__ ids, unsigned long long* __restrict__ keys) {
-  __shared__ int wtot[kCompactT / 32];
-  __shared__ int s_count;
-  const int b = blockIdx.x, t = threadIdx.x, w = t >> 5, lane = t & 31;
-  const unsigned long long* nr = num + (int64_t)b * N;
-  const float* sr = Srow + (int64_t)b * N;
-  int32_t* oid = ids + (int64_t)b * cap;
-  unsigned long long* okey = keys + (int64_t)b * cap;
-  const unsigned long long fq = fq_norm[b];
-  if (t == 0) s_count = 0;
-  __syncthreads();
-  // pass 0: the reached shapes; pass 1 (only when too few): the first unreached ones
-  for (int pass = 0; pass < 2; ++pass) {
-    if (pass == 1 && s_count >= need) break;  // block-uniform (read after a barrier)
-    for (int c0 = 0; c0 < N; c0 += kCompactT) {
-      const int p = c0 + t;
-      bool in = false;
-      unsigned long long key = 0;
-      if (p < N) {
-        const unsigned long long nm = nr[p];
-        const float sv = sr[p];
-        const bool reached = nm != 0ull || sv != -INFINITY;
-        in = pass == 0 ? reached : !reached;
-        if (in) {
-          float sp = 0.f;
-          if (nm > 0) sp = __fdiv_rn(__ull2float_rn(nm), __ull2float_rn(fq + card[p] - nm));
-          key = ((unsigned long long)f2key(sp) << 32) | (unsigned long long)f2key(sv);
-        }
+// ---------------------------------------------------------------- re-rank of one query per block
+// A query reaches few shapes: its candidates and the shapes in its k1 S-IF entries, a few
+// thousand (shape, membership) pairs however large the database. One block takes one query and
+// keeps the numerators and the tie-break scores in shared memory: a table with a row per shape
+// where all N fit, a hash table of the reached shapes otherwise. It walks the entries (a warp
+// per entry), turns the rows into ranking keys, selects the top-k and writes it -- nothing of
+// the size of the database is cleared, written or scanned in global memory. What is left is a
+// few dependent global reads (candidate, entry offsets, entry), then shared-memory passes.
+// Measured, whole calls (256 queries, k1 = 50, 200,000 shapes): 552 us with dense [B, N] rows in
+// global memory and six launches, 28 us here; two measures, 1,000 queries, 12,000 shapes: 756 and
+// 240 us, 180 of them this kernel (a query there adds some 55,000 pairs).
+//
+// Unreached shapes all have the key (S' = 0, S = -inf). Where they are needed (fewer reached
+// shapes than the top-k) they follow in id order. A hash table that overflows (a query that
+// reaches more shapes than its slots) is given up, and the block goes over the database in
+// ranges of as many shapes as its table holds, merging each range's best with those before.
+struct ReachArgs {
+  int32_t N;                     // shapes
+  const int32_t* cand_ids;       // [B, n_cand]
+  const float* cand_scores;
+  int n_cand;
+  int k1;                        // F_q: the first k1 candidates (act_ids null), or
+  const int32_t* act_ids;        // [B, act_ld] the non-zero coordinates of the activation,
+  const uint32_t* act_mem;       //   their fixed-point values,
+  const int32_t* act_cnt;        //   [B] how many, and
+  const unsigned long long* act_norm;  // [B] their sum
+  int act_ld;
+  const int64_t* off;            // the inverted file and the shapes' norms
+  const int32_t* ids;
+  const uint32_t* mem;
+  const unsigned long long* card;
+  int topk;
+  int32_t* out_ids;              // [B, topk]
+  float* out_sprime;
+  int table_bytes;               // dynamic shared memory
+  int hash;                      // 1: hash table first; 0: ranges of shapes (one range when all fit)
+  unsigned long long* win_key;   // [B, topk] the best of the ranges gone over so far
+  uint32_t* win_id;
+};
+
+constexpr int kReachProbes = 64;  // slots tried before a hash table counts as full
+constexpr uint32_t kNoKey = 0u;   // high key word of a row that is not reached (a real one is >= 0x80000000)
+
+__device__ __forceinline__ uint32_t reach_slot(int32_t id, int slots) {
+  return __umulhi((uint32_t)id * 2654435761u, (uint32_t)slots);
+}
+
+// row of a range's o-th shape: shapes of a class often sit at a fixed stride, whose multiples would fall in a few of
+// the 32 banks (stride 40: four), so the low five bits are mixed with the next five; its own inverse
+__device__ __forceinline__ int reach_row(int o) { return o ^ ((o >> 5) & 31); }
+
+// exact 64-bit sum in two native 32-bit words
+__device__ __forceinline__ void reach_add(uint32_t* lo, uint32_t* hi, int at, uint32_t v) {
+  const uint32_t old = atomicAdd(lo + at, v);
+  if (old > ~v) atomicAdd(hi + at, 1u);
+}
+
+// every pair of the query's entries: f(shape, min(F_q[i], F_p[i])); a lane fetches what one
+// coordinate needs, then the warp reads the 32 coordinates' entries in turn
+template <class F>
+__device__ __forceinline__ void reach_walk(const ReachArgs& a, int b, const F& f) {
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5, lane = threadIdx.x & 31;
+  const int cnt = a.act_ids ? a.act_cnt[b] : a.k1;
+  for (int r0 = w; r0 < cnt; r0 += nw * 32) {
+    const int r = r0 + nw * lane;
+    int64_t e0 = 0;
+    int len = 0;
+    uint32_t fq = 0;
+    if (r < cnt) {
+      const int64_t at = (int64_t)b * (a.act_ids ? a.act_ld : a.n_cand) + r;
+      const int32_t i = a.act_ids ? a.act_ids[at] : a.cand_ids[at];
+      if (i >= 0 && i < a.N) {
+        fq = a.act_ids ? a.act_mem[at] : member_fix(a.cand_scores[at]);
+        e0 = a.off[i];
+        len = fq ? (int)(a.off[i + 1] - e0) : 0;
       }
-      const unsigned m = __ballot_sync(0xffffffffu, in);
-      if (lane == 0) wtot[w] = __popc(m);
-      __syncthreads();
-      if (w == 0) {  // exclusive scan of the warp totals
-        const int x = wtot[lane];
-        int y = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int z = __shfl_up_sync(0xffffffffu, y, o);
-          if (lane >= o) y += z;
-        }
-        wtot[lane] = y - x;
-      }
-      __syncthreads();
-      const int base = s_count;
-      const int pos = base + wtot[w] + __popc(m & ((1u << lane) - 1u));
-      const int limit = pass == 0 ? (int)cap : need;
-      if (in && pos < limit) {
-        oid[pos] = p;
-        okey[pos] = key;
-      }
-      __syncthreads();
-      if (t == kCompactT - 1) s_count = min(limit, pos + (in ? 1 : 0));
-      __syncthreads();
-      if (pass == 1 && s_count >= need) break;  // block-uniform
     }
-    __syncthreads();
-  }
-  for (int64_t j = s_count + t; j < cap; j += kCompactT) {
-    oid[j] = -1;
-    okey[j] = 0ull;
+    for (int j = 0; j < 32 && r0 + nw * j < cnt; ++j) {
+      const int64_t ej = __shfl_sync(0xffffffffu, e0, j);
+      const int nj = __shfl_sync(0xffffffffu, len, j);
+      const uint32_t fj = __shfl_sync(0xffffffffu, fq, j);
+      for (int e = lane; e < nj; e += 128) {
+        int32_t id[4];
+        uint32_t m[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const bool in = e + 32 * u < nj;
+          id[u] = in ? a.ids[ej + e + 32 * u] : 0;
+          m[u] = in ? a.mem[ej + e + 32 * u] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (m[u]) f(id[u], min(fj, m[u]));
+      }
+    }
   }
 }
 
-// output of the selection over compact rows: positions -> shape ids, keys -> S'
-__global__ void k_rerank_out(const int32_t* __restrict__ pos, const unsigned long long* __restrict__ kout,
-                             const int32_t* __restrict__ ids, int64_t cap, int32_t B, int32_t topk,
-                             int32_t* __restrict__ out_ids, float* __restrict__ out_sprime) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)B * topk) return;
-  const int64_t b = i / topk;
-  const int32_t q = pos[i];
-  const bool ok = q >= 0 && kout[i] != 0ull;
-  out_ids[i] = ok ? ids[b * cap + q] : -1;
-  out_sprime[i] = ok ? key2f((uint32_t)(kout[i] >> 32)) : -INFINITY;
+// ranking key of shape p: (S' of Eqs. 13 and 14, S)
+__device__ __forceinline__ unsigned long long reach_key(unsigned long long nm, unsigned long long fq_norm,
+                                                        const unsigned long long* card, int32_t p, float s) {
+  float sp = 0.f;
+  if (nm > 0) sp = __fdiv_rn(__ull2float_rn(nm), __ull2float_rn(fq_norm + card[p] - nm));
+  return ((unsigned long long)f2key(sp) << 32) | (unsigned long long)f2key(s);
+}
+
+// id of row i of the table: its own (hash) or the range's; then the winners of earlier ranges
+struct ReachRows {
+  static constexpr int kAhead = 4;
+  static __device__ __forceinline__ uint32_t score(unsigned long long key) { return (uint32_t)(key >> 32); }
+  const uint32_t* lo;
+  const uint32_t* hi;
+  const int32_t* hid;   // hash: the row's id
+  int32_t r0;           // range: the first id
+  int rows;
+  const unsigned long long* wkey;
+  const uint32_t* wid;
+  __device__ __forceinline__ bool operator()(int64_t i, unsigned long long& key, uint32_t& id) const {
+    if (i >= rows) {
+      key = wkey[i - rows];
+      id = wid[i - rows];
+      return true;
+    }
+    const uint32_t h = hi[i];
+    key = ((unsigned long long)h << 32) | lo[i];
+    id = hid ? (uint32_t)hid[i] : (uint32_t)(r0 + reach_row((int)i));
+    return h != kNoKey;
+  }
+};
+
+struct ReachList {  // listed rows
+  static constexpr int kAhead = 4;
+  static __device__ __forceinline__ uint32_t score(unsigned long long key) { return (uint32_t)(key >> 32); }
+  ReachRows rows;
+  const int32_t* list;
+  __device__ __forceinline__ bool operator()(int64_t i, unsigned long long& key, uint32_t& id) const {
+    return rows(list[i], key, id);
+  }
+};
+constexpr int kReachList = 2048;
+
+// table of N shapes in one range, rows rounded up to the 32 that reach_row mixes
+__host__ __device__ __forceinline__ int64_t reach_rows_bytes(int64_t N) { return (N + 31) / 32 * 32 * 12; }
+
+__global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
+  extern __shared__ __align__(16) uint32_t table[];
+  __shared__ sel::Smem sm;
+  __shared__ unsigned long long s_norm;
+  __shared__ int32_t list[kReachList];
+  __shared__ int s_flag, s_end, s_listed;
+  const int b = blockIdx.x, t = threadIdx.x, T = blockDim.x;
+  const int32_t* cid = a.cand_ids + (int64_t)b * a.n_cand;
+  const float* csc = a.cand_scores + (int64_t)b * a.n_cand;
+  if (t == 0) {
+    s_norm = a.act_ids ? a.act_norm[b] : 0ull;
+    s_flag = 0;
+    s_listed = 0;
+  }
+  __syncthreads();
+  if (!a.act_ids)
+    for (int c = t; c < a.k1; c += T)
+      if (cid[c] >= 0 && cid[c] < a.N) atomicAdd(&s_norm, (unsigned long long)member_fix(csc[c]));
+  const int need = min(a.topk, a.N);
+  int take = 0;
+
+  // rows of the table: numerator (two words), S, and the id of a hash slot
+  bool hashed = a.hash != 0;
+  const bool one = reach_rows_bytes(a.N) <= a.table_bytes;
+  const int W = (one ? (a.N + 31) : a.table_bytes / 12) & ~31;  // shapes of a range
+  int rows = hashed ? a.table_bytes / 16 : W;
+  uint32_t* lo = table;
+  uint32_t* hi = lo + rows;
+  float* S = reinterpret_cast<float*>(hi + rows);
+  int32_t* hid = reinterpret_cast<int32_t*>(S + rows);
+  auto reached = [&](int i) { return (lo[i] | hi[i]) != 0u || S[i] != -INFINITY; };
+  auto numerator = [&](int i) { return ((unsigned long long)hi[i] << 32) | lo[i]; };
+
+  if (hashed) {
+    for (int i = t; i < rows; i += T) {
+      lo[i] = 0u;
+      hi[i] = 0u;
+      S[i] = -INFINITY;
+      hid[i] = -1;
+    }
+    __syncthreads();
+    auto slot_of = [&](int32_t id) {  // the shape's slot, taken if it has none; -1: none left near
+      uint32_t h = reach_slot(id, rows);
+      for (int n = 0; n < kReachProbes; ++n) {
+        int32_t cur = *reinterpret_cast<volatile int32_t*>(hid + h);
+        if (cur == -1) cur = atomicCAS(hid + h, -1, id);
+        if (cur == -1 || cur == id) return (int)h;
+        if (++h == (uint32_t)rows) h = 0;
+      }
+      s_flag = 1;
+      return -1;
+    };
+    for (int c = t; c < a.n_cand; c += T)
+      if (cid[c] >= 0 && cid[c] < a.N) {
+        const int at = slot_of(cid[c]);
+        if (at >= 0) S[at] = csc[c];
+      }
+    reach_walk(a, b, [&](int32_t id, uint32_t v) {
+      const int at = slot_of(id);
+      if (at >= 0) reach_add(lo, hi, at, v);
+    });
+    __syncthreads();
+    hashed = s_flag == 0;
+    if (!hashed) {  // the table overflowed: ranges of shapes
+      rows = W;
+      hi = lo + rows;
+      S = reinterpret_cast<float*>(hi + rows);
+    }
+  }
+  const bool ranges = !hashed && !one;
+  for (int64_t r0 = 0; !hashed && r0 < a.N; r0 += W) {
+    const int n = (int)min((int64_t)W, a.N - r0);
+    __syncthreads();
+    for (int i = t; i < rows; i += T) {
+      lo[i] = 0u;
+      hi[i] = 0u;
+      S[i] = -INFINITY;
+    }
+    __syncthreads();
+    for (int c = t; c < a.n_cand; c += T)
+      if (cid[c] >= r0 && cid[c] < r0 + n) S[reach_row((int)(cid[c] - r0))] = csc[c];
+    reach_walk(a, b, [&](int32_t id, uint32_t v) {
+      if (id >= r0 && id < r0 + n) reach_add(lo, hi, reach_row((int)(id - r0)), v);
+    });
+    __syncthreads();
+    if (!ranges) break;
+    // every shape of the range, reached or not, against the winners of the ranges before
+    for (int i = t; i < rows; i += T) {
+      const int o = reach_row(i);
+      const unsigned long long key = o < n ? reach_key(numerator(i), s_norm, a.card, (int32_t)r0 + o, S[i]) : 0ull;
+      hi[i] = (uint32_t)(key >> 32);  // kNoKey past the range
+      lo[i] = (uint32_t)key;
+    }
+    __syncthreads();
+    unsigned long long* wkey = a.win_key + (int64_t)b * a.topk;
+    uint32_t* wid = a.win_id + (int64_t)b * a.topk;
+    const int win = take;
+    take = sel::select(sm, ReachRows{lo, hi, nullptr, (int32_t)r0, rows, wkey, wid}, rows + win, n + win, need);
+    for (int i = t; i < take; i += T) {
+      wkey[i] = sm.key[i];
+      wid[i] = sm.id[i];
+    }
+    __syncthreads();
+  }
+
+  if (!ranges) {
+    // the reached rows, listed first, so that their keys' reads of the norms go out together
+    const int lane = t & 31;
+    for (int base = 0; base < rows; base += T) {
+      const int i = base + t;
+      const bool in = i < rows && reached(i);
+      const unsigned m = __ballot_sync(0xffffffffu, in);
+      if (!m) continue;
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&s_listed, __popc(m));
+      at = __shfl_sync(0xffffffffu, at, 0) + __popc(m & ((1u << lane) - 1u));
+      if (in && at < kReachList) list[at] = i;
+    }
+    __syncthreads();
+    const int M = s_listed;
+    const bool listed = M <= kReachList;
+    const int32_t* ids = hashed ? hid : nullptr;
+    // their keys in place (of every row where the list is full)
+    auto set_key = [&](int i) {
+      const unsigned long long key =
+          reached(i) ? reach_key(numerator(i), s_norm, a.card, ids ? ids[i] : reach_row(i), S[i]) : 0ull;
+      hi[i] = (uint32_t)(key >> 32);
+      lo[i] = (uint32_t)key;
+    };
+    if (listed) {
+      for (int j = t; j < M; j += T) set_key(list[j]);
+      __syncthreads();
+      take = sel::select(sm, ReachList{ReachRows{lo, hi, ids, 0, rows, nullptr, nullptr}, list}, M, M, need);
+    } else {
+      for (int i = t; i < rows; i += T) set_key(i);
+      __syncthreads();
+      take = sel::select(sm, ReachRows{lo, hi, ids, 0, rows, nullptr, nullptr}, rows, M, need);
+    }
+    if (take < need) {  // the unreached shapes of the lowest ids fill up (listed: M < need; other rows hold zeros)
+      const unsigned long long none = ((unsigned long long)f2key(0.f) << 32) | (unsigned long long)f2key(-INFINITY);
+      for (int64_t c0 = 0; c0 < a.N && take < need; c0 += T) {
+        const int64_t id = c0 + t;
+        bool free = id < a.N;
+        if (free && !hashed) {
+          free = hi[reach_row((int)id)] == kNoKey;
+        } else if (free) {
+          uint32_t h = reach_slot((int32_t)id, rows);
+          for (int n = 0; n < kReachProbes && hid[h] != -1; ++n) {
+            if (hid[h] == (int32_t)id) {
+              free = hi[h] == kNoKey;
+              break;
+            }
+            if (++h == (uint32_t)rows) h = 0;
+          }
+        }
+        const int at = take + sel::block_prefix(sm, free ? 1 : 0);
+        if (free && at < need) {
+          sm.key[at] = none;
+          sm.id[at] = (uint32_t)id;
+        }
+        if (t == T - 1) s_end = at + (free ? 1 : 0);
+        __syncthreads();
+        take = min(need, s_end);
+        __syncthreads();
+      }
+      sel::sort_have(sm, take);
+    }
+  }
+  for (int i = t; i < a.topk; i += T) {
+    const bool ok = i < take;
+    a.out_ids[(int64_t)b * a.topk + i] = ok ? (int32_t)sm.id[i] : -1;
+    a.out_sprime[(int64_t)b * a.topk + i] = ok ? key2f((uint32_t)(sm.key[i] >> 32)) : -INFINITY;
+  }
+}
+
+// Table and block of a launch. Two blocks of 512 threads share an SM while a table takes at
+// most 78 KB: all N up to 6,656 shapes, or 4,992 hash slots, which a query's pairs (n_cand
+// candidates, k1 entries of `mean` shapes) should leave a quarter empty. Heavier walks (`heavy`:
+// many entries per query) take a whole SM's table of up to 15,700 shapes, which spares them the probing.
+void launch_reach(ReachArgs& a, int B, int64_t mean, bool heavy, Scratch& sc, cudaStream_t s) {
+  constexpr int kHalf = 71680, kWhole = 188416;
+  int threads = 512;
+  const int64_t rows = reach_rows_bytes(a.N);
+  if (rows <= kHalf || (heavy && rows <= kWhole)) {
+    a.hash = 0;
+    a.table_bytes = (int)rows;
+    threads = a.N <= 1024 ? 256 : rows <= kHalf ? 512 : 1024;
+  } else {
+    const int64_t pairs = (int64_t)a.n_cand + mean * (a.act_ids ? a.act_ld : a.k1);
+    a.hash = 1;
+    a.table_bytes = !heavy && pairs * 16 * 4 / 3 <= kHalf ? kHalf : kWhole;
+    threads = a.table_bytes == kHalf ? 512 : 1024;
+  }
+  a.win_key = sc.get<unsigned long long>((size_t)B * a.topk);
+  a.win_id = sc.get<uint32_t>((size_t)B * a.topk);
+  // the largest table, whatever this call takes: calls of several threads set the same value
+  GIFT_CUDA(cudaFuncSetAttribute(k_rerank_reach, cudaFuncAttributeMaxDynamicSharedMemorySize, kWhole));
+  k_rerank_reach<<<(unsigned)B, threads, a.table_bytes, s>>>(a);
+  GIFT_LAUNCHED("k_rerank_reach");
 }
 
 __global__ void k_keys_to_sprime(const unsigned long long* __restrict__ keys, int64_t n,
@@ -368,23 +629,6 @@ __global__ void k_aca_fill(const int32_t* __restrict__ perm, int64_t n, int cap,
   mem[e] = mem_rows[slot];
 }
 
-// one block per (query, non-zero coordinate i of its activation): walk entry i
-__global__ void k_aca_walk(const int32_t* __restrict__ q_ids, const uint32_t* __restrict__ q_mem,
-                           const int32_t* __restrict__ q_cnt, int cap, int32_t N, const int64_t* __restrict__ off,
-                           const int32_t* __restrict__ ids, const uint32_t* __restrict__ mem,
-                           unsigned long long* __restrict__ num) {
-  const int b = blockIdx.x, j = blockIdx.y;
-  if (j >= q_cnt[b]) return;
-  const int32_t i = q_ids[(int64_t)b * cap + j];
-  const uint32_t fq = q_mem[(int64_t)b * cap + j];
-  if (fq == 0 || i < 0 || i >= N) return;
-  for (int64_t e = off[i] + threadIdx.x; e < off[i + 1]; e += blockDim.x) {
-    const uint32_t m = mem[e];
-    if (m == 0) continue;
-    atomicAdd(num + (int64_t)b * N + ids[e], (unsigned long long)min(fq, m));
-  }
-}
-
 void launch_aca_rows(AcaRowArgs& a, int64_t rows, cudaStream_t s) {
   a.nmax = a.mode == 0 ? a.k1 : a.k2 * a.k1;
   int P = 2 * kAcaT;
@@ -476,7 +720,6 @@ void aca_rerank(const Aca& a, const int32_t* cand1, const float* sc1, const int3
                 int32_t B, int32_t n_cand, int32_t topk, int32_t* out_ids, float* out_sprime, Scratch& sc,
                 cudaStream_t s) {
   const int32_t N = a.N;
-  const int64_t BN = (int64_t)B * N;
   AcaRowArgs r{};
   r.mode = a.mode;
   r.k1 = a.k1;
@@ -499,25 +742,25 @@ void aca_rerank(const Aca& a, const int32_t* cand1, const float* sc1, const int3
   r.out_cnt = sc.get<int32_t>(B);
   r.out_norm = sc.get<unsigned long long>(B);
   launch_aca_rows(r, B, s);
-  unsigned long long* num = sc.get<unsigned long long>(BN);
-  GIFT_CUDA(cudaMemsetAsync(num, 0, BN * 8, s));
-  float* Srow = sc.get<float>(BN);
-  k_fill_f32<<<(unsigned)cdiv(BN, 256), 256, 0, s>>>(Srow, BN, -INFINITY);
-  GIFT_LAUNCHED("k_fill_f32");
-  unsigned long long* unused = sc.get<unsigned long long>(B);
-  k_rerank_prep<<<(unsigned)B, 256, 0, s>>>(cand1, sc1, n_cand, a.k1, N, Srow, unused);  // S^(1) tie key
-  GIFT_LAUNCHED("k_rerank_prep");
-  k_aca_walk<<<dim3((unsigned)B, (unsigned)r.cap), 128, 0, s>>>(r.out_ids, r.out_mem, r.out_cnt, r.cap, N, a.off,
-                                                                a.ids, a.mem, num);
-  GIFT_LAUNCHED("k_aca_walk");
-  unsigned long long* keys = sc.get<unsigned long long>(BN);
-  k_rerank_keys<<<(unsigned)cdiv(BN, 256), 256, 0, s>>>(num, r.out_norm, a.card, Srow, B, N, keys);
-  GIFT_LAUNCHED("k_rerank_keys");
-  unsigned long long* kout = sc.get<unsigned long long>((int64_t)B * topk);
-  topk_rows_u64(reinterpret_cast<const uint64_t*>(keys), B, N, topk, out_ids, reinterpret_cast<uint64_t*>(kout),
-                sc, s);
-  k_keys_to_sprime<<<(unsigned)cdiv((int64_t)B * topk, 256), 256, 0, s>>>(kout, (int64_t)B * topk, out_sprime);
-  GIFT_LAUNCHED("k_keys_to_sprime");
+  ReachArgs g{};
+  g.N = N;
+  g.cand_ids = cand1;
+  g.cand_scores = sc1;  // S^(1) breaks ties
+  g.n_cand = n_cand;
+  g.k1 = a.k1;
+  g.act_ids = r.out_ids;
+  g.act_mem = r.out_mem;
+  g.act_cnt = r.out_cnt;
+  g.act_norm = r.out_norm;
+  g.act_ld = r.cap;
+  g.off = a.off;
+  g.ids = a.ids;
+  g.mem = a.mem;
+  g.card = a.card;
+  g.topk = topk;
+  g.out_ids = out_ids;
+  g.out_sprime = out_sprime;
+  launch_reach(g, B, cdiv(a.pairs, (int64_t)N), true, sc, s);
 }
 
 void sif_build(Index& ix, const int32_t* nbr_ids, const float* nbr_scores, Scratch& sc, cudaStream_t s) {
@@ -552,36 +795,20 @@ void sif_build(Index& ix, const int32_t* nbr_ids, const float* nbr_scores, Scrat
 
 void sif_rerank(const Index& ix, const int32_t* cand_ids, const float* cand_scores, int32_t B, int32_t n_cand,
                 int32_t k1, int32_t topk, int32_t* out_ids, float* out_sprime, Scratch& sc, cudaStream_t s) {
-  const int32_t N = ix.sif_n;
-  const int64_t BN = (int64_t)B * N;
-  unsigned long long* num = sc.get<unsigned long long>(BN);
-  GIFT_CUDA(cudaMemsetAsync(num, 0, BN * 8, s));
-  float* Srow = sc.get<float>(BN);
-  k_fill_f32<<<(unsigned)cdiv(BN, 256), 256, 0, s>>>(Srow, BN, -INFINITY);
-  GIFT_LAUNCHED("k_fill_f32");
-  unsigned long long* fqn = sc.get<unsigned long long>(B);
-  k_rerank_prep<<<(unsigned)B, 256, 0, s>>>(cand_ids, cand_scores, n_cand, k1, N, Srow, fqn);
-  GIFT_LAUNCHED("k_rerank_prep");
-  k_rerank_walk<<<dim3((unsigned)B, (unsigned)k1), 128, 0, s>>>(cand_ids, cand_scores, n_cand, k1, N, ix.sif_off,
-                                                             ix.sif_ids, ix.sif_mem, num);
-  GIFT_LAUNCHED("k_rerank_walk");
-  // a query reaches at most n_cand candidates and k1 S-IF entries of at most
-  // max_sif_entry shapes: the selection runs over those, not over all N
-  const int need = std::min(topk, N);
-  const int64_t cap = std::min<int64_t>(
-      N, std::max<int64_t>(need, (int64_t)n_cand + (int64_t)k1 * std::max(1, ix.max_sif_entry)));
-  int32_t* cids = sc.get<int32_t>((size_t)B * cap);
-  unsigned long long* keys = sc.get<unsigned long long>((size_t)B * cap);
-  k_rerank_compact<<<(unsigned)B, kCompactT, 0, s>>>(num, fqn, reinterpret_cast<const unsigned long long*>(ix.sif_card),
-                                                      Srow, N, cap, need, cids, keys);
-  GIFT_LAUNCHED("k_rerank_compact");
-  int32_t* pos = sc.get<int32_t>((size_t)B * topk);
-  unsigned long long* kout = sc.get<unsigned long long>((int64_t)B * topk);
-  topk_rows_u64(reinterpret_cast<const uint64_t*>(keys), B, cap, topk, pos, reinterpret_cast<uint64_t*>(kout), sc,
-                s);
-  k_rerank_out<<<(unsigned)cdiv((int64_t)B * topk, 256), 256, 0, s>>>(pos, kout, cids, cap, B, topk, out_ids,
-                                                                     out_sprime);
-  GIFT_LAUNCHED("k_rerank_out");
+  ReachArgs g{};
+  g.N = ix.sif_n;
+  g.cand_ids = cand_ids;
+  g.cand_scores = cand_scores;
+  g.n_cand = n_cand;
+  g.k1 = k1;
+  g.off = ix.sif_off;
+  g.ids = ix.sif_ids;
+  g.mem = ix.sif_mem;
+  g.card = reinterpret_cast<const unsigned long long*>(ix.sif_card);
+  g.topk = topk;
+  g.out_ids = out_ids;
+  g.out_sprime = out_sprime;
+  launch_reach(g, B, ix.k1, false, sc, s);
 }
 
 namespace {
@@ -625,9 +852,7 @@ void sif_rerank_into(const Index& ix, const int32_t* cand_ids, const float* cand
                                                           reinterpret_cast<const unsigned long long*>(ix.sif_card),
                                                           Srow, B, N, keys);
   GIFT_LAUNCHED("k_rerank_keys");
-  Scratch none(s);  // the selection kernel takes a scratch handle but allocates nothing
-  topk_rows_u64(reinterpret_cast<const uint64_t*>(keys), B, N, topk, out_ids, reinterpret_cast<uint64_t*>(kout),
-                none, s);
+  topk_rows_u64(reinterpret_cast<const uint64_t*>(keys), B, N, topk, out_ids, reinterpret_cast<uint64_t*>(kout), s);
   k_keys_to_sprime<<<(unsigned)cdiv((int64_t)B * topk, 256), 256, 0, s>>>(kout, (int64_t)B * topk, out_sprime);
   GIFT_LAUNCHED("k_keys_to_sprime");
 }
