@@ -412,7 +412,7 @@ void run_fif(Index& ix, const float* q, int64_t nv, const std::vector<int32_t>& 
   else if (ix.prm.storage != GIFT_F32)
     fif_scan_tc(ix, P, table, false, nullptr, 0, sc, s);
   else
-    fif_scan(ix, P, table, false, nullptr, 0, s);
+    fif_scan(ix, P, table, false, nullptr, 0, sc, s);
 
   tm.mark(ST_COMBINE);
   float* S = sc.get<float>((size_t)B * N);
@@ -436,7 +436,7 @@ void run_fif(Index& ix, const float* q, int64_t nv, const std::vector<int32_t>& 
     if (ix.list_lo)
       fif_scan_tc(ix, P, table, true, cand_sorted, Rr, sc, s);
     else
-      fif_scan(ix, P, table, true, cand_sorted, Rr, s);
+      fif_scan(ix, P, table, true, cand_sorted, Rr, sc, s);
   }
   float* cand_score = sc.get<float>((size_t)B * Rr);
   fif_combine(ix, P, fused ? table32 : table, nullptr, cand_sorted, Rr, cand_score, sc, s);

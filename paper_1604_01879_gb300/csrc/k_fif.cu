@@ -23,6 +23,7 @@
 
 #include "gift_internal.cuh"
 #include "fif_plan.cuh"
+#include "select.cuh"
 
 namespace gift {
 
@@ -43,23 +44,142 @@ __global__ void k_slot_setup(const int32_t* __restrict__ perm, int64_t nslots, i
   run_cnt[s] = nruns[skeys[s]];
 }
 
-// work items of list k: ceil(L_k / TE) entry tiles x ceil(M_k / TS) slot chunks
-__global__ void k_work_count(const int64_t* __restrict__ boff, const int64_t* __restrict__ list_off,
-                             int K, int64_t* __restrict__ wcnt, int64_t row_bytes,
-                             int64_t rescore_row_bytes, unsigned long long* __restrict__ stats) {
+// scanned bytes and pairs of the batch (timed calls only)
+__global__ void k_scan_stats(const int64_t* __restrict__ boff, const int64_t* __restrict__ list_off, int K,
+                             int64_t row_bytes, int64_t rescore_row_bytes, unsigned long long* __restrict__ stats) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k > K) return;
-  if (k == K) {
-    wcnt[K] = 0;
-    return;
-  }
+  if (k >= K) return;
   const int64_t M = boff[k + 1] - boff[k];
   const int64_t L = list_off[k + 1] - list_off[k];
-  wcnt[k] = (M > 0 && L > 0) ? cdiv(L, kScanTE) * cdiv(M, kScanTS) : 0;
-  if (stats && M > 0 && L > 0) {
+  if (M > 0 && L > 0) {
     atomicAdd(&stats[0], (unsigned long long)(L * row_bytes));
     atomicAdd(&stats[1], (unsigned long long)(L * M));
     atomicAdd(&stats[2], (unsigned long long)(L * rescore_row_bytes));
+  }
+}
+
+// inclusive prefix sum of one int64 per thread over a block of 1,024; wsum: 32 words
+__device__ __forceinline__ int64_t block_incl_i64(int64_t v, int64_t* wsum) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  __syncthreads();  // wsum may still be read from the call before
+  if (lane == 31) wsum[w] = v;
+  __syncthreads();
+  int64_t before = 0;
+  for (int k = 0; k < w; ++k) before += wsum[k];
+  return v + before;
+}
+
+constexpr int kPlanT = 1024;
+
+// one block per spec: the work offsets of the batch's lists
+__global__ __launch_bounds__(kPlanT) void k_plan_work(const int64_t* __restrict__ boff,
+                                                      const int64_t* __restrict__ list_off, int K,
+                                                      const WorkSpecs specs, int64_t fold,
+                                                      int64_t* __restrict__ woff) {
+  __shared__ int64_t wsum[kPlanT / 32];
+  __shared__ unsigned long long s_items;
+  __shared__ int s_most;
+  const int tid = threadIdx.x, c = blockIdx.x;
+  const int cls = specs.cls[c], tn = specs.tn[c], ts = specs.ts[c];
+  int64_t* out = woff + (int64_t)c * (K + 1);
+  int folded = 0;  // class that takes every slot-column list
+  if (fold > 0 && cls > 0) {
+    if (tid == 0) {
+      s_items = 0ull;
+      s_most = 0;
+    }
+    __syncthreads();
+    unsigned long long items = 0;
+    int most = 0;
+#pragma unroll 4
+    for (int k = tid; k < K; k += kPlanT) {
+      const int64_t M = boff[k + 1] - boff[k], L = list_off[k + 1] - list_off[k];
+      if (M > 0 && L > 0 && M <= 80) {
+        items += (unsigned long long)(((uint32_t)L + 127u) / 128u);
+        most = max(most, (int)M);
+      }
+    }
+    if (items) atomicAdd(&s_items, items);
+    if (most) atomicMax(&s_most, most);
+    __syncthreads();
+    if (s_items <= (unsigned long long)fold) folded = slot_class(s_most);
+  }
+  int64_t run = 0;
+  for (int k0 = 0; k0 <= K; k0 += 4 * kPlanT) {
+    int64_t n[4];  // four chunks' reads go out together
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = k0 + i * kPlanT + tid;
+      n[i] = 0;
+      if (k >= K) continue;
+      const int64_t M = boff[k + 1] - boff[k], L = list_off[k + 1] - list_off[k];
+      const int mine = M <= 80 && folded ? folded : slot_class(M);
+      // (entries and slots number fewer than 2^31: 32-bit divisions)
+      if (M > 0 && L > 0 && (cls <= 0 || mine == cls))
+        n[i] = (int64_t)(((uint32_t)L + tn - 1) / (uint32_t)tn) * (((uint32_t)M + ts - 1) / (uint32_t)ts);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int k = k0 + i * kPlanT + tid;
+      if (k0 + i * kPlanT > K) break;
+      const int64_t incl = block_incl_i64(n[i], wsum);
+      if (k <= K) out[k] = run + incl - n[i];
+#pragma unroll
+      for (int w = 0; w < kPlanT / 32; ++w) run += wsum[w];
+    }
+  }
+}
+
+// The slots of a small batch (up to kSmallSlots) in one block: sort by codeword (ties by item, as the stable
+// radix sort leaves them), list offsets, slot <-> view maps and the first table cell of each slot. Ten launches
+// of a few microseconds each otherwise, whose gaps are most of a small query's time.
+constexpr int kSmallSlots = sel::kCap;
+__global__ __launch_bounds__(kPlanT) void k_slots_small(const int32_t* __restrict__ codes, int n, int ma, int K,
+                                                        const int32_t* __restrict__ nruns,
+                                                        int32_t* __restrict__ skeys, int64_t* __restrict__ boff,
+                                                        int32_t* __restrict__ slot_view,
+                                                        int32_t* __restrict__ view_slot,
+                                                        int64_t* __restrict__ runbase) {
+  __shared__ unsigned long long key[kSmallSlots];
+  __shared__ uint32_t id[kSmallSlots];
+  __shared__ int64_t wsum[kPlanT / 32];
+  const int tid = threadIdx.x;
+  int P = 64;
+  while (P < n) P <<= 1;
+  for (int t = tid; t < P; t += kPlanT) {
+    key[t] = t < n ? ~(unsigned long long)(uint32_t)codes[t] : 0ull;  // best first: the lowest code
+    id[t] = (uint32_t)t;
+  }
+  sel::sort_pairs(key, id, P);
+  int64_t run = 0;
+  for (int s0 = 0; s0 <= n; s0 += kPlanT) {
+    const int s = s0 + tid;
+    int64_t cells = 0;
+    if (s < n) {
+      const int32_t k = (int32_t)~key[s], item = (int32_t)id[s];
+      skeys[s] = k;
+      slot_view[s] = item / ma;
+      view_slot[item] = s;
+      cells = nruns[k];
+    }
+    const int64_t incl = block_incl_i64(cells, wsum);
+    if (s <= n) runbase[s] = run + incl - cells;
+#pragma unroll
+    for (int w = 0; w < kPlanT / 32; ++w) run += wsum[w];
+  }
+  for (int k = tid; k <= K; k += kPlanT) {  // the first slot of a code >= k
+    int lo = 0, hi = n;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if ((int32_t)~key[mid] < k) lo = mid + 1;
+      else hi = mid;
+    }
+    boff[k] = lo;
   }
 }
 
@@ -498,41 +618,56 @@ void fif_zero_table(const FifPlan& P, uint32_t* table, cudaStream_t s) {
   GIFT_LAUNCHED("k_zero_cells");
 }
 
+int64_t* plan_work(const Index& ix, const FifPlan& P, const WorkSpecs& specs, int64_t fold, Scratch& sc,
+                   cudaStream_t s) {
+  const int K = ix.prm.n_codewords;
+  int64_t* woff = sc.get<int64_t>((size_t)specs.n * (K + 1));
+  k_plan_work<<<(unsigned)specs.n, kPlanT, 0, s>>>(P.boff, ix.list_off, K, specs, fold, woff);
+  GIFT_LAUNCHED("k_plan_work");
+  return woff;
+}
+
 void fif_plan(const Index& ix, FifPlan& P, Scratch& sc, cudaStream_t s) {
   const int K = ix.prm.n_codewords;
   P.nslots = P.nv * P.ma;
   const int64_t n = P.nslots;
   P.skeys = sc.get<int32_t>(n);
-  int32_t* perm = sc.get<int32_t>(n);
-  stable_sort_by_key(P.q_code, n, K, perm, P.skeys, sc, s);
   P.boff = sc.get<int64_t>(K + 1);
-  bin_offsets(P.skeys, n, K, P.boff, s);
   P.slot_view = sc.get<int32_t>(n);
   P.view_slot = sc.get<int32_t>(n);
-  int64_t* run_cnt = sc.get<int64_t>(n + 1);
-  k_slot_setup<<<(unsigned)cdiv(n + 1, 256), 256, 0, s>>>(perm, n, P.ma, P.skeys, ix.nruns, P.slot_view,
-                                                            P.view_slot, run_cnt);
-  GIFT_LAUNCHED("k_slot_setup");
   P.runbase = sc.get<int64_t>(n + 1);
-  scan_exclusive_i64(run_cnt, P.runbase, n + 1, sc, s);  // runbase[n] = table cells in use
+  if (n <= kSmallSlots) {
+    k_slots_small<<<1, kPlanT, 0, s>>>(P.q_code, (int)n, P.ma, K, ix.nruns, P.skeys, P.boff, P.slot_view, P.view_slot,
+                                       P.runbase);
+    GIFT_LAUNCHED("k_slots_small");
+  } else {
+    int32_t* perm = sc.get<int32_t>(n);
+    stable_sort_by_key(P.q_code, n, K, perm, P.skeys, sc, s);
+    bin_offsets(P.skeys, n, K, P.boff, s);
+    int64_t* run_cnt = sc.get<int64_t>(n + 1);
+    k_slot_setup<<<(unsigned)cdiv(n + 1, 256), 256, 0, s>>>(perm, n, P.ma, P.skeys, ix.nruns, P.slot_view,
+                                                              P.view_slot, run_cnt);
+    GIFT_LAUNCHED("k_slot_setup");
+    scan_exclusive_i64(run_cnt, P.runbase, n + 1, sc, s);  // runbase[n] = table cells in use
+  }
   P.table_upper = n * (int64_t)std::max(1, ix.max_runs);
-  int64_t* wcnt = sc.get<int64_t>(K + 1);
-  P.woff = sc.get<int64_t>(K + 1);
-  const int64_t row_bytes = (int64_t)ix.prm.dim * (int64_t)dtype_bytes(ix.prm.storage) + 12;
-  const int64_t rescore_row_bytes = (int64_t)ix.prm.dim * 4 + 12;
-  k_work_count<<<(unsigned)cdiv(K + 1, 256), 256, 0, s>>>(P.boff, ix.list_off, K, wcnt, row_bytes,
-                                                            rescore_row_bytes, P.stats);
-  GIFT_LAUNCHED("k_work_count");
-  scan_exclusive_i64(wcnt, P.woff, K + 1, sc, s);
+  if (P.stats) {
+    const int64_t row_bytes = (int64_t)ix.prm.dim * (int64_t)dtype_bytes(ix.prm.storage) + 12;
+    const int64_t rescore_row_bytes = (int64_t)ix.prm.dim * 4 + 12;
+    k_scan_stats<<<(unsigned)cdiv(K, 256), 256, 0, s>>>(P.boff, ix.list_off, K, row_bytes, rescore_row_bytes, P.stats);
+    GIFT_LAUNCHED("k_scan_stats");
+  }
   const int64_t max_tiles = cdiv(std::max(1, ix.max_list), kScanTE);
   P.upper_items = ix.scan_tiles_upper + max_tiles * (cdiv(n, kScanTS) + 1);
 }
 
 void fif_scan(const Index& ix, const FifPlan& P, uint32_t* table, bool rescore,
-              const int32_t* cand_sorted, int R, cudaStream_t s) {
+              const int32_t* cand_sorted, int R, Scratch& sc, cudaStream_t s) {
   if (P.upper_items <= 0) return;
   ScanArgs a;
-  a.woff = P.woff;
+  WorkSpecs specs;
+  specs.add(0, kScanTE, kScanTS);
+  a.woff = plan_work(ix, P, specs, 0, sc, s);
   a.K = ix.prm.n_codewords;
   a.boff = P.boff;
   a.list_off = ix.list_off;

@@ -47,9 +47,8 @@ struct ListSched {
   const int64_t* list_off;  // [K+1]
   int nkb;
   __device__ __forceinline__ int64_t total_items() const { return woff[K]; }
-  // TN entries x TS slots per item
-  template <int TN, int TS = tc::kTM>
-  __device__ __forceinline__ ListItem decode_list(int64_t item) const {
+  // tn entries x ts slots per item
+  __device__ __forceinline__ ListItem decode_list(int64_t item, int tn, int ts = tc::kTM) const {
     int lo = 0, hi = K;
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
@@ -58,17 +57,23 @@ struct ListSched {
     const int k = lo;
     const int64_t L = list_off[k + 1] - list_off[k];
     const int64_t M = boff[k + 1] - boff[k];
-    const int64_t nts = cdiv(M, (int64_t)TS);
+    const int64_t nts = cdiv(M, (int64_t)ts);
     const int64_t local = item - woff[k];
-    const int64_t te = local / nts, ts = local % nts;
+    const int64_t te = local / nts, st = local % nts;
     ListItem it;
     it.k = k;
-    it.e0 = list_off[k] + te * TN;
-    it.ne = (int)min((int64_t)TN, L - te * TN);
-    it.s0 = boff[k] + ts * TS;
-    it.ns = (int)min((int64_t)TS, M - ts * TS);
+    it.e0 = list_off[k] + te * tn;
+    it.ne = (int)min((int64_t)tn, L - te * tn);
+    it.s0 = boff[k] + st * ts;
+    it.ns = (int)min((int64_t)ts, M - st * ts);
     return it;
   }
+};
+
+// work items of one slot class kept by the rescore's pre-pass, decoded: items[base[0] .. base[1])
+struct KeptItems {
+  const ListItem* items = nullptr;
+  const int64_t* base = nullptr;
 };
 
 struct SlotInfo {
@@ -148,7 +153,7 @@ struct ScanPolicy : ListSched {
     float cur_max;
   };
   __device__ __forceinline__ int64_t total() const { return total_items(); }
-  __device__ __forceinline__ Item decode(int64_t item) const { return decode_list<TN>(item); }
+  __device__ __forceinline__ Item decode(int64_t item) const { return decode_list(item, TN); }
   __device__ __forceinline__ int nchunks(const Item&) const { return 1; }
   __device__ __forceinline__ void chunk(const Item& it, int, int& br, int& kb0, int& kb1) const {
     br = (int)it.e0;
@@ -198,16 +203,16 @@ struct RescorePolicy : ListSched {
   SlotInfo si;
   const int32_t* cand;      // [B, R] candidate ids sorted ascending
   int R;
-  const int64_t* item_map;  // [n_items] the work items holding a candidate run (ascending); null: every item,
-  const int64_t* n_items;   // every run written (the FP32-level scan of a BF16 store with its two-part rows)
+  KeptItems kept;           // the work items holding a candidate run; none: every item, every run
+                            // written (the FP32-level scan of a BF16 store with its two-part rows)
   using Item = ListItem;
   struct Ctx {
     RowCtx row;
     float sum[TN];
   };
-  __device__ __forceinline__ int64_t total() const { return item_map ? *n_items : total_items(); }
+  __device__ __forceinline__ int64_t total() const { return kept.items ? kept.base[1] - kept.base[0] : total_items(); }
   __device__ __forceinline__ Item decode(int64_t item) const {
-    return decode_list<TN>(item_map ? item_map[item] : item);
+    return kept.items ? kept.items[*kept.base + item] : decode_list(item, TN);
   }
   // never an empty chunk: each chunk must write its own accumulator
   // chunks bound the MMA steps feeding one accumulator (about 192, 3 products
@@ -290,10 +295,9 @@ struct RescorePolicy : ListSched {
 // EB = 1, SPLIT = 1: E4M3 scan (per-slot and per-entry scales, one chunk).
 // EB = 2, SPLIT = 3: FP32-level rescore with two-part BF16 operands, the
 // reduction in kRescChunks chunks summed in FP32 (as RescorePolicy).
-__host__ __device__ constexpr int slot_class(int64_t M) {
-  return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : M <= 80 ? 80 : 128;
-}
-
+// A small batch touches so few lists that a class may not fill the SMs once; its
+// classes are folded into the smallest that holds them all (plan_work), one launch
+// with work instead of several, and a (slot, entry) value does not depend on the class.
 template <int EB_, int SPLIT_, int TS_>
 struct SlotsPolicy : ListSched {
   static constexpr int TN = TS_, EB = EB_, SPLIT = SPLIT_;
@@ -313,8 +317,7 @@ struct SlotsPolicy : ListSched {
   static_assert(TS_ == 16 || TS_ == 32 || TS_ == 64 || TS_ == 80, "slot tile of 16, 32, 64 or 80");
   static_assert(kResc ? EB_ == 2 : (EB_ == 1 && SPLIT_ == 1), "E4M3 scan or two-part BF16 rescore");
   SlotInfo si;
-  const int64_t* item_map;  // rescore: [n_items] the kept work items (ascending); scan: null
-  const int64_t* n_items;
+  KeptItems kept;  // rescore: the kept work items; scan: none
   using Item = ListItem;
   struct Ctx {
     int run;
@@ -322,9 +325,9 @@ struct SlotsPolicy : ListSched {
     bool valid;
     float sum[TS_];
   };
-  __device__ __forceinline__ int64_t total() const { return kResc ? *n_items : total_items(); }
+  __device__ __forceinline__ int64_t total() const { return kResc ? kept.base[1] - kept.base[0] : total_items(); }
   __device__ __forceinline__ Item decode(int64_t item) const {
-    return decode_list<tc::kTM, TS_>(kResc ? item_map[item] : item);
+    return kResc ? kept.items[*kept.base + item] : decode_list(item, tc::kTM, TS_);
   }
   __device__ __forceinline__ int nch() const {
     if (!kResc) return 1;
@@ -454,41 +457,99 @@ __global__ __launch_bounds__(256) void k_slot_fp8(const float* __restrict__ q, c
   if (threadIdx.x == 0) scale[s] = sc;
 }
 
+// The slot classes of a batch: offsets of their work items over the lists (128 entries per item; the last class,
+// slot rows, also with the scan's 256)
+constexpr int kClasses = 5;
+__host__ __device__ constexpr int class_ts(int c) { return c == 0 ? 16 : c == 1 ? 32 : c == 2 ? 64 : c == 3 ? 80 : 128; }
+struct ClassWork {
+  const int64_t* woff[kClasses];
+  const int64_t* woff_scan128;
+};
+ClassWork class_work(const Index& ix, const FifPlan& P, Scratch& sc, cudaStream_t s) {
+  const int K = ix.prm.n_codewords;
+  if (!P.class_woff) {
+    WorkSpecs specs;
+    for (int c = 0; c < kClasses; ++c) specs.add(class_ts(c), kRescTN, class_ts(c));
+    specs.add(128, kScanTN, 128);
+    // folding up to three items per SM: a launch takes an item's time (43 us for 128 two-part rows of D = 4096)
+    // times its rounds, so one launch of three rounds against up to four of one or more
+    P.class_woff = plan_work(ix, P, specs, 3 * (int64_t)device_sm_count(), sc, s);
+  }
+  ClassWork w;
+  for (int c = 0; c < kClasses; ++c) w.woff[c] = P.class_woff + (int64_t)c * (K + 1);
+  w.woff_scan128 = P.class_woff + (int64_t)kClasses * (K + 1);
+  return w;
+}
+
+// The items of all classes, class after class: item g of them
+struct ClassItem {
+  int cls;       // -1: past the last
+  int64_t item;  // within the class
+};
+__device__ __forceinline__ ClassItem class_item(const ClassWork& cw, int K, int first_class, int64_t g) {
+  ClassItem r{-1, g};
+#pragma unroll
+  for (int c = 0; c < kClasses; ++c)
+    if (c >= first_class && r.cls < 0) {
+      const int64_t n = cw.woff[c][K];
+      if (r.item < n) r.cls = c;
+      else r.item -= n;
+    }
+  return r;
+}
+__device__ __forceinline__ ListItem class_decode(ListSched ls, const ClassWork& cw, const ClassItem& ci) {
+  const int64_t* w = cw.woff[0];
+#pragma unroll
+  for (int c = 1; c < kClasses; ++c)
+    if (ci.cls == c) w = cw.woff[c];
+  ls.woff = w;
+  return ls.decode_list(ci.item, kRescTN, class_ts(ci.cls));
+}
+
 // Rescore work items that hold a candidate run: item (list k, entry tile,
 // slot tile) is kept when some slot of the tile has, among the tile's
 // entries, a run whose shape is one of its query's top-R candidates. One warp
-// per item tests every (slot, run start) pair; items past the real total (the
-// grid covers an upper bound) are not kept. With stats (timed calls only):
+// per item of any class tests every (slot, run start) pair; masks (optional) gets a
+// bit per item. Items past the real total (the grid covers an upper bound) are not
+// kept. With stats (timed calls only):
 //   [3] items, [4] kept items, [5] candidate (slot, entry) pairs, [6] candidate
 //   rows (entries whose shape is a candidate of some slot of their list, each
 //   list's entries counted once, by its first slot tile), [7] rows of kept items.
-template <int TS>
-__global__ __launch_bounds__(256) void k_resc_flags(const ListSched ls, const int32_t* __restrict__ slot_view,
+__global__ __launch_bounds__(256) void k_resc_flags(const ListSched ls, const ClassWork cw, int first_class,
+                                                    const int32_t* __restrict__ slot_view,
                                                     const int32_t* __restrict__ vquery,
                                                     const int32_t* __restrict__ entry_run,
                                                     const int32_t* __restrict__ list_shape,
-                                                    const int32_t* __restrict__ cand, int R, int64_t upper,
-                                                    int64_t* __restrict__ flags,
+                                                    const int32_t* __restrict__ cand, int R,
+                                                    uint8_t* __restrict__ masks,
                                                     unsigned long long* __restrict__ stats) {
-  const int64_t item = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (item >= upper) return;
-  if (item >= ls.total_items()) {
-    if (lane == 0) flags[item] = 0;
-    return;
-  }
-  const ListItem it = ls.decode_list<kRescTN, TS>(item);
+  __shared__ uint8_t s_hit[8];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const ClassItem ci = class_item(cw, ls.K, first_class, (int64_t)blockIdx.x * 8 + w);
   bool hit = false;
-  for (int m = 0; m < it.ns && !hit; ++m) {
-    const int32_t* cq = cand + (int64_t)vquery[slot_view[it.s0 + m]] * R;
-    for (int c = lane; c < it.ne && !hit; c += 32) {
-      const int64_t e = it.e0 + c;
-      if ((c == 0 || entry_run[e] != entry_run[e - 1]) && is_candidate(cq, R, list_shape[e])) hit = true;
+  ListItem it;
+  if (ci.cls >= 0) {
+    it = class_decode(ls, cw, ci);
+    for (int m = 0; m < it.ns && !hit; ++m) {
+      const int32_t* cq = cand + (int64_t)vquery[slot_view[it.s0 + m]] * R;
+      for (int c = lane; c < it.ne && !hit; c += 32) {
+        const int64_t e = it.e0 + c;
+        if ((c == 0 || entry_run[e] != entry_run[e - 1]) && is_candidate(cq, R, list_shape[e])) hit = true;
+      }
+      hit = __any_sync(0xffffffffu, hit);
     }
-    hit = __any_sync(0xffffffffu, hit);
   }
-  if (lane == 0) flags[item] = hit ? 1 : 0;
-  if (!stats) return;
+  if (masks) {
+    if (lane == 0) s_hit[w] = hit ? 1 << w : 0;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int m = 0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) m |= s_hit[k];
+      masks[blockIdx.x] = (uint8_t)m;
+    }
+  }
+  if (!stats || ci.cls < 0) return;
   unsigned long long pairs = 0, rows = 0;
   for (int m = 0; m < it.ns; ++m) {
     const int32_t* cq = cand + (int64_t)vquery[slot_view[it.s0 + m]] * R;
@@ -517,112 +578,99 @@ __global__ __launch_bounds__(256) void k_resc_flags(const ListSched ls, const in
   }
 }
 
-// item_map[pos[i]] = i for every kept item i < upper; *n_items = the count
-__global__ void k_compact_items(const int64_t* __restrict__ flags, const int64_t* __restrict__ pos, int64_t upper,
-                                int64_t* __restrict__ item_map, int64_t* __restrict__ n_items) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= upper) return;
-  if (flags[i]) item_map[pos[i]] = i;
-  if (i == upper - 1) *n_items = pos[i] + flags[i];
-}
-
-// ts_class > 0: only the lists of that slot class (slot tiles of ts_class slots);
-// otherwise every touched list, slot tiles of 128
-__global__ void k_work_count_tc(const int64_t* __restrict__ boff, const int64_t* __restrict__ list_off, int K,
-                                int tn, int ts_class, int64_t* __restrict__ wcnt) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k > K) return;
-  if (k == K) {
-    wcnt[K] = 0;
-    return;
+// Kept items, decoded, in their order (neighbouring items share list rows and slot tiles; appended as blocks
+// finish, the largest class took 8% longer), and where each class's begin: base[c], base[kClasses] the end. A
+// block takes 1,024 items and counts the bits of the masks before them itself (a byte per eight items, from L2),
+// so one launch does for any number of items.
+constexpr int kCompactT = 1024;
+__global__ __launch_bounds__(kCompactT) void k_resc_compact(const ListSched ls, const ClassWork cw,
+                                                            const uint8_t* __restrict__ masks, int64_t nmasks,
+                                                            ListItem* __restrict__ items,
+                                                            int64_t* __restrict__ base) {
+  __shared__ int part[kCompactT / 32], own[kCompactT / 32];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int64_t m0 = (int64_t)blockIdx.x * (kCompactT / 8), g = (int64_t)blockIdx.x * kCompactT + tid;
+  int before = 0;  // (fewer than 2^31 items)
+  for (int64_t i = tid; i < m0 / 16; i += kCompactT) {
+    const uint4 v = reinterpret_cast<const uint4*>(masks)[i];
+    before += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
   }
-  const int64_t M = boff[k + 1] - boff[k];
-  const int64_t L = list_off[k + 1] - list_off[k];
-  const int ts = ts_class > 0 ? ts_class : tc::kTM;
-  const bool mine = ts_class <= 0 || slot_class(M) == ts_class;
-  wcnt[k] = (M > 0 && L > 0 && mine) ? cdiv(L, (int64_t)tn) * cdiv(M, (int64_t)ts) : 0;
+  before = __reduce_add_sync(0xffffffffu, before);
+  const bool keep = g / 8 < nmasks && ((masks[g / 8] >> (int)(g & 7)) & 1);
+  const unsigned kept = __ballot_sync(0xffffffffu, keep);
+  if (lane == 0) {
+    part[w] = before;
+    own[w] = __popc(kept);
+  }
+  __syncthreads();
+  int64_t at = __popc(kept & ((1u << lane) - 1u));
+#pragma unroll
+  for (int k = 0; k < kCompactT / 32; ++k) at += part[k] + (k < w ? own[k] : 0);
+  int64_t start = 0;
+  for (int c = 0; c <= kClasses; ++c) {
+    if (start == g) base[c] = at;
+    if (c < kClasses) start += cw.woff[c][ls.K];
+  }
+  if (keep) items[at] = class_decode(ls, cw, class_item(cw, ls.K, 0, g));
 }
 
-// work items (list, entry tile of tn entries, slot tile) of the batch's touched lists
-ListSched list_sched(const Index& ix, const FifPlan& P, int tn, Scratch& sc, cudaStream_t s, int ts_class = 0) {
-  const int K = ix.prm.n_codewords;
-  int64_t* wcnt = sc.get<int64_t>(K + 1);
-  int64_t* woff = sc.get<int64_t>(K + 1);
-  k_work_count_tc<<<(unsigned)cdiv(K + 1, 256), 256, 0, s>>>(P.boff, ix.list_off, K, tn, ts_class, wcnt);
-  GIFT_LAUNCHED("k_work_count_tc");
-  scan_exclusive_i64(wcnt, woff, K + 1, sc, s);
+ListSched list_sched(const Index& ix, const FifPlan& P, const int64_t* woff, int nkb) {
   ListSched ls;
   ls.woff = woff;
-  ls.K = K;
+  ls.K = ix.prm.n_codewords;
   ls.boff = P.boff;
   ls.list_off = ix.list_off;
-  ls.nkb = 0;
+  ls.nkb = nkb;
   return ls;
 }
 
 // E4M3 scan of the lists of one slot class
 template <int TS>
-void scan_fp8_class(const Index& ix, const FifPlan& P, const SlotInfo& si, const CUtensorMap& tA, const void* q8,
-                    int64_t qrows, Scratch& sc, cudaStream_t s, int grid) {
+void scan_fp8_class(const Index& ix, const FifPlan& P, const int64_t* woff, const SlotInfo& si, const CUtensorMap& tA,
+                    const void* q8, int64_t qrows, cudaStream_t s, int grid) {
   SlotsPolicy<1, 1, TS> pol;
-  static_cast<ListSched&>(pol) = list_sched(ix, P, tc::kTM, sc, s, TS);
-  pol.nkb = (int)cdiv((int64_t)ix.prm.dim, (int64_t)128);
+  static_cast<ListSched&>(pol) = list_sched(ix, P, woff, (int)cdiv((int64_t)ix.prm.dim, (int64_t)128));
   pol.si = si;
-  pol.item_map = nullptr;
-  pol.n_items = nullptr;
   const CUtensorMap tB = make_tmap_u8(q8, qrows, ix.prm.dim, TS);
   tc::launch_engine(tA, tB, tA, tB, pol, ix.d_err, grid, s);
 }
 
-// the rescore work of one slot class: its items that hold a candidate run
-// (slot classes of up to 80 slots: slot columns; 128: slot rows, RescorePolicy)
+// the rescore of one slot class's kept items (slot classes of up to 80 slots: slot columns; 128: slot rows)
+// tE, tE2: the entry rows (hi, lo), 128-row boxes
 template <int TS>
-struct RescoreClass {
+void rescore_class(const Index& ix, const FifPlan& P, const ListSched& ls, const SlotInfo& si, const KeptItems& kept,
+                   const int32_t* cand_sorted, int R, const CUtensorMap& tE, const CUtensorMap& tE2, const void* qhi,
+                   const void* qlo, int64_t qrows, int grid, cudaStream_t s) {
   using Pol = std::conditional_t<TS == 128, RescorePolicy, SlotsPolicy<2, 3, (TS < 128 ? TS : 64)>>;
   Pol pol;
-  void plan(const Index& ix, const FifPlan& P, const SlotInfo& si, const int32_t* cand_sorted, int R,
-            int64_t upper, int64_t* flags, int64_t* pos, Scratch& sc, cudaStream_t s) {
-    ListSched ls = list_sched(ix, P, kRescTN, sc, s, TS);
-    ls.nkb = (int)cdiv((int64_t)ix.prm.dim, (int64_t)64);
-    static_cast<ListSched&>(pol) = ls;
-    pol.si = si;
-    if constexpr (TS == 128) {
-      pol.cand = cand_sorted;
-      pol.R = R;
-    }
-    int64_t* item_map = sc.get<int64_t>(upper);
-    int64_t* n_items = sc.get<int64_t>(1);
-    k_resc_flags<TS><<<(unsigned)cdiv(upper, 8), 256, 0, s>>>(ls, P.slot_view, P.vquery, ix.entry_run,
-                                                             ix.list_shape, cand_sorted, R, upper, flags, P.stats);
-    GIFT_LAUNCHED("k_resc_flags");
-    scan_exclusive_i64(flags, pos, upper, sc, s);
-    k_compact_items<<<(unsigned)cdiv(upper, 256), 256, 0, s>>>(flags, pos, upper, item_map, n_items);
-    GIFT_LAUNCHED("k_compact_items");
-    pol.item_map = item_map;
-    pol.n_items = n_items;
+  static_cast<ListSched&>(pol) = ls;
+  pol.si = si;
+  pol.kept = kept;
+  const CUtensorMap tS = make_tmap_bf16(qhi, qrows, ix.prm.dim, TS);
+  const CUtensorMap tS2 = make_tmap_bf16(qlo, qrows, ix.prm.dim, TS);
+  if constexpr (TS == 128) {
+    pol.cand = cand_sorted;
+    pol.R = R;
+    tc::launch_engine(tS, tE, tS2, tE2, pol, ix.d_err, grid, s);  // slots are the MMA rows
+  } else {
+    tc::launch_engine(tE, tS, tE2, tS2, pol, ix.d_err, grid, s);
   }
-  // tE, tE2: the entry rows (hi, lo), 128-row boxes
-  void run(const Index& ix, const CUtensorMap& tE, const CUtensorMap& tE2, const void* qhi, const void* qlo,
-           int64_t qrows, int grid, cudaStream_t s) {
-    const CUtensorMap tS = make_tmap_bf16(qhi, qrows, ix.prm.dim, TS);
-    const CUtensorMap tS2 = make_tmap_bf16(qlo, qrows, ix.prm.dim, TS);
-    if constexpr (TS == 128)
-      tc::launch_engine(tS, tE, tS2, tE2, pol, ix.d_err, grid, s);  // slots are the MMA rows
-    else
-      tc::launch_engine(tE, tS, tE2, tS2, pol, ix.d_err, grid, s);
-  }
-};
+}
 
 }  // namespace
 
 void fif_rescore_stats(const Index& ix, const FifPlan& P, const int32_t* cand_sorted, int R, Scratch& sc,
                        cudaStream_t s) {
   if (!P.stats || P.nslots <= 0) return;
-  const ListSched ls = list_sched(ix, P, kRescTN, sc, s);
+  WorkSpecs specs;
+  specs.add(0, kRescTN, tc::kTM);
+  ClassWork cw{};
+  cw.woff[kClasses - 1] = plan_work(ix, P, specs, 0, sc, s);
   const int64_t upper = std::max<int64_t>(P.upper_items, 1);
-  int64_t* flags = sc.get<int64_t>(upper);
-  k_resc_flags<tc::kTM><<<(unsigned)cdiv(upper, 8), 256, 0, s>>>(ls, P.slot_view, P.vquery, ix.entry_run, ix.list_shape,
-                                                        cand_sorted, R, upper, flags, P.stats);
+  for (int c = 0; c < kClasses; ++c) cw.woff[c] = cw.woff[kClasses - 1];  // (only the last class's items are counted)
+  k_resc_flags<<<(unsigned)cdiv(upper, 8), 256, 0, s>>>(list_sched(ix, P, nullptr, 0), cw, kClasses - 1, P.slot_view,
+                                                        P.vquery, ix.entry_run, ix.list_shape, cand_sorted, R, nullptr,
+                                                        P.stats);
   GIFT_LAUNCHED("k_resc_flags");
 }
 
@@ -661,9 +709,9 @@ void fif_scan_tc(const Index& ix, const FifPlan& P, uint32_t* table, bool rescor
   }
   // the BF16 scan and the FP32-level pass schedule 128 slots x tn entries per item
   auto sched = [&](int tn) {
-    ListSched ls = list_sched(ix, P, tn, sc, s);
-    ls.nkb = (int)cdiv(D, 64);
-    return ls;
+    WorkSpecs specs;
+    specs.add(0, tn, tc::kTM);
+    return list_sched(ix, P, plan_work(ix, P, specs, 0, sc, s), (int)cdiv(D, 64));
   };
   SlotInfo si;
   si.runbase = P.runbase;
@@ -680,15 +728,15 @@ void fif_scan_tc(const Index& ix, const FifPlan& P, uint32_t* table, bool rescor
     // lists of up to 80 slots: list entries are the MMA rows, query slots the columns,
     // one launch per slot class
     const CUtensorMap tA = make_tmap_u8(ix.list_feat, ix.list_rows_alloc, D, tc::kTM);
+    const ClassWork cw = class_work(ix, P, sc, s);
     if (P.kc) P.kc->begin(1);
-    scan_fp8_class<16>(ix, P, si, tA, q8, qrows, sc, s, grid);
-    scan_fp8_class<32>(ix, P, si, tA, q8, qrows, sc, s, grid);
-    scan_fp8_class<64>(ix, P, si, tA, q8, qrows, sc, s, grid);
-    scan_fp8_class<80>(ix, P, si, tA, q8, qrows, sc, s, grid);
-    {  // lists of more than 80 slots: slots are the MMA rows, 256 entries per item
+    scan_fp8_class<16>(ix, P, cw.woff[0], si, tA, q8, qrows, s, grid);
+    scan_fp8_class<32>(ix, P, cw.woff[1], si, tA, q8, qrows, s, grid);
+    scan_fp8_class<64>(ix, P, cw.woff[2], si, tA, q8, qrows, s, grid);
+    scan_fp8_class<80>(ix, P, cw.woff[3], si, tA, q8, qrows, s, grid);
+    if (ns > 80) {  // lists of more than 80 slots: slots are the MMA rows, 256 entries per item
       ScanPolicy<1> pol;
-      static_cast<ListSched&>(pol) = list_sched(ix, P, kScanTN, sc, s, 128);
-      pol.nkb = (int)cdiv(D, 128);
+      static_cast<ListSched&>(pol) = list_sched(ix, P, cw.woff_scan128, (int)cdiv(D, 128));
       pol.si = si;
       const CUtensorMap tS = make_tmap_u8(q8, qrows, D, tc::kTM);
       const CUtensorMap tE = make_tmap_u8(ix.list_feat, ix.list_rows_alloc, D, ScanPolicy<1>::TN);
@@ -713,8 +761,6 @@ void fif_scan_tc(const Index& ix, const FifPlan& P, uint32_t* table, bool rescor
     pol.si.table = table32;
     pol.cand = nullptr;
     pol.R = 0;
-    pol.item_map = nullptr;
-    pol.n_items = nullptr;
     const CUtensorMap tA = make_tmap_bf16(qhi, qrows, D, tc::kTM);
     const CUtensorMap tB = make_tmap_bf16(ix.list_feat, ix.list_rows_alloc, D, RescorePolicy::TN);
     const CUtensorMap tA2 = make_tmap_bf16(qlo, qrows, D, tc::kTM);
@@ -728,28 +774,28 @@ void fif_scan_tc(const Index& ix, const FifPlan& P, uint32_t* table, bool rescor
     const void* bhi = ix.list_hi ? ix.list_hi : ix.list_feat;
     SlotInfo sr = si;
     sr.scale = ix.list_hi ? ix.list_scale_hi : ix.list_scale;
-    // the work items that hold a candidate run, per slot class, in their original order
+    // the work items that hold a candidate run, per slot class
+    const ClassWork cw = class_work(ix, P, sc, s);
     const int64_t upper = std::max<int64_t>(P.upper_items, 1);
-    int64_t* flags = sc.get<int64_t>(upper);
-    int64_t* pos = sc.get<int64_t>(upper);
-    RescoreClass<16> c16;
-    RescoreClass<32> c32;
-    RescoreClass<64> c64;
-    RescoreClass<80> c80;
-    RescoreClass<128> c128;
-    c16.plan(ix, P, sr, cand_sorted, R, upper, flags, pos, sc, s);
-    c32.plan(ix, P, sr, cand_sorted, R, upper, flags, pos, sc, s);
-    c64.plan(ix, P, sr, cand_sorted, R, upper, flags, pos, sc, s);
-    c80.plan(ix, P, sr, cand_sorted, R, upper, flags, pos, sc, s);
-    c128.plan(ix, P, sr, cand_sorted, R, upper, flags, pos, sc, s);
+    const int64_t nmasks = cdiv(upper, (int64_t)8);
+    uint8_t* masks = sc.get<uint8_t>(nmasks);
+    ListItem* items = sc.get<ListItem>(upper);
+    int64_t* base = sc.get<int64_t>(kClasses + 1);
+    const ListSched ls = list_sched(ix, P, nullptr, (int)cdiv((int64_t)D, (int64_t)64));
+    k_resc_flags<<<(unsigned)nmasks, 256, 0, s>>>(ls, cw, 0, P.slot_view, P.vquery, ix.entry_run, ix.list_shape,
+                                                  cand_sorted, R, masks, P.stats);
+    GIFT_LAUNCHED("k_resc_flags");
+    k_resc_compact<<<(unsigned)(8 * nmasks / kCompactT + 1), kCompactT, 0, s>>>(ls, cw, masks, nmasks, items, base);
+    GIFT_LAUNCHED("k_resc_compact");
     const CUtensorMap tA = make_tmap_bf16(bhi, ix.list_rows_alloc, D, tc::kTM);
     const CUtensorMap tA2 = make_tmap_bf16(ix.list_lo, ix.list_rows_alloc, D, tc::kTM);
     if (P.kc) P.kc->begin(2);
-    c16.run(ix, tA, tA2, qhi, qlo, qrows, grid, s);
-    c32.run(ix, tA, tA2, qhi, qlo, qrows, grid, s);
-    c64.run(ix, tA, tA2, qhi, qlo, qrows, grid, s);
-    c80.run(ix, tA, tA2, qhi, qlo, qrows, grid, s);
-    c128.run(ix, tA, tA2, qhi, qlo, qrows, grid, s);
+    auto kept = [&](int c) { return KeptItems{items, base + c}; };
+    rescore_class<16>(ix, P, ls, sr, kept(0), cand_sorted, R, tA, tA2, qhi, qlo, qrows, grid, s);
+    rescore_class<32>(ix, P, ls, sr, kept(1), cand_sorted, R, tA, tA2, qhi, qlo, qrows, grid, s);
+    rescore_class<64>(ix, P, ls, sr, kept(2), cand_sorted, R, tA, tA2, qhi, qlo, qrows, grid, s);
+    rescore_class<80>(ix, P, ls, sr, kept(3), cand_sorted, R, tA, tA2, qhi, qlo, qrows, grid, s);
+    if (ns > 80) rescore_class<128>(ix, P, ls, sr, kept(4), cand_sorted, R, tA, tA2, qhi, qlo, qrows, grid, s);
     if (P.kc) P.kc->end(2);
   }
 }

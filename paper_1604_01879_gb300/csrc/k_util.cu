@@ -106,9 +106,32 @@ __global__ __launch_bounds__(kScanT) void k_scan_blocks(const int64_t* __restric
   if (tid == kScanT - 1) block_sums[blockIdx.x] = run;
 }
 
-__global__ void k_scan_add(int64_t* __restrict__ out, int64_t n, const int64_t* __restrict__ offs) {
+// out[i] += the exclusive prefix of its block's sum
+__global__ void k_scan_shift(int64_t* __restrict__ out, int64_t n, const int64_t* __restrict__ offs) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] += offs[i / kScanPerBlock];
+}
+
+// out[i] += the sums of the blocks before i's: each block adds them up itself
+__global__ __launch_bounds__(kScanT) void k_scan_add(int64_t* __restrict__ out, int64_t n,
+                                                     const int64_t* __restrict__ sums) {
+  __shared__ int64_t part[kScanT / 32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int64_t b = blockIdx.x + 1;  // block 0 has none before it
+  int64_t v = 0;
+  for (int64_t i = tid; i < b; i += kScanT) v += sums[i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
+  if (lane == 0) part[tid >> 5] = v;
+  __syncthreads();
+  v = 0;
+#pragma unroll
+  for (int w = 0; w < kScanT / 32; ++w) v += part[w];
+#pragma unroll
+  for (int k = 0; k < kScanItems; ++k) {
+    const int64_t i = b * kScanPerBlock + (int64_t)k * kScanT + tid;
+    if (i < n) out[i] += v;
+  }
 }
 
 // ---------------------------------------------------------------- radix sort
@@ -194,18 +217,24 @@ void launch_fill_i32(int32_t* p, int64_t n, int32_t v, cudaStream_t s) {
   GIFT_LAUNCHED("k_fill_i32");
 }
 
+// Two launches: blocks of 2,048, then each later block adds the sums before it (at most 8,192 of them, read
+// from L2; a third launch for their prefix costs more below that). Longer arrays scan the sums first.
 void scan_exclusive_i64(const int64_t* in, int64_t* out, int64_t n, Scratch& sc, cudaStream_t s) {
   if (n <= 0) return;
   const int64_t nb = cdiv(n, kScanPerBlock);
   int64_t* sums = sc.get<int64_t>(nb);
   k_scan_blocks<<<(unsigned)nb, kScanT, 0, s>>>(in, out, n, sums);
   GIFT_LAUNCHED("k_scan_blocks");
-  if (nb > 1) {
-    int64_t* sums_x = sc.get<int64_t>(nb);
-    scan_exclusive_i64(sums, sums_x, nb, sc, s);
-    k_scan_add<<<(unsigned)cdiv(n, 256), 256, 0, s>>>(out, n, sums_x);
+  if (nb <= 1) return;
+  if (nb <= 8192) {
+    k_scan_add<<<(unsigned)(nb - 1), kScanT, 0, s>>>(out, n, sums);
     GIFT_LAUNCHED("k_scan_add");
+    return;
   }
+  int64_t* sums_x = sc.get<int64_t>(nb);
+  scan_exclusive_i64(sums, sums_x, nb, sc, s);
+  k_scan_shift<<<(unsigned)cdiv(n, 256), 256, 0, s>>>(out, n, sums_x);
+  GIFT_LAUNCHED("k_scan_shift");
 }
 
 void stable_sort_by_key(const int32_t* keys, int64_t n, int32_t nbins, int32_t* perm_out,
