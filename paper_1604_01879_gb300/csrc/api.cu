@@ -381,9 +381,11 @@ void run_fif(Index& ix, const float* q, int64_t nv, const std::vector<int32_t>& 
     vquery = t;
   }
   float* q_inv = sc.get<float>(nv);
-  launch_row_invnorm(q, nv, ix.prm.dim, q_inv, s);
+  SplitRows parts;
+  if (nv <= kAssignChunk) parts = split_for_assign(q, nv, ix.prm.dim, q_inv, sc, s);
+  else launch_row_invnorm(q, nv, ix.prm.dim, q_inv, s);
   int32_t* q_code = sc.get<int32_t>(nv * ma);
-  assign_codes(ix, q, nv, ma, q_code, sc, s, q_inv, &tm.kc);
+  assign_codes(ix, q, nv, ma, q_code, sc, s, q_inv, &tm.kc, parts.hi ? &parts : nullptr);
 
   tm.mark(ST_BUCKET);
   FifPlan P;

@@ -182,7 +182,8 @@ struct SplitRows {
   __nv_bfloat16* hi = nullptr;  // [n + padding, D]
   __nv_bfloat16* lo = nullptr;
 };
-SplitRows split_for_assign(const float* X, int64_t n, int D, Scratch& sc, cudaStream_t s);
+// the two-part copy and 1/||x|| of the rows, from one read
+SplitRows split_for_assign(const float* X, int64_t n, int D, float* inv, Scratch& sc, cudaStream_t s);
 void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* codes,
                   Scratch& sc, cudaStream_t s, const float* x_inv = nullptr, KernelClock* kc = nullptr,
                   const SplitRows* parts = nullptr, const float* cb_max = nullptr);

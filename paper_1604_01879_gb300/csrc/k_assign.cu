@@ -403,6 +403,45 @@ __global__ void k_split_rows(const float* __restrict__ X, int64_t n, int D, __nv
   reinterpret_cast<__nv_bfloat162*>(lo)[2 * i + 1] = __floats2bfloat162_rn(v.z - fb.x, v.w - fb.y);
 }
 
+// the same and 1 / ||x|| of each row (0 for a zero row) from one read; warp per row, the norm's terms added as
+// k_row_invnorm adds them
+__global__ __launch_bounds__(256) void k_split_norm(const float* __restrict__ X, int64_t n, int D,
+                                                    __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
+                                                    float* __restrict__ inv) {
+  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (row >= n) return;
+  const float4* p = reinterpret_cast<const float4*>(X + row * (int64_t)D);
+  uint2* h = reinterpret_cast<uint2*>(hi + row * (int64_t)D);
+  uint2* l = reinterpret_cast<uint2*>(lo + row * (int64_t)D);
+  float acc = 0.f;
+  for (int base = lane; base < (D >> 2); base += 32 * 8) {
+    float4 x[8];  // eight reads in flight
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (base + 32 * k < (D >> 2)) x[k] = p[base + 32 * k];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int i = base + 32 * k;
+      if (i >= (D >> 2)) break;
+      const float4 v = x[k];
+      acc = fmaf(v.x, v.x, acc);
+      acc = fmaf(v.y, v.y, acc);
+      acc = fmaf(v.z, v.z, acc);
+      acc = fmaf(v.w, v.w, acc);
+      const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+      const float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
+      const __nv_bfloat162 c = __floats2bfloat162_rn(v.x - fa.x, v.y - fa.y);
+      const __nv_bfloat162 d = __floats2bfloat162_rn(v.z - fb.x, v.w - fb.y);
+      h[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      l[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&c), *reinterpret_cast<const uint32_t*>(&d));
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(kFull, acc, o);
+  if (lane == 0) inv[row] = acc > 0.f ? 1.0f / sqrtf(acc) : 0.f;
+}
+
 }  // namespace
 
 void split_rows_bf16(const float* X, int64_t n, int D, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t s) {
@@ -412,12 +451,14 @@ void split_rows_bf16(const float* X, int64_t n, int D, __nv_bfloat16* hi, __nv_b
   GIFT_LAUNCHED("k_split_rows");
 }
 
-SplitRows split_for_assign(const float* X, int64_t n, int D, Scratch& sc, cudaStream_t s) {
+SplitRows split_for_assign(const float* X, int64_t n, int D, float* inv, Scratch& sc, cudaStream_t s) {
   SplitRows r;
   const int64_t rows_alloc = n + tc::kTM;  // one box of padding rows
   r.hi = sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
   r.lo = sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
-  split_rows_bf16(X, n, D, r.hi, r.lo, s);
+  if (n <= 0) return r;
+  k_split_norm<<<(unsigned)cdiv(n, 8), 256, 0, s>>>(X, n, D, r.hi, r.lo, inv);
+  GIFT_LAUNCHED("k_split_norm");
   return r;
 }
 

@@ -58,8 +58,8 @@ __global__ void k_scan_stats(const int64_t* __restrict__ boff, const int64_t* __
   }
 }
 
-// inclusive prefix sum of one int64 per thread over a block of 1,024; wsum: 32 words
-__device__ __forceinline__ int64_t block_incl_i64(int64_t v, int64_t* wsum) {
+// inclusive prefix sum of one int64 per thread over a block of 1,024, and the block's total; wsum: 33 words
+__device__ __forceinline__ int64_t block_incl_i64(int64_t v, int64_t* wsum, int64_t& total) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -69,9 +69,20 @@ __device__ __forceinline__ int64_t block_incl_i64(int64_t v, int64_t* wsum) {
   __syncthreads();  // wsum may still be read from the call before
   if (lane == 31) wsum[w] = v;
   __syncthreads();
-  int64_t before = 0;
-  for (int k = 0; k < w; ++k) before += wsum[k];
-  return v + before;
+  if (w == 0) {
+    const int64_t y = wsum[lane];
+    int64_t z = y;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t q = __shfl_up_sync(0xffffffffu, z, o);
+      if (lane >= o) z += q;
+    }
+    wsum[lane] = z - y;
+    if (lane == 31) wsum[32] = z;
+  }
+  __syncthreads();
+  total = wsum[32];
+  return v + wsum[w];
 }
 
 constexpr int kPlanT = 1024;
@@ -81,7 +92,7 @@ __global__ __launch_bounds__(kPlanT) void k_plan_work(const int64_t* __restrict_
                                                       const int64_t* __restrict__ list_off, int K,
                                                       const WorkSpecs specs, int64_t fold,
                                                       int64_t* __restrict__ woff) {
-  __shared__ int64_t wsum[kPlanT / 32];
+  __shared__ int64_t wsum[kPlanT / 32 + 1];
   __shared__ unsigned long long s_items;
   __shared__ int s_most;
   const int tid = threadIdx.x, c = blockIdx.x;
@@ -127,10 +138,10 @@ __global__ __launch_bounds__(kPlanT) void k_plan_work(const int64_t* __restrict_
     for (int i = 0; i < 4; ++i) {
       const int k = k0 + i * kPlanT + tid;
       if (k0 + i * kPlanT > K) break;
-      const int64_t incl = block_incl_i64(n[i], wsum);
+      int64_t total;
+      const int64_t incl = block_incl_i64(n[i], wsum, total);
       if (k <= K) out[k] = run + incl - n[i];
-#pragma unroll
-      for (int w = 0; w < kPlanT / 32; ++w) run += wsum[w];
+      run += total;
     }
   }
 }
@@ -147,7 +158,7 @@ __global__ __launch_bounds__(kPlanT) void k_slots_small(const int32_t* __restric
                                                         int64_t* __restrict__ runbase) {
   __shared__ unsigned long long key[kSmallSlots];
   __shared__ uint32_t id[kSmallSlots];
-  __shared__ int64_t wsum[kPlanT / 32];
+  __shared__ int64_t wsum[kPlanT / 32 + 1];
   const int tid = threadIdx.x;
   int P = 64;
   while (P < n) P <<= 1;
@@ -167,10 +178,10 @@ __global__ __launch_bounds__(kPlanT) void k_slots_small(const int32_t* __restric
       view_slot[item] = s;
       cells = nruns[k];
     }
-    const int64_t incl = block_incl_i64(cells, wsum);
+    int64_t total;
+    const int64_t incl = block_incl_i64(cells, wsum, total);
     if (s <= n) runbase[s] = run + incl - cells;
-#pragma unroll
-    for (int w = 0; w < kPlanT / 32; ++w) run += wsum[w];
+    run += total;
   }
   for (int k = tid; k <= K; k += kPlanT) {  // the first slot of a code >= k
     int lo = 0, hi = n;

@@ -110,7 +110,6 @@ void kmeans(const float* X, int64_t n, int D, int K, const std::vector<int32_t>&
   k_km_rows<<<(unsigned)K, 256, 0, s>>>(X, D, d_init, K, tmp.codebook);
   GIFT_LAUNCHED("k_km_rows");
   float* x_inv = sc.get<float>(n);
-  launch_row_invnorm(X, n, D, x_inv, s);
   float* C_new = sc.get<float>((size_t)K * D);
   int32_t* lab = sc.get<int32_t>(n);
   int32_t* perm = sc.get<int32_t>(n);
@@ -120,7 +119,8 @@ void kmeans(const float* X, int64_t n, int D, int K, const std::vector<int32_t>&
   std::vector<int64_t> h_off((size_t)K + 1);
   // rows of one quantiser pass: their two-part copy is the same in every iteration
   SplitRows parts;
-  if (iters > 0 && n <= kAssignChunk) parts = split_for_assign(X, n, D, sc, s);
+  if (iters > 0 && n <= kAssignChunk) parts = split_for_assign(X, n, D, x_inv, sc, s);
+  else launch_row_invnorm(X, n, D, x_inv, s);
   for (int it = 0; it < iters; ++it) {
     Scratch isc(s);
     const float* cb_max = prepare_codebook_async(tmp, isc, s);

@@ -411,50 +411,68 @@ struct SlotsPolicy : ListSched {
   }
 };
 
-// slot-ordered BF16 copies of the query views: hi = bf16(q), lo = bf16(q - hi)
-__global__ void k_slot_split(const float* __restrict__ q, const int32_t* __restrict__ slot_view, int64_t nslots,
-                             int D, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
-  const int64_t s = blockIdx.x;
-  if (s >= nslots) return;
-  const float4* src = reinterpret_cast<const float4*>(q + (int64_t)slot_view[s] * D);
-  __nv_bfloat162* h2 = reinterpret_cast<__nv_bfloat162*>(hi + s * D);
-  __nv_bfloat162* l2 = lo ? reinterpret_cast<__nv_bfloat162*>(lo + s * D) : nullptr;
-  for (int i = threadIdx.x; i < D / 4; i += blockDim.x) {
-    const float4 v = src[i];
-    const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y);
-    const __nv_bfloat162 b = __floats2bfloat162_rn(v.z, v.w);
-    h2[2 * i] = a;
-    h2[2 * i + 1] = b;
-    if (l2) {
-      const float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
-      l2[2 * i] = __floats2bfloat162_rn(v.x - fa.x, v.y - fa.y);
-      l2[2 * i + 1] = __floats2bfloat162_rn(v.z - fb.x, v.w - fb.y);
-    }
+// Slot-ordered copies of the query views: BF16 parts hi = bf16(q), lo = bf16(q - hi) (each optional) and E4M3 rows
+// (optional) with one scale per slot, stored = q / scale, scale = max|q| / 448 (the largest finite E4M3 value). A
+// block reads a view once and writes it to each of its ma slots: bound by those bytes (16,384 views of D = 4096, MA =
+// 2, all three copies: 0.94 GB), where a block per slot and a kernel per copy read every view six times (446 us
+// against 138).
+constexpr int kSlotT = 256, kSlotHeld = 4;  // float4s of a row held per thread: D up to 4,096 is read once
+__global__ __launch_bounds__(kSlotT) void k_slot_rows(const float* __restrict__ q,
+                                                      const int32_t* __restrict__ view_slot, int ma, int D,
+                                                      __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
+                                                      uint32_t* __restrict__ out8, float* __restrict__ scale) {
+  __shared__ float red[kSlotT / 32];
+  const int64_t v = blockIdx.x;
+  const float4* src = reinterpret_cast<const float4*>(q + v * D);
+  const int n4 = D / 4;
+  float4 held[kSlotHeld];
+#pragma unroll
+  for (int k = 0; k < kSlotHeld; ++k) {
+    const int i = threadIdx.x + k * kSlotT;
+    if (i < n4) held[k] = src[i];
   }
-}
-
-// slot-ordered E4M3 copies of the query views with one scale per slot:
-// stored = q / scale, scale = max|q| / 448 (the largest finite E4M3 value)
-__global__ __launch_bounds__(256) void k_slot_fp8(const float* __restrict__ q, const int32_t* __restrict__ slot_view,
-                                                  int64_t nslots, int D, __nv_fp8_e4m3* __restrict__ out,
-                                                  float* __restrict__ scale) {
-  __shared__ float red[8];
-  const int64_t s = blockIdx.x;
-  if (s >= nslots) return;
-  const float* src = q + (int64_t)slot_view[s] * D;
-  float m = 0.f;
-  for (int i = threadIdx.x; i < D; i += blockDim.x) m = fmaxf(m, fabsf(src[i]));
+  float sc = 1.f, inv = 1.f;
+  if (out8) {
+    float m = 0.f;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  float mx = 0.f;
+    for (int k = 0; k < kSlotHeld; ++k)
+      if (threadIdx.x + k * kSlotT < n4)
+        m = fmaxf(m, fmaxf(fmaxf(fabsf(held[k].x), fabsf(held[k].y)), fmaxf(fabsf(held[k].z), fabsf(held[k].w))));
+    for (int i = threadIdx.x + kSlotHeld * kSlotT; i < n4; i += kSlotT) {
+      const float4 x = src[i];
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))));
+    }
 #pragma unroll
-  for (int w = 0; w < 8; ++w) mx = fmaxf(mx, red[w]);
-  const float sc = mx > 0.f ? mx / 448.f : 1.f;
-  const float inv = 1.f / sc;
-  for (int i = threadIdx.x; i < D; i += blockDim.x) out[s * D + i] = __nv_fp8_e4m3(src[i] * inv);
-  if (threadIdx.x == 0) scale[s] = sc;
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    float mx = 0.f;
+#pragma unroll
+    for (int w = 0; w < kSlotT / 32; ++w) mx = fmaxf(mx, red[w]);
+    sc = mx > 0.f ? mx / 448.f : 1.f;
+    inv = 1.f / sc;
+  }
+  auto put = [&](int i, const float4 x) {
+    const __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y), b = __floats2bfloat162_rn(x.z, x.w);
+    const float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
+    const __nv_bfloat162 c = __floats2bfloat162_rn(x.x - fa.x, x.y - fa.y);
+    const __nv_bfloat162 d = __floats2bfloat162_rn(x.z - fb.x, x.w - fb.y);
+    const uint2 h = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    const uint2 l = make_uint2(*reinterpret_cast<const uint32_t*>(&c), *reinterpret_cast<const uint32_t*>(&d));
+    uint32_t e = 0u;
+    if (out8) e = __nv_fp8x4_e4m3(make_float4(x.x * inv, x.y * inv, x.z * inv, x.w * inv)).__x;
+    for (int t = 0; t < ma; ++t) {
+      const int64_t o = (int64_t)view_slot[v * ma + t] * n4 + i;
+      if (hi) reinterpret_cast<uint2*>(hi)[o] = h;
+      if (lo) reinterpret_cast<uint2*>(lo)[o] = l;
+      if (out8) out8[o] = e;
+    }
+  };
+#pragma unroll
+  for (int k = 0; k < kSlotHeld; ++k)
+    if (threadIdx.x + k * kSlotT < n4) put(threadIdx.x + k * kSlotT, held[k]);
+  for (int i = threadIdx.x + kSlotHeld * kSlotT; i < n4; i += kSlotT) put(i, src[i]);
+  if (out8 && (int)threadIdx.x < ma) scale[view_slot[v * ma + threadIdx.x]] = sc;
 }
 
 // The slot classes of a batch: offsets of their work items over the lists (128 entries per item; the last class,
@@ -689,21 +707,21 @@ void fif_scan_tc(const Index& ix, const FifPlan& P, uint32_t* table, bool rescor
   __nv_bfloat16* qlo = nullptr;
   __nv_fp8_e4m3* q8 = nullptr;
   float* q8s = nullptr;
-  if (fp8) {
-    q8 = sc.get<__nv_fp8_e4m3>((size_t)qrows * D);
-    q8s = sc.get<float>(ns);
-    k_slot_fp8<<<(unsigned)ns, 256, 0, s>>>(P.q, P.slot_view, ns, D, q8, q8s);
-    GIFT_LAUNCHED("k_slot_fp8");
-  } else if (P.slot_hi && (P.slot_lo || !rescore)) {
+  // the parts a rescore of this batch will need are made with the scan's rows, and reused there
+  const bool parts = rescore || (ix.prm.rescore_r > 0 && ix.list_lo != nullptr);
+  if (!fp8 && P.slot_hi && (P.slot_lo || !rescore)) {
     qhi = P.slot_hi;  // made by the scan of this batch
     qlo = P.slot_lo;
   } else {
-    // the low parts too when this index rescores next, so the rescore reuses both
-    const bool want_lo = rescore || (ix.prm.rescore_r > 0 && ix.list_lo != nullptr);
-    qhi = sc.get<__nv_bfloat16>((size_t)qrows * D);
-    qlo = want_lo ? sc.get<__nv_bfloat16>((size_t)qrows * D) : nullptr;
-    k_slot_split<<<(unsigned)ns, 256, 0, s>>>(P.q, P.slot_view, ns, D, qhi, qlo);
-    GIFT_LAUNCHED("k_slot_split");
+    if (fp8) {
+      q8 = sc.get<__nv_fp8_e4m3>((size_t)qrows * D);
+      q8s = sc.get<float>(ns);
+    }
+    if (!fp8 || parts) qhi = sc.get<__nv_bfloat16>((size_t)qrows * D);
+    if (parts) qlo = sc.get<__nv_bfloat16>((size_t)qrows * D);
+    k_slot_rows<<<(unsigned)P.nv, kSlotT, 0, s>>>(P.q, P.view_slot, P.ma, D, qhi, qlo, reinterpret_cast<uint32_t*>(q8),
+                                                  q8s);
+    GIFT_LAUNCHED("k_slot_rows");
     P.slot_hi = qhi;
     P.slot_lo = qlo;
   }
