@@ -26,11 +26,20 @@ namespace gift {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kT = 16;    // coarse candidates kept per row and chunk
-constexpr int TNA = 256;  // codewords per chunk (AssignPolicy::TN)
+// coarse scores kept per row and chunk of tn codewords: the best 16, or all 32 (which spares the epilogue its
+// insertions, most of a small item's time)
+__host__ __device__ constexpr int kept_scores(int tn) { return tn == 32 ? 32 : 16; }
 
+// TN_: codewords per chunk. 256 where the (row tile, chunk) items fill the SMs; with few rows 64 or 32, whose more
+// items run on more SMs at once with more stages in flight: an item's time is a chain of D / 64 k-blocks, 1.7 us each
+// with two stages of 96 KB, 0.6 us with five of 40 KB (108 rows, D = 4096, K = 512: 110 us against 44, and the refine
+// 52 against 20 with a block per row).
+template <int TN_>
 struct AssignPolicy {
-  static constexpr int TN = TNA, NBUF = 2, STAGES = 2, SPLIT = 3, EB = 2;
+  static constexpr int TN = TN_, NBUF = 2, SPLIT = 3, EB = 2;
+  static constexpr int STAGES = TN_ == 256 ? 2 : TN_ == 64 ? 4 : 5;
+  static constexpr int kT = kept_scores(TN_);
+  static constexpr bool kAll = kT == TN_;
   static constexpr int kWarpSmem = TN * 4;
   int64_t n;          // rows
   int K;
@@ -79,6 +88,18 @@ struct AssignPolicy {
       hs[j] = k < K ? half_sq[k] : INFINITY;
     }
     __syncwarp();
+    if constexpr (kAll) {
+      uint32_t r[32];
+      tc::tmem_ld32(taddr, r);
+      tc::tmem_wait_ld();
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        x.val[j] = __uint_as_float(r[j]) - hs[j];
+        x.idx[j] = c * TN + j < K ? c * TN + j : 0x7fffffff;
+      }
+      __syncwarp();
+      return;
+    }
     const int npieces = min(TN, K - c * TN + 31) >> 5;
     for (int pc = 0; pc < npieces; ++pc) {
       uint32_t r[32];
@@ -123,55 +144,26 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   e = (a - (s - bb)) + (b - bb);
 }
 
-// exact-ish ||x - b||^2 as a normalised two-float (hi, lo), warp cooperative
-__device__ void dist_df(const float* __restrict__ x, const float* __restrict__ b, int D, int lane, float& ohi,
-                        float& olo) {
-  float hi = 0.f, lo = 0.f;
-  for (int d = lane * 4; d < D; d += 128) {
-    const float4 xv = *reinterpret_cast<const float4*>(x + d);
-    const float4 bv = *reinterpret_cast<const float4*>(b + d);
-    const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
-    const float bs[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      float s, e;
-      two_sum(xs[c], -bs[c], s, e);  // x - b = s + e exactly
-      const float p = s * s;
-      float pe = fmaf(s, s, -p);     // s^2 = p + pe exactly
-      pe = fmaf(2.f * s, e, pe);     // + 2 s e (e^2 is below 2^-48 s^2)
-      float t, te;
-      two_sum(hi, p, t, te);
-      hi = t;
-      lo += te + pe;
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float h2 = __shfl_xor_sync(kFull, hi, o);
-    const float l2 = __shfl_xor_sync(kFull, lo, o);
-    float t, te;
-    two_sum(hi, h2, t, te);
-    hi = t;
-    lo = lo + l2 + te;
-  }
-  float t, te;
-  two_sum(hi, lo, t, te);
-  ohi = t;
-  olo = te;
-}
-
-// the same two-float distances for up to kBatch candidates at once: each chunk
-// of the row is read once and compared with every candidate
+// the two-float distances ||x - b||^2 of up to kBatch candidates at once: each chunk
+// of the row is read once and compared with every candidate. WPR warps share a
+// row (warp `sub` takes every WPR-th 128 elements; their sums are added in warp order
+// through `part`, and all of the block's threads call this together).
 constexpr int kBatch = 8;
+struct DfPart {
+  float hi[8], lo[8];
+};
+template <int WPR>
 __device__ void dist_df_batch(const float* __restrict__ x, const float* __restrict__ cb, const int (&kc)[kBatch],
-                              int n, int D, int lane, float (&ohi)[kBatch], float (&olo)[kBatch]) {
+                              int n, int D, int lane, int sub, DfPart* part, float (&ohi)[kBatch],
+                              float (&olo)[kBatch]) {
   float hi[kBatch], lo[kBatch];
 #pragma unroll
   for (int c = 0; c < kBatch; ++c) {
     hi[c] = 0.f;
     lo[c] = 0.f;
   }
-  for (int d = lane * 4; d < D; d += 128) {
+#pragma unroll(WPR == 1 ? 1 : 2)
+  for (int d = (sub * 32 + lane) * 4; d < D; d += 128 * WPR) {
     const float4 xv = *reinterpret_cast<const float4*>(x + d);
     const float xs[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
@@ -182,10 +174,10 @@ __device__ void dist_df_batch(const float* __restrict__ x, const float* __restri
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         float s2, e;
-        two_sum(xs[q], -bs[q], s2, e);
+        two_sum(xs[q], -bs[q], s2, e);  // x - b = s2 + e exactly
         const float p = s2 * s2;
-        float pe = fmaf(s2, s2, -p);
-        pe = fmaf(2.f * s2, e, pe);
+        float pe = fmaf(s2, s2, -p);    // s2^2 = p + pe exactly
+        pe = fmaf(2.f * s2, e, pe);     // + 2 s2 e (e^2 is below 2^-48 s2^2)
         float t, te;
         two_sum(hi[c], p, t, te);
         hi[c] = t;
@@ -205,6 +197,33 @@ __device__ void dist_df_batch(const float* __restrict__ x, const float* __restri
       hi[c] = t;
       lo[c] = lo[c] + l2 + te;
     }
+  }
+  if constexpr (WPR > 1) {
+    __syncthreads();  // part may still be read from the call before
+    if (lane == 0)
+#pragma unroll
+      for (int c = 0; c < kBatch; ++c) {
+        part[sub].hi[c] = hi[c];
+        part[sub].lo[c] = lo[c];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < kBatch; ++c) {
+      if (c >= n) break;
+      hi[c] = part[0].hi[c];
+      lo[c] = part[0].lo[c];
+#pragma unroll
+      for (int w = 1; w < WPR; ++w) {
+        float t, te;
+        two_sum(hi[c], part[w].hi[c], t, te);
+        hi[c] = t;
+        lo[c] = lo[c] + part[w].lo[c] + te;
+      }
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < kBatch; ++c) {
+    if (c >= n) break;
     float t, te;
     two_sum(hi[c], lo[c], t, te);
     ohi[c] = t;
@@ -244,16 +263,20 @@ __device__ __forceinline__ void next_best(const float* __restrict__ v, const int
   }
 }
 
+// WPR: warps per row, 1, or 8 (a block per row) where the rows are few: a row's distances are then eight times
+// shorter chains of dependent reads
+template <int WPR>
 __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__ X, int64_t n, int D,
                                                        const float* __restrict__ cb, int K, int ma,
                                                        const float* __restrict__ cval,
-                                                       const int32_t* __restrict__ cidx, int nch,
+                                                       const int32_t* __restrict__ cidx, int nch, int tn, int kT,
                                                        const float* __restrict__ x_inv, float bmax_host,
                                                        const float* __restrict__ bmax_dev,
                                                        int32_t* __restrict__ codes) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t r = (int64_t)blockIdx.x * 8 + w;
-  if (r >= n) return;
+  __shared__ DfPart part[8];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = w % WPR;
+  const int64_t r = (int64_t)blockIdx.x * (8 / WPR) + w / WPR;
+  if (r >= n) return;  // (with a block per row every warp decides everything alike)
   const float* x = X + r * (int64_t)D;
   const int tot = nch * kT;
   const float* v = cval + r * tot;
@@ -279,7 +302,7 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
   bool full = xi == 0.f || found < ma;  // (fewer kept scores than ma only with non-finite inputs)
   for (int c = lane; c < nch; c += 32) {
     const int e = c * kT + kT - 1;
-    if (id[e] != 0x7fffffff && v[e] >= lim && min(TNA, K - c * TNA) > kT) full = true;
+    if (id[e] != 0x7fffffff && v[e] >= lim && min(tn, K - c * tn) > kT) full = true;
   }
   full = __any_sync(kFull, full);
   if (!full && ma == 1) {
@@ -295,7 +318,7 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
       cnt += __popc(m);
     }
     if (cnt == 1) {
-      if (lane == 0) codes[r] = only;
+      if (lane == 0 && sub == 0) codes[r] = only;
       return;
     }
   }
@@ -350,7 +373,7 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
     }
     if (n <= kBatch) {
       float hh[kBatch], ll[kBatch];
-      dist_df_batch(x, cb, kc, n, D, lane, hh, ll);
+      dist_df_batch<WPR>(x, cb, kc, n, D, lane, sub, part, hh, ll);
 #pragma unroll
       for (int c = 0; c < kBatch; ++c)
         if (c < n) insert(hh[c], ll[c], kc[c]);
@@ -374,12 +397,15 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
       const int j = __ffs(mask) - 1;
       mask &= mask - 1;
       const int k = __shfl_sync(kFull, kk, j);
-      float h, l;
-      dist_df(x, cb + (int64_t)k * D, D, lane, h, l);
-      insert(h, l, k);
+      float hh[kBatch], ll[kBatch];
+      int kc[kBatch];
+#pragma unroll
+      for (int c = 0; c < kBatch; ++c) kc[c] = k;
+      dist_df_batch<WPR>(x, cb, kc, 1, D, lane, sub, part, hh, ll);
+      insert(hh[0], ll[0], k);
     }
   }
-  if (lane < ma) {
+  if (lane < ma && sub == 0) {
     int out = Kx[0];
 #pragma unroll
     for (int a = 1; a < GIFT_MAX_MA; ++a)
@@ -472,7 +498,12 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
   GIFT_REQUIRE(!parts || n <= chunk, "a two-part copy made before covers one pass");
   __nv_bfloat16* hi = parts ? parts->hi : sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
   __nv_bfloat16* lo = parts ? parts->lo : sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
-  const int nch = (int)cdiv(K, TNA);
+  const int sms = device_sm_count();
+  // codewords per item: as many as leave an item for every SM (one pass over the rows)
+  const int64_t row_tiles = cdiv(chunk, (int64_t)tc::kTM);
+  // (a vocabulary of more than 1,024 keeps 64: the refine reads kT scores per chunk and row)
+  const int tn = row_tiles * cdiv(K, 256) >= sms ? 256 : K > 1024 || row_tiles * cdiv(K, 64) >= sms ? 64 : 32;
+  const int nch = (int)cdiv(K, tn), kT = kept_scores(tn);
   float* cval = sc.get<float>((size_t)chunk * nch * kT);
   int32_t* cidx = sc.get<int32_t>((size_t)chunk * nch * kT);
   float* inv = nullptr;
@@ -481,31 +512,38 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
     launch_row_invnorm(X, n, D, inv, s);
     x_inv = inv;
   }
-  const CUtensorMap tB = make_tmap_bf16(ix.cb_hi, ix.cb_rows_alloc, D, AssignPolicy::TN);
-  const CUtensorMap tB2 = make_tmap_bf16(ix.cb_lo, ix.cb_rows_alloc, D, AssignPolicy::TN);
-  const int sms = device_sm_count();
+  const CUtensorMap tB = make_tmap_bf16(ix.cb_hi, ix.cb_rows_alloc, D, tn);
+  const CUtensorMap tB2 = make_tmap_bf16(ix.cb_lo, ix.cb_rows_alloc, D, tn);
   for (int64_t r0 = 0; r0 < n; r0 += chunk) {
     const int64_t m = std::min(chunk, n - r0);
     if (!parts) split_rows_bf16(X + r0 * D, m, D, hi, lo, s);
-    AssignPolicy p;
-    p.n = m;
-    p.K = K;
-    p.nch = nch;
-    p.nkb = (int)cdiv(D, tc::kTK);
-    p.half_sq = ix.cb_half_sq;
-    p.cval = cval;
-    p.cidx = cidx;
     const CUtensorMap tA = make_tmap_bf16(hi, rows_alloc, D, tc::kTM);
     const CUtensorMap tA2 = make_tmap_bf16(lo, rows_alloc, D, tc::kTM);
     const int grid = (int)std::min<int64_t>(sms, cdiv(m, tc::kTM) * nch);
+    auto coarse = [&](auto p) {
+      p.n = m;
+      p.K = K;
+      p.nch = nch;
+      p.nkb = (int)cdiv(D, tc::kTK);
+      p.half_sq = ix.cb_half_sq;
+      p.cval = cval;
+      p.cidx = cidx;
+      tc::launch_engine(tA, tB, tA2, tB2, p, ix.d_err, grid, s);
+    };
     if (kc) kc->begin(0);
-    tc::launch_engine(tA, tB, tA2, tB2, p, ix.d_err, grid, s);
+    if (tn == 256) coarse(AssignPolicy<256>{});
+    else if (tn == 64) coarse(AssignPolicy<64>{});
+    else coarse(AssignPolicy<32>{});
     if (kc) {
       kc->end(0);
       kc->assign_rows += m;
     }
-    k_assign_refine<<<(unsigned)cdiv(m, 8), 256, 0, s>>>(X + r0 * D, m, D, ix.codebook, K, ma, cval, cidx, nch,
-                                                          x_inv + r0, ix.cb_max_norm, cb_max, codes + r0 * ma);
+    if (m >= 8 * sms)
+      k_assign_refine<1><<<(unsigned)cdiv(m, 8), 256, 0, s>>>(X + r0 * D, m, D, ix.codebook, K, ma, cval, cidx, nch,
+                                                              tn, kT, x_inv + r0, ix.cb_max_norm, cb_max, codes + r0 * ma);
+    else
+      k_assign_refine<8><<<(unsigned)m, 256, 0, s>>>(X + r0 * D, m, D, ix.codebook, K, ma, cval, cidx, nch, tn, kT,
+                                                     x_inv + r0, ix.cb_max_norm, cb_max, codes + r0 * ma);
     GIFT_LAUNCHED("k_assign_refine");
   }
 }
