@@ -290,8 +290,13 @@ __global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
   }
   __syncthreads();
   if (!a.act_ids)
-    for (int c = t; c < a.k1; c += T)
-      if (cid[c] >= 0 && cid[c] < a.N) atomicAdd(&s_norm, (unsigned long long)member_fix(csc[c]));
+    for (int base = t - (t & 31); base < a.k1; base += T) {  // a warp's sum, then one 64-bit atomic
+      const int c = base + (t & 31);
+      unsigned long long f = c < a.k1 && cid[c] >= 0 && cid[c] < a.N ? member_fix(csc[c]) : 0u;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+      if ((t & 31) == 0) atomicAdd(&s_norm, f);
+    }
   const int need = min(a.topk, a.N);
   int take = 0;
 
@@ -593,6 +598,7 @@ __global__ __launch_bounds__(kAcaT) void k_aca_rows(const AcaRowArgs a) {
   }
   __syncthreads();
   int o = part[tid];
+  unsigned long long sum = 0ull;
   const float div = a.mode == 0 ? 1.f : (float)a.k2;
   for (int t = c0; t < c0 + per; ++t) {
     if (!pos[t]) continue;
@@ -605,9 +611,12 @@ __global__ __launch_bounds__(kAcaT) void k_aca_rows(const AcaRowArgs a) {
     const uint32_t m = member_fix(gen_mean(s0 / div, s1 / div, a.alpha));
     a.out_ids[r * a.cap + o] = (int32_t)id;
     a.out_mem[r * a.cap + o] = m;
-    atomicAdd(&norm, (unsigned long long)m);
+    sum += m;
     ++o;
   }
+#pragma unroll
+  for (int k = 16; k > 0; k >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, k);
+  if ((tid & 31) == 0) atomicAdd(&norm, sum);  // (64-bit atomics in shared memory are loops: one per warp)
   __syncthreads();
   if (tid == 0) a.out_norm[r] = norm;
 }
