@@ -13,7 +13,7 @@
 // rows, folding runs of equal shape instead of N_v-column groups.
 #include "gift_internal.cuh"
 #include "segmax.cuh"
-#include "tc_engine.cuh"
+#include "tc_pair.cuh"
 
 namespace gift {
 
@@ -65,6 +65,22 @@ struct ExactPolicy {
     kb1 = (int)((int64_t)nkb * (c + 1) / nch);
   }
   __device__ __forceinline__ int a_row(const Item& it) const { return (int)it.r0; }
+  // pair form: 256 x 256 tiles, a CTA's epilogue part takes 128 x 128 of them
+  static constexpr int TN_PAIR = 256;
+  __device__ __forceinline__ int64_t total_pair() const { return cdiv(rows, (int64_t)256) * cdiv(ncols, (int64_t)256); }
+  __device__ __forceinline__ Item decode_pair(int64_t item) const {
+    const int64_t nt = cdiv(rows, (int64_t)256), ct = item / nt, rt = item % nt;
+    Item it;
+    it.r0 = rt * 256;
+    it.c0 = ct * 256;
+    it.nr = (int)min((int64_t)256, rows - it.r0);
+    it.nc = (int)min((int64_t)256, ncols - it.c0);
+    return it;
+  }
+  __device__ __forceinline__ Item sub(const Item& w, int rank, int part) const {
+    return Item{w.r0 + 128 * rank, w.c0 + 128 * part, min(128, max(0, w.nr - 128 * rank)),
+                min(128, max(0, w.nc - 128 * part))};
+  }
   __device__ __forceinline__ void epi_begin(const Item& it, Ctx& x, int, int, uint8_t* ws) const {
     float* ri = reinterpret_cast<float*>(ws);
     const int lane = threadIdx.x & 31;
@@ -154,6 +170,22 @@ struct ShortSegPolicy {
     kb1 = nkb;
   }
   __device__ __forceinline__ int a_row(const Item& it) const { return (int)it.r0; }
+  // pair form: 256 x 256 tiles, a CTA's epilogue part takes 128 x 128 of them
+  static constexpr int TN_PAIR = 256;
+  __device__ __forceinline__ int64_t total_pair() const { return cdiv(rows, (int64_t)256) * cdiv(ncols, (int64_t)256); }
+  __device__ __forceinline__ Item decode_pair(int64_t item) const {
+    const int64_t nt = cdiv(rows, (int64_t)256), ct = item / nt, rt = item % nt;
+    Item it;
+    it.r0 = rt * 256;
+    it.c0 = ct * 256;
+    it.nr = (int)min((int64_t)256, rows - it.r0);
+    it.nc = (int)min((int64_t)256, ncols - it.c0);
+    return it;
+  }
+  __device__ __forceinline__ Item sub(const Item& w, int rank, int part) const {
+    return Item{w.r0 + 128 * rank, w.c0 + 128 * part, min(128, max(0, w.nr - 128 * rank)),
+                min(128, max(0, w.nc - 128 * part))};
+  }
   __device__ __forceinline__ void epi_begin(const Item& it, Ctx& x, int m, int, uint8_t* ws) const {
     float* ri = reinterpret_cast<float*>(ws);
     const int lane = threadIdx.x & 31;
@@ -234,6 +266,22 @@ struct ExactListPolicy {
     kb1 = (int)((int64_t)nkb * (c + 1) / nch);
   }
   __device__ __forceinline__ int a_row(const Item& it) const { return (int)it.r0; }
+  // pair form: 256 x 256 tiles, a CTA's epilogue part takes 128 x 128 of them
+  static constexpr int TN_PAIR = 256;
+  __device__ __forceinline__ int64_t total_pair() const { return cdiv(rows, (int64_t)256) * cdiv(ncols, (int64_t)256); }
+  __device__ __forceinline__ Item decode_pair(int64_t item) const {
+    const int64_t nt = cdiv(rows, (int64_t)256), ct = item / nt, rt = item % nt;
+    Item it;
+    it.r0 = rt * 256;
+    it.c0 = ct * 256;
+    it.nr = (int)min((int64_t)256, rows - it.r0);
+    it.nc = (int)min((int64_t)256, ncols - it.c0);
+    return it;
+  }
+  __device__ __forceinline__ Item sub(const Item& w, int rank, int part) const {
+    return Item{w.r0 + 128 * rank, w.c0 + 128 * part, min(128, max(0, w.nr - 128 * rank)),
+                min(128, max(0, w.nc - 128 * part))};
+  }
   __device__ __forceinline__ void epi_begin(const Item& it, Ctx& x, int, int, uint8_t* ws) const {
     float* sc = reinterpret_cast<float*>(ws);
     int32_t* sh = reinterpret_cast<int32_t*>(ws + TN * 4);
@@ -281,6 +329,19 @@ struct ExactListPolicy {
   }
 };
 
+// on pairs of SMs or single ones, whichever takes fewer rounds of their time (both tilings use boxes of 128 rows)
+template <class P>
+void run_tiles(const CUtensorMap& tA, const CUtensorMap& tB, const CUtensorMap& tA2, const CUtensorMap& tB2, const P& p,
+               int* err, cudaStream_t s) {
+  const int sms = device_sm_count();
+  const int64_t items = p.n_rt * cdiv(p.ncols, (int64_t)128);
+  const int64_t pair_items = cdiv(p.rows, (int64_t)256) * cdiv(p.ncols, (int64_t)256);
+  if (tc::pair_wins(items, pair_items, sms, tc::pair_clusters<P>()))
+    tc::launch_pair(tA, tB, tA2, tB2, p, err, pair_items, s);
+  else
+    tc::launch_engine(tA, tB, tA2, tB2, p, err, (int)std::min<int64_t>(sms, items), s);
+}
+
 }  // namespace
 
 void segmax_tc(const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int64_t a_rows_alloc, const float* a_inv,
@@ -293,7 +354,6 @@ void segmax_tc(const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int64_t a_r
   int64_t cell_rows = 0;
   const CUtensorMap tB = make_tmap_bf16(b_hi, b_rows_alloc, D, ExactPolicy::TN);
   const CUtensorMap tB2 = make_tmap_bf16(b_lo, b_rows_alloc, D, ExactPolicy::TN);
-  const int sms = device_sm_count();
   int32_t b0 = 0;
   while (b0 < B) {
     int32_t b1 = b0 + 1;
@@ -317,8 +377,7 @@ void segmax_tc(const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int64_t a_r
       p.q_inv = a_inv + v0;
       p.r_inv = b_inv;
       p.cell = cell;
-      const int grid = (int)std::min<int64_t>(sms, p.n_rt * cdiv(ncols, ShortSegPolicy::TN));
-      tc::launch_engine(tA, tB, tA2, tB2, p, err, grid, s);
+      run_tiles(tA, tB, tA2, tB2, p, err, s);
       segmax_reduce(cell, N, d_qoff, b0, b1 - b0, (int32_t)v0, S, argmax, s);
       b0 = b1;
       continue;
@@ -333,8 +392,7 @@ void segmax_tc(const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int64_t a_r
     p.q_inv = a_inv + v0;
     p.r_inv = b_inv;
     p.cell = cell;
-    const int grid = (int)std::min<int64_t>(sms, p.n_rt * cdiv(ncols, ExactPolicy::TN));
-    tc::launch_engine(tA, tB, tA2, tB2, p, err, grid, s);
+    run_tiles(tA, tB, tA2, tB2, p, err, s);
     segmax_reduce(cell, N, d_qoff, b0, b1 - b0, (int32_t)v0, S, argmax, s);
     b0 = b1;
   }
@@ -372,7 +430,6 @@ void exact_scores_lists(const Index& ix, const float* q, const float* q_inv, int
   const int64_t cap = std::max<int64_t>(1, ((int64_t)1 << 28) / N);  // cell block <= 2 GiB
   unsigned long long* cell = nullptr;
   int64_t cell_rows = 0;
-  const int sms = device_sm_count();
   int32_t b0 = 0;
   while (b0 < B) {
     int32_t b1 = b0 + 1;
@@ -395,8 +452,7 @@ void exact_scores_lists(const Index& ix, const float* q, const float* q_inv, int
     p.cell = cell;
     const CUtensorMap tA = make_tmap_bf16(hi + v0 * D, qrows - v0, D, tc::kTM);
     const CUtensorMap tA2 = make_tmap_bf16(lo + v0 * D, qrows - v0, D, tc::kTM);
-    const int grid = (int)std::min<int64_t>(sms, p.n_rt * cdiv(ncols, ExactListPolicy::TN));
-    tc::launch_engine(tA, tB, tA2, tB2, p, ix.d_err, grid, s);
+    run_tiles(tA, tB, tA2, tB2, p, ix.d_err, s);
     segmax_reduce(cell, N, d_qoff, b0, b1 - b0, (int32_t)v0, S, nullptr, s);
     b0 = b1;
   }

@@ -16,8 +16,12 @@ void run_gemm(const CUtensorMap& tA, const CUtensorMap& tB, const CUtensorMap& t
   p.ldc = ldc;
   p.accumulate = accumulate;
   p.row_major = cdiv(M, tc::kTM) >= cdiv(N, 128);
-  const int grid = (int)std::min<int64_t>(device_sm_count(), cdiv(M, tc::kTM) * cdiv(N, 128));
-  tc::launch_engine(tA, tB, tA2, tB2, p, err, grid, s);
+  const int sms = device_sm_count();
+  const int64_t items = cdiv(M, tc::kTM) * cdiv(N, 128), pair_items = cdiv(M, 256) * cdiv(N, 256);
+  if (tc::pair_wins(items, pair_items, sms, tc::pair_clusters<GemmPolicy<SPLIT>>()))
+    tc::launch_pair(tA, tB, tA2, tB2, p, err, pair_items, s);
+  else
+    tc::launch_engine(tA, tB, tA2, tB2, p, err, (int)std::min<int64_t>(sms, items), s);
 }
 
 }  // namespace

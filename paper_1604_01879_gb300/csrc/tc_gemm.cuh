@@ -9,7 +9,7 @@
 // each A tile (read from memory once) and all of B; otherwise column-tile-
 // major, sharing the B tile.
 #pragma once
-#include "tc_engine.cuh"
+#include "tc_pair.cuh"
 
 namespace gift {
 
@@ -57,6 +57,18 @@ struct GemmPolicy {
     kb1 = (int)((int64_t)nkb * (c + 1) / nch);
   }
   __device__ __forceinline__ int a_row(const Item& it) const { return (int)it.r0; }
+  // pair form: 256 x 256 tiles in the same order, a CTA's epilogue part takes 128 x 128 of them
+  static constexpr int TN_PAIR = 256;
+  __device__ __forceinline__ int64_t total_pair() const { return cdiv(M, (int64_t)256) * cdiv(N, (int64_t)256); }
+  __device__ __forceinline__ Item decode_pair(int64_t item) const {
+    const int64_t mt = cdiv(M, (int64_t)256), nt = cdiv(N, (int64_t)256);
+    const int64_t ct = row_major ? item % nt : item / mt, rt = row_major ? item / nt : item % mt;
+    return Item{rt * 256, ct * 256, (int)min((int64_t)256, M - rt * 256), (int)min((int64_t)256, N - ct * 256)};
+  }
+  __device__ __forceinline__ Item sub(const Item& w, int rank, int part) const {
+    return Item{w.r0 + 128 * rank, w.c0 + 128 * part, min(128, max(0, w.nr - 128 * rank)),
+                min(128, max(0, w.nc - 128 * part))};
+  }
   __device__ __forceinline__ void epi_begin(const Item&, Ctx& x, int, int, uint8_t*) const {
 #pragma unroll
     for (int j = 0; j < TN; ++j) x.sum[j] = 0.f;
