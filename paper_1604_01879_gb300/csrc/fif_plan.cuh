@@ -39,6 +39,8 @@ struct FifPlan {
 constexpr int kMaxSpecs = 6;
 struct WorkSpecs {
   int n = 0;
+  int sms = 0, pairs = 0;  // > 0: specs 0 and 1 are the same work one SM or one pair of SMs per item, and the slower
+                           // one's offsets are all zero (tc::pair_wins, decided where the item counts are)
   int cls[kMaxSpecs], tn[kMaxSpecs], ts[kMaxSpecs];
   void add(int c, int n_, int s) {
     cls[n] = c;

@@ -24,6 +24,7 @@
 #include "gift_internal.cuh"
 #include "fif_plan.cuh"
 #include "select.cuh"
+#include "tc_common.cuh"
 
 namespace gift {
 
@@ -95,6 +96,7 @@ __global__ __launch_bounds__(kPlanT) void k_plan_work(const int64_t* __restrict_
   __shared__ int64_t wsum[kPlanT / 32 + 1];
   __shared__ unsigned s_items;
   __shared__ int s_most;
+  __shared__ unsigned s_both[2];
   const int tid = threadIdx.x, c = blockIdx.x;
   const int cls = specs.cls[c], tn = specs.tn[c], ts = specs.ts[c];
   int64_t* out = woff + (int64_t)c * (K + 1);
@@ -124,6 +126,26 @@ __global__ __launch_bounds__(kPlanT) void k_plan_work(const int64_t* __restrict_
     __syncthreads();
     if ((int64_t)s_items <= fold) folded = slot_class(s_most);
   }
+  bool drop = false;
+  if (specs.pairs > 0) {  // items of both tilings, then the slower one has none
+    if (tid < 2) s_both[tid] = 0u;
+    __syncthreads();
+    unsigned n0 = 0, n1 = 0;
+#pragma unroll 4
+    for (int k = tid; k < K; k += kPlanT) {
+      const uint32_t M = (uint32_t)(boff[k + 1] - boff[k]), L = (uint32_t)(list_off[k + 1] - list_off[k]);
+      n0 += ((L + specs.tn[0] - 1) / specs.tn[0]) * ((M + specs.ts[0] - 1) / specs.ts[0]);
+      n1 += ((L + specs.tn[1] - 1) / specs.tn[1]) * ((M + specs.ts[1] - 1) / specs.ts[1]);
+    }
+    n0 = __reduce_add_sync(0xffffffffu, n0);
+    n1 = __reduce_add_sync(0xffffffffu, n1);
+    if ((tid & 31) == 0) {
+      atomicAdd(&s_both[0], n0);
+      atomicAdd(&s_both[1], n1);
+    }
+    __syncthreads();
+    drop = (c == 1) != tc::pair_wins(s_both[0], s_both[1], specs.sms, specs.pairs);
+  }
   int64_t run = 0;
   for (int k0 = 0; k0 <= K; k0 += 4 * kPlanT) {
     int64_t n[4];  // four chunks' reads go out together
@@ -135,7 +157,7 @@ __global__ __launch_bounds__(kPlanT) void k_plan_work(const int64_t* __restrict_
       const int64_t M = boff[k + 1] - boff[k], L = list_off[k + 1] - list_off[k];
       const int mine = M <= 80 && folded ? folded : slot_class(M);
       // (entries and slots number fewer than 2^31: 32-bit divisions)
-      if (M > 0 && L > 0 && (cls <= 0 || mine == cls))
+      if (!drop && M > 0 && L > 0 && (cls <= 0 || mine == cls))
         n[i] = (int64_t)(((uint32_t)L + tn - 1) / (uint32_t)tn) * (((uint32_t)M + ts - 1) / (uint32_t)ts);
     }
 #pragma unroll
