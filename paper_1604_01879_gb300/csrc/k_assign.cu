@@ -19,7 +19,7 @@
 // (distance, index) are the codes. Results equal an exact evaluation except
 // where distances tie to ~1e-13.
 #include "gift_internal.cuh"
-#include "tc_engine.cuh"
+#include "tc_pair.cuh"
 
 namespace gift {
 
@@ -37,7 +37,7 @@ __host__ __device__ constexpr int kept_scores(int tn) { return tn == 32 ? 32 : 1
 template <int TN_>
 struct AssignPolicy {
   static constexpr int TN = TN_, NBUF = 2, SPLIT = 3, EB = 2;
-  static constexpr int STAGES = TN_ == 256 ? 2 : TN_ == 64 ? 4 : 5;
+  static constexpr int STAGES = TN_ == 256 ? 2 : TN_ == 128 ? 3 : TN_ == 64 ? 4 : 5;
   static constexpr int kT = kept_scores(TN_);
   static constexpr bool kAll = kT == TN_;
   static constexpr int kWarpSmem = TN * 4;
@@ -135,6 +135,26 @@ struct AssignPolicy {
       cval[o + t] = x.val[t];
       cidx[o + t] = x.idx[t];
     }
+  }
+};
+
+// The same on pairs of SMs: 256 rows x 256 codewords per item, each epilogue part keeping the best scores of its
+// 128 codewords as a chunk of its own (16,384 rows, D = 4096, K = 4,096: 972 us one SM per item, 825 in pairs; tiles of
+// 128 columns, which fill a last round better, load as many bytes per product as one SM's and were no faster).
+struct PairAssignPolicy : AssignPolicy<128> {
+  static constexpr int TN_PAIR = 256;
+  __device__ __forceinline__ int64_t total_pair() const { return cdiv(this->n, (int64_t)256) * ((this->nch + 1) / 2); }
+  __device__ __forceinline__ Item decode_pair(int64_t item) const {
+    const int cols = (this->nch + 1) / 2;
+    Item it;
+    it.r0 = item / cols * 256;
+    it.c = 2 * (int)(item % cols);
+    it.nr = (int)min((int64_t)256, this->n - it.r0);
+    return it;
+  }
+  __device__ __forceinline__ Item sub(const Item& w, int rank, int part) const {
+    const bool in = w.c + part < this->nch;  // (no last half chunk: no rows to write)
+    return Item{w.r0 + 128 * rank, in ? min(128, max(0, w.nr - 128 * rank)) : 0, w.c + part};
   }
 };
 
@@ -502,7 +522,14 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
   // codewords per item: as many as leave an item for every SM (one pass over the rows)
   const int64_t row_tiles = cdiv(chunk, (int64_t)tc::kTM);
   // (a vocabulary of more than 1,024 keeps 64: the refine reads kT scores per chunk and row)
-  const int tn = row_tiles * cdiv(K, 256) >= sms ? 256 : K > 1024 || row_tiles * cdiv(K, 64) >= sms ? 64 : 32;
+  int tn = row_tiles * cdiv(K, 256) >= sms ? 256 : K > 1024 || row_tiles * cdiv(K, 64) >= sms ? 64 : 32;
+  // full SMs: pairs of them, where their rounds, each 0.85 of the others' time (measured), take less
+  bool pair = false;
+  if (tn == 256) {
+    const int64_t items = cdiv(chunk, (int64_t)256) * cdiv(K, 256);
+    pair = 0.85 * cdiv(items, (int64_t)tc::pair_clusters<PairAssignPolicy>()) < cdiv(row_tiles * cdiv(K, 256), (int64_t)sms);
+    if (pair) tn = 128;  // chunks of kept scores
+  }
   const int nch = (int)cdiv(K, tn), kT = kept_scores(tn);
   float* cval = sc.get<float>((size_t)chunk * nch * kT);
   int32_t* cidx = sc.get<int32_t>((size_t)chunk * nch * kT);
@@ -520,7 +547,7 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
     const CUtensorMap tA = make_tmap_bf16(hi, rows_alloc, D, tc::kTM);
     const CUtensorMap tA2 = make_tmap_bf16(lo, rows_alloc, D, tc::kTM);
     const int grid = (int)std::min<int64_t>(sms, cdiv(m, tc::kTM) * nch);
-    auto coarse = [&](auto p) {
+    auto coarse = [&](auto p, auto launch) {
       p.n = m;
       p.K = K;
       p.nch = nch;
@@ -528,12 +555,17 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
       p.half_sq = ix.cb_half_sq;
       p.cval = cval;
       p.cidx = cidx;
-      tc::launch_engine(tA, tB, tA2, tB2, p, ix.d_err, grid, s);
+      launch(p);
+    };
+    auto single = [&](const auto& p) { tc::launch_engine(tA, tB, tA2, tB2, p, ix.d_err, grid, s); };
+    auto paired = [&](const auto& p) {  // (B boxes of half the pair's columns: tn)
+      tc::launch_pair(tA, tB, tA2, tB2, p, ix.d_err, cdiv(m, (int64_t)256) * cdiv(nch, 2), s);
     };
     if (kc) kc->begin(0);
-    if (tn == 256) coarse(AssignPolicy<256>{});
-    else if (tn == 64) coarse(AssignPolicy<64>{});
-    else coarse(AssignPolicy<32>{});
+    if (pair) coarse(PairAssignPolicy{}, paired);
+    else if (tn == 256) coarse(AssignPolicy<256>{}, single);
+    else if (tn == 64) coarse(AssignPolicy<64>{}, single);
+    else coarse(AssignPolicy<32>{}, single);
     if (kc) {
       kc->end(0);
       kc->assign_rows += m;

@@ -2,10 +2,10 @@
 // 256-row tile with tcgen05.mma.cta_group::2.
 //
 // Each CTA stages 128 rows of A and half of the tile's B rows, and the pair's tensor
-// cores read both halves of B; each CTA's TMEM receives its 128 rows x TN columns. Per
-// product a CTA's shared memory is read half as often as by the one-SM engine's
-// 128 x 128 tiles, whose reads (128 bytes per clock) are as many as shared memory gives, and
-// a stage of the same 64 KB feeds twice the products, so L2 is read half as often too.
+// cores read both halves of B; each CTA's TMEM receives its 128 rows x 256 columns. A
+// stage of the same 64 KB feeds twice the products of the one-SM engine's 128 x 128
+// tiles, which ask L2 for 85 bytes per clock and SM and their shared memory for 128 at
+// the tensor cores' full rate: what L2 delivers to an SM bounded them.
 //
 //   warp 0        TMA producer (one thread of each CTA): its own stage, signalled on the
 //                 leader's (rank 0) full barrier, which counts both CTAs' bytes
@@ -116,7 +116,7 @@ template <class P>
 struct PairLayout {
   static_assert(P::EB == 2, "BF16 operands");
   static constexpr int TN = P::TN_PAIR;
-  static_assert(TN == 128 || TN == 256, "columns of the pair's tile");
+  static_assert(TN == 256, "columns of the pair's tile");
   static constexpr int kABytes = kTM * 128;
   static constexpr int kBBytes = TN / 2 * 128;
   static constexpr int kPartsA = P::SPLIT == 1 ? 1 : 2;

@@ -40,3 +40,17 @@ def test_exact_scores_do_not_depend_on_the_batch(gpu_lib, storage, keep):
         lo, hi = int(off[b]), int(off[b + 1])
         i1, s1 = ix.query(q[lo:hi].contiguous(), off[b:b + 2] - off[b], mode="exact", topk=40)
         assert torch.equal(ids[b], i1[0]) and torch.equal(sc[b], s1[0])
+
+
+@pytest.mark.parametrize("K,ma", [(300, 1), (640, 2), (1000, 3), (1100, 2), (2100, 1)])
+def test_codes_do_not_depend_on_the_batch(gpu_lib, K, ma):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(K)
+    n, D = 20011, 64
+    cb = torch.randn((K, D), generator=g, device="cuda")
+    x = (cb[torch.randint(0, K, (n,), generator=g, device="cuda")]
+         + torch.randn((n, D), generator=g, device="cuda")).contiguous()
+    ix = gpu_lib.Index(x[:1].contiguous(), cb, 1, 1, K, keep_exact=False)
+    codes = ix.assign(x, ma)
+    for lo in (0, 9999, n - 300):
+        assert torch.equal(codes[lo:lo + 300], ix.assign(x[lo:lo + 300].contiguous(), ma))
