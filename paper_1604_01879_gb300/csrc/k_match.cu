@@ -531,7 +531,7 @@ __global__ __launch_bounds__(kCsrT) void k_onehot_csr(const int16_t* __restrict_
 // H[r] = sum of wV[e] U[e mod ld] over the entries e of row r (perm[beg[r]] ..
 // perm[beg[r] + cnt[r]]), in ascending e: one warp per database view, lane c owns columns
 // 4 c + 128 t, up to kHCols columns per pass (dout % 4 == 0)
-constexpr int kHCols = 512;
+template <int kHCols, int kAhead>
 __global__ __launch_bounds__(256) void k_segment_rows_sum(const float* __restrict__ U, const int32_t* __restrict__ perm,
                                                           const int64_t* __restrict__ beg,
                                                           const int32_t* __restrict__ cnt,
@@ -557,7 +557,7 @@ __global__ __launch_bounds__(256) void k_segment_rows_sum(const float* __restric
         src = (int64_t)(e % ld) * dout;
         wl = wT[e];
       }
-#pragma unroll 4
+#pragma unroll(kAhead)
       for (int k = 0; k < n; ++k) {  // unrolled: several entries' row loads in flight
         const int64_t sk = __shfl_sync(0xffffffffu, src, k);
         const float wk = __shfl_sync(0xffffffffu, wl, k);
@@ -766,10 +766,12 @@ void match_backward(const void* q, const std::vector<int32_t>& h_qoff, int32_t B
     // parts of the step range: a block's time is ~ steps / parts, the launch takes
     // ceil(blocks x parts / SMs) rounds of one block per SM; partial rows cost a little
     const int64_t units = cdiv(nq, (int64_t)kGRows) * cdiv((int64_t)dout, (int64_t)kGCols);
+    // (in microseconds: 1.1 a step, and a part's row written and read twice at 4 TB/s, or its reads' latency)
     int parts = 1;
     double best = 1e30;
-    for (int pc = 1; pc <= 8 && pc <= st.n; ++pc) {
-      const double cost = (double)cdiv(units * pc, (int64_t)sms) / pc + 0.02 * pc;
+    const double part_us = std::max(1.0, (double)nq * dout * 12 / 4e6);
+    for (int pc = 1; pc <= 64 && pc <= st.n; ++pc) {
+      const double cost = 1.1 * (double)cdiv(units * pc, (int64_t)sms) * st.n / pc + part_us * pc;
       if (cost < best - 1e-9) {
         best = cost;
         parts = pc;
@@ -797,7 +799,11 @@ void match_backward(const void* q, const std::vector<int32_t>& h_qoff, int32_t B
       GIFT_CUDA(cudaFuncSetAttribute(k_onehot_csr, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       k_onehot_csr<<<(unsigned)Np, kCsrT, smem, s>>>(amT, nq, ldq, nv, perm, beg, cnt);
       GIFT_LAUNCHED("k_onehot_csr");
-      k_segment_rows_sum<<<(unsigned)cdiv(nr, (int64_t)8), 256, 0, s>>>(U16, perm, beg, cnt, wV, ldq, nr, dout, H);
+      // (a view that many query views prefer is one warp's chain of reads: narrow rows keep more of them in flight)
+      if (dout <= 128)
+        k_segment_rows_sum<128, 16><<<(unsigned)cdiv(nr, (int64_t)8), 256, 0, s>>>(U16, perm, beg, cnt, wV, ldq, nr, dout, H);
+      else
+        k_segment_rows_sum<512, 4><<<(unsigned)cdiv(nr, (int64_t)8), 256, 0, s>>>(U16, perm, beg, cnt, wV, ldq, nr, dout, H);
       GIFT_LAUNCHED("k_segment_rows_sum");
     } else {  // larger shapes: the staged gather
       const size_t smem = (size_t)kHStages * kHStageBytes;
@@ -815,11 +821,11 @@ void match_backward(const void* q, const std::vector<int32_t>& h_qoff, int32_t B
     const Operand dUt = make_transposed(dU, GIFT_F32, nq, dout, ldq, sc, s);
     const Operand Qt = make_transposed(q, dtype, nq, din, ldq, sc, s);
     gemm_tc(dUt.hi, dUt.lo, dout, dUt.rows_alloc, ldq, Qt.hi, Qt.lo, din, Qt.rows_alloc, ldq, (int)ldq, dW, din, 0,
-            err, s);
+            err, s, &sc);
     const Operand dVt = make_transposed(dV, GIFT_F32, nr, dout, ldr, sc, s);
     const Operand Pt = make_transposed(p, dtype, nr, din, ldr, sc, s);
     gemm_tc(dVt.hi, dVt.lo, dout, dVt.rows_alloc, ldr, Pt.hi, Pt.lo, din, Pt.rows_alloc, ldr, (int)ldr, dW, din, 1,
-            err, s);
+            err, s, &sc);
   }
   if (dQ || dP) {
     int64_t ldo = 0;

@@ -24,18 +24,25 @@ struct GemmPolicy {
   int64_t ldc;
   int accumulate;
   bool row_major;  // item order: row tile slow (true) or column tile slow
+  // parts > 1: the reduction is cut in so many parts, items of a part together, each with its own result at
+  // C + part * pstride (added up in part order by k_add_parts)
+  int parts = 1;
+  int64_t pstride = 0;
   struct Item {
     int64_t r0, c0;
     int nr, nc;
+    int part;
   };
   struct Ctx {
     float sum[TN];
   };
   __device__ __forceinline__ int64_t n_mt() const { return cdiv(M, tc::kTM); }
-  __device__ __forceinline__ int64_t total() const { return n_mt() * cdiv(N, TN); }
+  __device__ __forceinline__ int64_t total() const { return n_mt() * cdiv(N, TN) * parts; }
   __device__ __forceinline__ Item decode(int64_t item) const {
     Item it;
     const int64_t mt = n_mt(), nt = cdiv(N, TN);
+    it.part = (int)(item / (mt * nt));
+    item -= it.part * (mt * nt);
     const int64_t ct = row_major ? item % nt : item / mt, rt = row_major ? item / nt : item % mt;
     it.r0 = rt * tc::kTM;
     it.c0 = ct * TN;
@@ -46,29 +53,33 @@ struct GemmPolicy {
   // chunks bound the MMA steps feeding one accumulator (about 192, 3 products
   // x 4 sub-steps per k-block), however long the reduction (the weight
   // gradient reduces over every database view); short reductions use one chunk
-  __device__ __forceinline__ int nch() const {
-    const int want = (nkb * 12 + 191) / 192;
+  __device__ __forceinline__ int part_kb(int part) const { return (int)((int64_t)nkb * part / parts); }
+  __device__ __forceinline__ int nchunks(const Item& it) const {
+    const int want = ((part_kb(it.part + 1) - part_kb(it.part)) * 12 + 191) / 192;
     return want < 1 ? 1 : want;
   }
-  __device__ __forceinline__ int nchunks(const Item&) const { return nch(); }
   __device__ __forceinline__ void chunk(const Item& it, int c, int& br, int& kb0, int& kb1) const {
-    const int nch = this->nch();
+    const int n = nchunks(it), p0 = part_kb(it.part), len = part_kb(it.part + 1) - p0;
     br = (int)it.c0;
-    kb0 = (int)((int64_t)nkb * c / nch);
-    kb1 = (int)((int64_t)nkb * (c + 1) / nch);
+    kb0 = p0 + (int)((int64_t)len * c / n);
+    kb1 = p0 + (int)((int64_t)len * (c + 1) / n);
   }
   __device__ __forceinline__ int a_row(const Item& it) const { return (int)it.r0; }
   // pair form: 256 x 256 tiles in the same order, a CTA's epilogue part takes 128 x 128 of them
   static constexpr int TN_PAIR = 256;
-  __device__ __forceinline__ int64_t total_pair() const { return cdiv(M, (int64_t)256) * cdiv(N, (int64_t)256); }
+  __device__ __forceinline__ int64_t total_pair() const {
+    return cdiv(M, (int64_t)256) * cdiv(N, (int64_t)256) * parts;
+  }
   __device__ __forceinline__ Item decode_pair(int64_t item) const {
     const int64_t mt = cdiv(M, (int64_t)256), nt = cdiv(N, (int64_t)256);
+    const int part = (int)(item / (mt * nt));
+    item -= part * (mt * nt);
     const int64_t ct = row_major ? item % nt : item / mt, rt = row_major ? item / nt : item % mt;
-    return Item{rt * 256, ct * 256, (int)min((int64_t)256, M - rt * 256), (int)min((int64_t)256, N - ct * 256)};
+    return Item{rt * 256, ct * 256, (int)min((int64_t)256, M - rt * 256), (int)min((int64_t)256, N - ct * 256), part};
   }
   __device__ __forceinline__ Item sub(const Item& w, int rank, int part) const {
     return Item{w.r0 + 128 * rank, w.c0 + 128 * part, min(128, max(0, w.nr - 128 * rank)),
-                min(128, max(0, w.nc - 128 * part))};
+                min(128, max(0, w.nc - 128 * part)), w.part};
   }
   __device__ __forceinline__ void epi_begin(const Item&, Ctx& x, int, int, uint8_t*) const {
 #pragma unroll
@@ -90,7 +101,8 @@ struct GemmPolicy {
   __device__ __forceinline__ void epi_end(const Item& it, Ctx& x, int m, uint8_t* ws) const {
     float* t = reinterpret_cast<float*>(ws);  // [32][kTurn]
     const int lane = threadIdx.x & 31, m0 = m - lane;
-    const bool vec = (ldc % 4) == 0 && ((it.c0 % 4) == 0) && (reinterpret_cast<uintptr_t>(C) % 16) == 0;
+    float* out = C + it.part * pstride;
+    const bool vec = (ldc % 4) == 0 && ((it.c0 % 4) == 0) && (reinterpret_cast<uintptr_t>(out) % 16) == 0;
 #pragma unroll
     for (int pc = 0; pc < TN / 16; ++pc) {
       if (pc * 16 >= it.nc) break;  // warp-uniform
@@ -106,7 +118,7 @@ struct GemmPolicy {
         const int r = i * 8 + (lane >> 2);
         if (m0 + r >= it.nr || c >= it.nc) continue;
         float4 v = *reinterpret_cast<const float4*>(t + r * kTurn + q);
-        float* dst = C + (it.r0 + m0 + r) * ldc + it.c0 + c;
+        float* dst = out + (it.r0 + m0 + r) * ldc + it.c0 + c;
         if (vec && c + 4 <= it.nc) {
           if (accumulate) {
             const float4 o = *reinterpret_cast<const float4*>(dst);
@@ -128,9 +140,10 @@ struct GemmPolicy {
 // Two-part (SPLIT 3), two-part A with one-part B (SPLIT 2, b_lo null) or
 // one-part (SPLIT 1, both lo parts null) BF16 operands; a_rows_alloc /
 // b_rows_alloc are the rows the tensor maps cover (rows past M or N read as
-// zeros); lda / ldb are row pitches in elements (0 = K): C[M, N] (+)= A * B^T.
+// zeros); lda / ldb are row pitches in elements (0 = K): C[M, N] (+)= A * B^T. With `split` the
+// reduction may be cut in parts where the tiles alone would leave SMs idle (another order of sums).
 void gemm_tc(const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int64_t M, int64_t a_rows_alloc, int64_t lda,
              const __nv_bfloat16* b_hi, const __nv_bfloat16* b_lo, int64_t N, int64_t b_rows_alloc, int64_t ldb, int K,
-             float* C, int64_t ldc, int accumulate, int* err, cudaStream_t s);
+             float* C, int64_t ldc, int accumulate, int* err, cudaStream_t s, Scratch* split = nullptr);
 
 }  // namespace gift
