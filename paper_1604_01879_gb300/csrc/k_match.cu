@@ -47,16 +47,32 @@ __global__ void k_split_any(const T* __restrict__ in, int64_t n, __nv_bfloat16* 
   if (lo) lo[i] = __float2bfloat16_rn(v - __bfloat162float(h));
 }
 
-// the same for FP32 input, four elements per thread (n % 4 == 0, 16-byte aligned input, 8-byte aligned output)
-__global__ void k_split4(const float4* __restrict__ in, int64_t n4, uint2* __restrict__ hi, uint2* __restrict__ lo) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-    const float4 v = in[i];
+// the same for FP32 inputs, four elements per thread (sizes multiples of four, 16-byte aligned inputs, 8-byte aligned
+// outputs): up to three matrices in one launch, of which a small step would otherwise notice the launches
+struct Split4 {
+  const float4* in;
+  uint2* hi;
+  uint2* lo;
+  int64_t end;  // elements / 4 of this matrix and those before it
+};
+struct Split4s {
+  int n = 0;
+  Split4 m[3];
+};
+__global__ void k_split4(const Split4s a) {
+  const int64_t total = a.m[a.n - 1].end;
+  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < total; g += (int64_t)gridDim.x * blockDim.x) {
+    int k = 0;
+    while (g >= a.m[k].end) ++k;
+    const int64_t i = k ? g - a.m[k - 1].end : g;
+    const float4 v = a.m[k].in[i];
     const __nv_bfloat162 h01 = __floats2bfloat162_rn(v.x, v.y), h23 = __floats2bfloat162_rn(v.z, v.w);
     const float2 f01 = __bfloat1622float2(h01), f23 = __bfloat1622float2(h23);
     const __nv_bfloat162 l01 = __floats2bfloat162_rn(v.x - f01.x, v.y - f01.y);
     const __nv_bfloat162 l23 = __floats2bfloat162_rn(v.z - f23.x, v.w - f23.y);
-    hi[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&h01), *reinterpret_cast<const uint32_t*>(&h23));
-    if (lo) lo[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&l01), *reinterpret_cast<const uint32_t*>(&l23));
+    a.m[k].hi[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&h01), *reinterpret_cast<const uint32_t*>(&h23));
+    if (a.m[k].lo)
+      a.m[k].lo[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&l01), *reinterpret_cast<const uint32_t*>(&l23));
   }
 }
 
@@ -66,41 +82,67 @@ __global__ void k_to_float(const T* __restrict__ in, int64_t n, float* __restric
   if (i < n) out[i] = ld_f<T>(in, i);
 }
 
-// out[c, r] (two-part BF16, row pitch ld) = in[r, c] for r < rows; zero for rows <= r < ld
+// Transposes: out[c, r] (row pitch ld) = in[r, c] for r < rows, zero for rows <= r < ld; several matrices of one kind
+// in one launch, a block per tile of any of them.
+struct Turn {
+  const void* in;
+  int64_t rows, cols, ld;
+  __nv_bfloat16* hi;
+  __nv_bfloat16* lo;  // two-part output; null: one part
+  int64_t tiles_x, end;  // tiles across, and tiles of this matrix and those before it
+};
+constexpr int kTurns = 5;
+struct Turns {
+  int n = 0;
+  Turn m[kTurns];
+};
+__device__ __forceinline__ const Turn& turn_of(const Turns& a, int64_t tile, int64_t& tx, int64_t& ty) {
+  int k = 0;
+  while (tile >= a.m[k].end) ++k;
+  const uint32_t t = (uint32_t)(k ? tile - a.m[k - 1].end : tile), w = (uint32_t)a.m[k].tiles_x;  // (below 2^31)
+  tx = t % w;
+  ty = t / w;
+  return a.m[k];
+}
+
+// two-part BF16 from FP32 or one-part from BF16, 32 x 32 tiles
 template <typename T>
-__global__ void k_transpose_split(const T* __restrict__ in, int64_t rows, int64_t cols, __nv_bfloat16* __restrict__ hi,
-                                  __nv_bfloat16* __restrict__ lo, int64_t ld) {
+__global__ void k_transpose_split(const Turns a) {
   __shared__ float t[32][33];
-  const int64_t r0 = (int64_t)blockIdx.y * 32, c0 = (int64_t)blockIdx.x * 32;
+  int64_t tx, ty;
+  const Turn& m = turn_of(a, blockIdx.x, tx, ty);
+  const T* in = static_cast<const T*>(m.in);
+  const int64_t r0 = ty * 32, c0 = tx * 32;
   for (int y = threadIdx.y; y < 32; y += 8) {
     const int64_t r = r0 + y, c = c0 + threadIdx.x;
-    t[y][threadIdx.x] = (r < rows && c < cols) ? ld_f<T>(in, r * cols + c) : 0.f;
+    t[y][threadIdx.x] = (r < m.rows && c < m.cols) ? ld_f<T>(in, r * m.cols + c) : 0.f;
   }
   __syncthreads();
   for (int y = threadIdx.y; y < 32; y += 8) {
     const int64_t c = c0 + y, r = r0 + threadIdx.x;
-    if (c < cols && r < ld) {
+    if (c < m.cols && r < m.ld) {
       const float v = t[threadIdx.x][y];
       const __nv_bfloat16 h = __float2bfloat16_rn(v);
-      hi[c * ld + r] = h;
-      if (lo) lo[c * ld + r] = __float2bfloat16_rn(v - __bfloat162float(h));
+      m.hi[c * m.ld + r] = h;
+      if (m.lo) m.lo[c * m.ld + r] = __float2bfloat16_rn(v - __bfloat162float(h));
     }
   }
 }
 
-// out[c, r] = in[r, c] for BF16 (one part), 64 x 64 tiles moved in 16-byte
-// pieces (cols % 8 == 0, ld % 64 == 0, 16-byte aligned rows); zero for rows <= r < ld
-__global__ __launch_bounds__(256) void k_transpose_bf16(const __nv_bfloat16* __restrict__ in, int64_t rows,
-                                                        int64_t cols, __nv_bfloat16* __restrict__ out, int64_t ld) {
+// BF16 in one part, 64 x 64 tiles moved in 16-byte pieces (cols % 8 == 0, ld % 64 == 0, 16-byte aligned rows)
+__global__ __launch_bounds__(256) void k_transpose_bf16(const Turns a) {
   __shared__ __nv_bfloat16 t[64][72];
-  const int64_t r0 = (int64_t)blockIdx.y * 64, c0 = (int64_t)blockIdx.x * 64;
+  int64_t tx, ty;
+  const Turn& m = turn_of(a, blockIdx.x, tx, ty);
+  const __nv_bfloat16* in = static_cast<const __nv_bfloat16*>(m.in);
+  const int64_t r0 = ty * 64, c0 = tx * 64;
   const int tid = threadIdx.x, part = tid & 7;
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const int row = (tid >> 3) + 32 * i;
     const int64_t r = r0 + row, c = c0 + part * 8;
     uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (r < rows && c < cols) v = *reinterpret_cast<const uint4*>(in + r * cols + c);
+    if (r < m.rows && c < m.cols) v = *reinterpret_cast<const uint4*>(in + r * m.cols + c);
     *reinterpret_cast<uint4*>(&t[row][part * 8]) = v;
   }
   __syncthreads();
@@ -108,11 +150,11 @@ __global__ __launch_bounds__(256) void k_transpose_bf16(const __nv_bfloat16* __r
   for (int i = 0; i < 2; ++i) {
     const int oc = (tid >> 3) + 32 * i;
     const int64_t c = c0 + oc, r = r0 + part * 8;
-    if (c >= cols || r >= ld) continue;
+    if (c >= m.cols || r >= m.ld) continue;
     __align__(16) __nv_bfloat16 v[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) v[k] = t[part * 8 + k][oc];
-    *reinterpret_cast<uint4*>(out + c * ld + r) = *reinterpret_cast<const uint4*>(v);
+    *reinterpret_cast<uint4*>(m.hi + c * m.ld + r) = *reinterpret_cast<const uint4*>(v);
   }
 }
 
@@ -301,40 +343,124 @@ __global__ void k_onehot_prep(const int16_t* __restrict__ argmax, int64_t nq, in
   }
 }
 
-__global__ void k_view_coef(const int32_t* __restrict__ vquery, const int32_t* __restrict__ qoff, int64_t nq,
-                            float* __restrict__ coef) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nq) return;
-  const int b = vquery[i];
-  coef[i] = 1.f / (float)(qoff[b + 1] - qoff[b]);
-}
-
 // out_r = inv_r (g_r - (g_r . x_r inv_r) x_r inv_r): the gradient through x / |x| (warp per
-// row); g_r is the sum of `parts` partial rows G[s pstride + r dout], added in part order
-__global__ void k_tangent(const float* __restrict__ X, const float* __restrict__ inv, const float* __restrict__ G,
-                          int parts, int64_t pstride, int64_t n, int dout, float* __restrict__ out) {
-  const int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+// row), for the rows of U and V in one launch; g_r is the sum of `parts` partial rows
+// G[s pstride + r dout], added in part order. hi / lo (optional): the result's two-part copy.
+struct Tangent {
+  const float* x;
+  const float* inv;
+  const float* g;
+  int parts;
+  int64_t pstride, n;
+  float* out;
+  __nv_bfloat16* hi;
+  __nv_bfloat16* lo;
+};
+struct Tangents {
+  Tangent m[2];
+};
+// VW: elements per read, 4 where every row is 16-byte aligned
+template <int VW>
+struct VecOf;
+template <>
+struct VecOf<1> {
+  typedef float F;
+  typedef __nv_bfloat16 H;
+};
+template <>
+struct VecOf<4> {
+  typedef float4 F;
+  typedef uint2 H;
+};
+template <int VW>
+__global__ __launch_bounds__(256) void k_tangent(const Tangents a, int dout) {
+  typedef typename VecOf<VW>::F F;
+  typedef typename VecOf<VW>::H H;
+  int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  if (r >= n) return;
-  const float iv = inv[r];
-  const float* x = X + r * dout;
-  const float* g = G + r * dout;
-  auto g_at = [&](int d) {
-    float v = g[d];
-    for (int s = 1; s < parts; ++s) v += g[s * pstride + d];
-    return v;
+  const bool second = r >= a.m[0].n;
+  const Tangent m = second ? a.m[1] : a.m[0];
+  if (second) r -= a.m[0].n;
+  if (r >= m.n) return;
+  const float iv = m.inv[r];
+  const F* x = reinterpret_cast<const F*>(m.x + r * dout);
+  const F* g = reinterpret_cast<const F*>(m.g + r * dout);
+  const int64_t ps = m.pstride / VW;
+  const int n = dout / VW;
+  auto load = [&](const F* p, float (&v)[VW]) {
+    const F f = *p;
+#pragma unroll
+    for (int c = 0; c < VW; ++c) v[c] = reinterpret_cast<const float*>(&f)[c];
   };
+  auto g_at = [&](int i, float (&v)[VW]) {
+    load(g + i, v);
+    for (int s = 1; s < m.parts; ++s) {
+      float w[VW];
+      load(g + s * ps + i, w);
+#pragma unroll
+      for (int c = 0; c < VW; ++c) v[c] += w[c];
+    }
+  };
+  constexpr int kHeld = 16 / VW;  // reads held per lane: dout up to 512 reads everything once
+  float held[kHeld][VW], xs[kHeld][VW];
   float dot = 0.f;
-  for (int d = lane; d < dout; d += 32) dot = fmaf(x[d], g_at(d), dot);
+#pragma unroll
+  for (int k = 0; k < kHeld; ++k)
+    if (lane + 32 * k < n) {
+      g_at(lane + 32 * k, held[k]);
+      load(x + lane + 32 * k, xs[k]);
+    }
+#pragma unroll
+  for (int k = 0; k < kHeld; ++k)
+    if (lane + 32 * k < n)
+#pragma unroll
+      for (int c = 0; c < VW; ++c) dot = fmaf(xs[k][c], held[k][c], dot);
+  for (int i = lane + 32 * kHeld; i < n; i += 32) {
+    float gv[VW], xv[VW];
+    g_at(i, gv);
+    load(x + i, xv);
+#pragma unroll
+    for (int c = 0; c < VW; ++c) dot = fmaf(xv[c], gv[c], dot);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
   const float t = dot * iv * iv;
-  for (int d = lane; d < dout; d += 32) out[r * dout + d] = iv * (g_at(d) - t * x[d]);
+  auto put = [&](int i, const float (&gv)[VW], const float (&xv)[VW]) {
+    F f;
+    H hv, lv;
+#pragma unroll
+    for (int c = 0; c < VW; ++c) {
+      const float v = iv * (gv[c] - t * xv[c]);
+      reinterpret_cast<float*>(&f)[c] = v;
+      const __nv_bfloat16 h = __float2bfloat16_rn(v);
+      reinterpret_cast<__nv_bfloat16*>(&hv)[c] = h;
+      reinterpret_cast<__nv_bfloat16*>(&lv)[c] = __float2bfloat16_rn(v - __bfloat162float(h));
+    }
+    reinterpret_cast<F*>(m.out + r * dout)[i] = f;
+    if (m.hi) {
+      reinterpret_cast<H*>(m.hi + r * dout)[i] = hv;
+      reinterpret_cast<H*>(m.lo + r * dout)[i] = lv;
+    }
+  };
+#pragma unroll
+  for (int k = 0; k < kHeld; ++k)
+    if (lane + 32 * k < n) put(lane + 32 * k, held[k], xs[k]);
+  for (int i = lane + 32 * kHeld; i < n; i += 32) {
+    float gv[VW], xv[VW];
+    g_at(i, gv);
+    load(x + i, xv);
+    put(i, gv, xv);
+  }
 }
 
-__global__ void k_view_query(const int32_t* __restrict__ qoff, int32_t* __restrict__ vq) {
+// query of each view and 1 / |V(x_b)|
+__global__ void k_view_query(const int32_t* __restrict__ qoff, int32_t* __restrict__ vq, float* __restrict__ coef) {
   const int b = blockIdx.x;
-  for (int v = qoff[b] + threadIdx.x; v < qoff[b + 1]; v += blockDim.x) vq[v] = b;
+  const int v0 = qoff[b], v1 = qoff[b + 1];
+  for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
+    vq[v] = b;
+    coef[v] = 1.f / (float)(v1 - v0);
+  }
 }
 
 // ---------------------------------------------------------------- H = A^T U on the CUDA cores
@@ -591,7 +717,9 @@ struct Operand {
   int64_t rows_alloc = 0;
 };
 
-Operand make_operand(const void* x, int dtype, int64_t rows, int cols, bool force_split, Scratch& sc, cudaStream_t s) {
+// several: matrices whose split is left to be launched together (launch_splits)
+Operand make_operand(const void* x, int dtype, int64_t rows, int cols, bool force_split, Split4s& several, Scratch& sc,
+                     cudaStream_t s) {
   Operand o;
   if (dtype != GIFT_F32 && !force_split && rows >= tc::kTM && reinterpret_cast<uintptr_t>(x) % 16 == 0) {
     // a BF16 input is its own one-part operand: the tensor map covers its rows
@@ -607,11 +735,10 @@ Operand make_operand(const void* x, int dtype, int64_t rows, int cols, bool forc
   const bool vec = dtype == GIFT_F32 && n % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0 &&
                    reinterpret_cast<uintptr_t>(o.hi) % 8 == 0 && reinterpret_cast<uintptr_t>(o.lo) % 8 == 0;
   if (vec) {
-    const int64_t n4 = n / 4;
-    const unsigned grid = (unsigned)std::min<int64_t>(cdiv(n4, 256), (int64_t)device_sm_count() * 16);
-    k_split4<<<grid, 256, 0, s>>>(static_cast<const float4*>(x), n4, reinterpret_cast<uint2*>(o.hi),
-                                  reinterpret_cast<uint2*>(o.lo));
-    GIFT_LAUNCHED("k_split4");
+    several.m[several.n] = Split4{static_cast<const float4*>(x), reinterpret_cast<uint2*>(o.hi),
+                                  reinterpret_cast<uint2*>(o.lo),
+                                  n / 4 + (several.n ? several.m[several.n - 1].end : 0)};
+    ++several.n;
     return o;
   }
   if (dtype == GIFT_F32)
@@ -623,31 +750,52 @@ Operand make_operand(const void* x, int dtype, int64_t rows, int cols, bool forc
   return o;
 }
 
-// transposed operand: out [cols, ld] with ld = rows rounded up to 64; two-part
+void launch_splits(const Split4s& several, cudaStream_t s) {
+  if (!several.n) return;
+  const int64_t n4 = several.m[several.n - 1].end;
+  const unsigned grid = (unsigned)std::min<int64_t>(cdiv(n4, 256), (int64_t)device_sm_count() * 16);
+  k_split4<<<grid, 256, 0, s>>>(several);
+  GIFT_LAUNCHED("k_split4");
+}
+
+// transposed operands: out [cols, ld] with ld = rows rounded up to 64; two-part
 // for FP32 input, one-part (lo null) for BF16 input, which BF16 holds exactly
-Operand make_transposed(const void* x, int dtype, int64_t rows, int64_t cols, int64_t& ld, Scratch& sc,
-                        cudaStream_t s) {
-  Operand o;
-  ld = cdiv(rows, 64) * 64;
-  o.rows_alloc = cols + 128;
-  o.hi = sc.get<__nv_bfloat16>((size_t)o.rows_alloc * ld);
-  if (dtype == GIFT_F32) o.lo = sc.get<__nv_bfloat16>((size_t)o.rows_alloc * ld);
-  if (dtype != GIFT_F32 && cols % 8 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0 &&
-      reinterpret_cast<uintptr_t>(o.hi) % 16 == 0) {
-    const dim3 g64((unsigned)cdiv(cols, 64), (unsigned)cdiv(ld, 64));
-    k_transpose_bf16<<<g64, 256, 0, s>>>(static_cast<const __nv_bfloat16*>(x), rows, cols, o.hi, ld);
-    GIFT_LAUNCHED("k_transpose_bf16");
+struct Transposes {
+  Turns f32, bf16, wide;  // FP32 inputs, BF16 inputs, BF16 inputs in 16-byte pieces
+  Operand add(const void* x, int dtype, int64_t rows, int64_t cols, int64_t& ld, Scratch& sc) {
+    Operand o;
+    ld = cdiv(rows, 64) * 64;
+    o.rows_alloc = cols + 128;
+    o.hi = sc.get<__nv_bfloat16>((size_t)o.rows_alloc * ld);
+    if (dtype == GIFT_F32) o.lo = sc.get<__nv_bfloat16>((size_t)o.rows_alloc * ld);
+    const bool pieces = dtype != GIFT_F32 && cols % 8 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0 &&
+                        reinterpret_cast<uintptr_t>(o.hi) % 16 == 0;
+    Turns& t = dtype == GIFT_F32 ? f32 : pieces ? wide : bf16;
+    const int64_t side = pieces ? 64 : 32, tx = cdiv(cols, side);
+    t.m[t.n] = Turn{x, rows, cols, ld, o.hi, o.lo, tx, tx * cdiv(ld, side) + (t.n ? t.m[t.n - 1].end : 0)};
+    ++t.n;
     return o;
   }
-  const dim3 grid((unsigned)cdiv(cols, 32), (unsigned)cdiv(ld, 32)), blk(32, 8);
-  if (dtype == GIFT_F32)
-    k_transpose_split<float><<<grid, blk, 0, s>>>(static_cast<const float*>(x), rows, cols, o.hi, o.lo, ld);
-  else
-    k_transpose_split<__nv_bfloat16><<<grid, blk, 0, s>>>(static_cast<const __nv_bfloat16*>(x), rows, cols, o.hi,
-                                                          o.lo, ld);
-  GIFT_LAUNCHED("k_transpose_split");
-  return o;
-}
+  static unsigned blocks(const Turns& t) {
+    const int64_t n = t.m[t.n - 1].end;
+    GIFT_REQUIRE(n < (int64_t)INT32_MAX, "too many views for the weight gradient");
+    return (unsigned)n;
+  }
+  void launch(cudaStream_t s) const {
+    if (f32.n) {
+      k_transpose_split<float><<<blocks(f32), dim3(32, 8), 0, s>>>(f32);
+      GIFT_LAUNCHED("k_transpose_split");
+    }
+    if (bf16.n) {
+      k_transpose_split<__nv_bfloat16><<<blocks(bf16), dim3(32, 8), 0, s>>>(bf16);
+      GIFT_LAUNCHED("k_transpose_split");
+    }
+    if (wide.n) {
+      k_transpose_bf16<<<blocks(wide), 256, 0, s>>>(wide);
+      GIFT_LAUNCHED("k_transpose_bf16");
+    }
+  }
+};
 
 float* as_float(const void* x, int dtype, int64_t n, Scratch& sc, cudaStream_t s) {
   if (dtype == GIFT_F32) return const_cast<float*>(static_cast<const float*>(x));
@@ -662,15 +810,58 @@ struct Proj {
   float* V;
   float* uinv;
   float* vinv;
+  Operand Uo, Vo;  // two-part copies (forward)
 };
 
+// inverse norms of the rows of U and V, and their two-part copies where hi is given; warp per row, both matrices in one
+// launch (sums as k_row_invnorm's)
+struct NormRows {
+  const float* x[2];
+  int64_t n[2];
+  float* inv[2];
+  __nv_bfloat16* hi[2];
+  __nv_bfloat16* lo[2];
+};
+template <bool PARTS>
+__global__ __launch_bounds__(256) void k_norm_rows(const NormRows a, int D) {
+  int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  const int m = row >= a.n[0] ? 1 : 0;
+  if (m) row -= a.n[0];
+  if (row >= a.n[m]) return;
+  const float4* p = reinterpret_cast<const float4*>(a.x[m] + row * (int64_t)D);
+  uint2* h = reinterpret_cast<uint2*>(a.hi[m] + row * (int64_t)D);
+  uint2* l = reinterpret_cast<uint2*>(a.lo[m] + row * (int64_t)D);
+  float acc = 0.f;
+#pragma unroll 4
+  for (int i = lane; i < (D >> 2); i += 32) {
+    const float4 v = p[i];
+    acc = fmaf(v.x, v.x, acc);
+    acc = fmaf(v.y, v.y, acc);
+    acc = fmaf(v.z, v.z, acc);
+    acc = fmaf(v.w, v.w, acc);
+    if (!PARTS) continue;
+    const __nv_bfloat162 a2 = __floats2bfloat162_rn(v.x, v.y), b2 = __floats2bfloat162_rn(v.z, v.w);
+    const float2 fa = __bfloat1622float2(a2), fb = __bfloat1622float2(b2);
+    const __nv_bfloat162 c2 = __floats2bfloat162_rn(v.x - fa.x, v.y - fa.y);
+    const __nv_bfloat162 d2 = __floats2bfloat162_rn(v.z - fb.x, v.w - fb.y);
+    h[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&a2), *reinterpret_cast<const uint32_t*>(&b2));
+    l[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&c2), *reinterpret_cast<const uint32_t*>(&d2));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) a.inv[m][row] = acc > 0.f ? 1.0f / sqrtf(acc) : 0.f;
+}
+
 Proj project(const void* q, int64_t nq, const void* p, int64_t nr, const void* W, int din, int dout, int dtype,
-             int* err, Scratch& sc, cudaStream_t s) {
+             bool parts, int* err, Scratch& sc, cudaStream_t s) {
   Proj P;
   if (W) {
-    const Operand Qo = make_operand(q, dtype, nq, din, false, sc, s);
-    const Operand Po = make_operand(p, dtype, nr, din, false, sc, s);
-    const Operand Wo = make_operand(W, dtype, dout, din, false, sc, s);
+    Split4s several;
+    const Operand Qo = make_operand(q, dtype, nq, din, false, several, sc, s);
+    const Operand Po = make_operand(p, dtype, nr, din, false, several, sc, s);
+    const Operand Wo = make_operand(W, dtype, dout, din, false, several, sc, s);
+    launch_splits(several, s);
     P.U = sc.get<float>((size_t)nq * dout);
     P.V = sc.get<float>((size_t)nr * dout);
     gemm_tc(Qo.hi, Qo.lo, nq, Qo.rows_alloc, 0, Wo.hi, Wo.lo, dout, Wo.rows_alloc, 0, din, P.U, dout, 0, err, s);
@@ -681,8 +872,20 @@ Proj project(const void* q, int64_t nq, const void* p, int64_t nr, const void* W
   }
   P.uinv = sc.get<float>(nq);
   P.vinv = sc.get<float>(nr);
-  launch_row_invnorm(P.U, nq, dout, P.uinv, s);
-  launch_row_invnorm(P.V, nr, dout, P.vinv, s);
+  NormRows nr2{{P.U, P.V}, {nq, nr}, {P.uinv, P.vinv}, {nullptr, nullptr}, {nullptr, nullptr}};
+  if (parts) {
+    Operand* o[2] = {&P.Uo, &P.Vo};
+    for (int m = 0; m < 2; ++m) {
+      o[m]->rows_alloc = nr2.n[m] + 128;
+      o[m]->hi = nr2.hi[m] = sc.get<__nv_bfloat16>((size_t)o[m]->rows_alloc * dout);
+      o[m]->lo = nr2.lo[m] = sc.get<__nv_bfloat16>((size_t)o[m]->rows_alloc * dout);
+    }
+  }
+  if (parts)
+    k_norm_rows<true><<<(unsigned)cdiv(nq + nr, 8), 256, 0, s>>>(nr2, dout);
+  else
+    k_norm_rows<false><<<(unsigned)cdiv(nq + nr, 8), 256, 0, s>>>(nr2, dout);
+  GIFT_LAUNCHED("k_norm_rows");
   return P;
 }
 
@@ -706,11 +909,9 @@ void match_forward(const void* q, const std::vector<int32_t>& h_qoff, int32_t Bq
   const int64_t nq = h_qoff[Bq];
   const int64_t nr = (int64_t)Np * nv;
   int* err = device_flag(sc, s);
-  const Proj P = project(q, nq, p, nr, W, din, dout, dtype, err, sc, s);
-  const Operand Uo = make_operand(P.U, GIFT_F32, nq, dout, true, sc, s);
-  const Operand Vo = make_operand(P.V, GIFT_F32, nr, dout, true, sc, s);
+  const Proj P = project(q, nq, p, nr, W, din, dout, dtype, true, err, sc, s);
   int32_t* d_qoff = device_offsets(h_qoff, sc, s);
-  segmax_tc(Uo.hi, Uo.lo, Uo.rows_alloc, P.uinv, Vo.hi, Vo.lo, Vo.rows_alloc, P.vinv, nr, nv, dout, d_qoff, h_qoff,
+  segmax_tc(P.Uo.hi, P.Uo.lo, P.Uo.rows_alloc, P.uinv, P.Vo.hi, P.Vo.lo, P.Vo.rows_alloc, P.vinv, nr, nv, dout, d_qoff, h_qoff,
             Bq, S, argmax, err, sc, s);
 }
 
@@ -720,17 +921,15 @@ void match_backward(const void* q, const std::vector<int32_t>& h_qoff, int32_t B
   const int64_t nq = h_qoff[Bq];
   const int64_t nr = (int64_t)Np * nv;
   int* err = device_flag(sc, s);
-  const Proj P = project(q, nq, p, nr, W, din, dout, dtype, err, sc, s);
+  const Proj P = project(q, nq, p, nr, W, din, dout, dtype, false, err, sc, s);
   int32_t* d_qoff = device_offsets(h_qoff, sc, s);
   int32_t* vquery = sc.get<int32_t>(nq);
-  k_view_query<<<(unsigned)Bq, 128, 0, s>>>(d_qoff, vquery);
+  float* vcoef = sc.get<float>(nq);
+  k_view_query<<<(unsigned)Bq, 128, 0, s>>>(d_qoff, vquery, vcoef);
   GIFT_LAUNCHED("k_view_query");
   // gradients w.r.t. the projected views (without a projection these are dQ, dP)
   float* dU = (W || !dQ) ? sc.get<float>((size_t)nq * dout) : dQ;
   float* dV = (W || !dP) ? sc.get<float>((size_t)nr * dout) : dP;
-  float* vcoef = sc.get<float>(nq);
-  k_view_coef<<<(unsigned)cdiv(nq, 256), 256, 0, s>>>(vquery, d_qoff, nq, vcoef);
-  GIFT_LAUNCHED("k_view_coef");
   // steps of the query-side gather
   GatherSteps st;
   if (nv <= kGViews) {
@@ -762,7 +961,8 @@ void match_backward(const void* q, const std::vector<int32_t>& h_qoff, int32_t B
   const float* U16 = aligned16(P.U, nq * dout);
   const float* V16 = aligned16(P.V, nr * dout);
   const int sms = device_sm_count();
-  {  // G = A V, then dU
+  Tangents tg;
+  {  // G = A V
     // parts of the step range: a block's time is ~ steps / parts, the launch takes
     // ceil(blocks x parts / SMs) rounds of one block per SM; partial rows cost a little
     const int64_t units = cdiv(nq, (int64_t)kGRows) * cdiv((int64_t)dout, (int64_t)kGCols);
@@ -784,10 +984,9 @@ void match_backward(const void* q, const std::vector<int32_t>& h_qoff, int32_t B
                     (unsigned)parts);
     k_gather_views<<<grid, kGT, smem, s>>>(V16, gR, nq, ldq, Np, nv, dout, st, Gp);
     GIFT_LAUNCHED("k_gather_views");
-    k_tangent<<<(unsigned)cdiv(nq, 8), 256, 0, s>>>(P.U, P.uinv, Gp, parts, nq * dout, nq, dout, dU);
-    GIFT_LAUNCHED("k_tangent");
+    tg.m[0] = Tangent{P.U, P.uinv, Gp, parts, nq * dout, nq, dU, nullptr, nullptr};
   }
-  {  // H = A^T U, then dV
+  {  // H = A^T U
     float* H = sc.get<float>((size_t)nr * dout);
     if (nv <= kCsrMaxNv) {  // entries grouped per shape, then one warp per database view
       const int64_t ne = ldq * (int64_t)Np;
@@ -812,35 +1011,48 @@ void match_backward(const void* q, const std::vector<int32_t>& h_qoff, int32_t B
       k_gather_entries<<<grid, kHT, smem, s>>>(U16, amT, wV, nq, ldq, nr, nv, dout, H);
       GIFT_LAUNCHED("k_gather_entries");
     }
-    k_tangent<<<(unsigned)cdiv(nr, 8), 256, 0, s>>>(P.V, P.vinv, H, 1, 0, nr, dout, dV);
-    GIFT_LAUNCHED("k_tangent");
+    tg.m[1] = Tangent{P.V, P.vinv, H, 1, 0, nr, dV, nullptr, nullptr};
   }
+  // through the normalisation; the gradients that dQ and dP multiply leave as two parts too
+  Operand dUo, dVo;
+  auto two_parts = [&](Operand& o, Tangent& t) {
+    o.rows_alloc = t.n + 128;
+    o.hi = t.hi = sc.get<__nv_bfloat16>((size_t)o.rows_alloc * dout);
+    o.lo = t.lo = sc.get<__nv_bfloat16>((size_t)o.rows_alloc * dout);
+  };
+  if (W && dQ) two_parts(dUo, tg.m[0]);
+  if (W && dP) two_parts(dVo, tg.m[1]);
+  bool wide = true;  // (d_out is a multiple of 16)
+  for (const Tangent& t : tg.m)
+    for (const void* ptr : {(const void*)t.x, (const void*)t.g, (const void*)t.out})
+      wide = wide && reinterpret_cast<uintptr_t>(ptr) % 16 == 0;
+  if (wide)
+    k_tangent<4><<<(unsigned)cdiv(nq + nr, 8), 256, 0, s>>>(tg, dout);
+  else
+    k_tangent<1><<<(unsigned)cdiv(nq + nr, 8), 256, 0, s>>>(tg, dout);
+  GIFT_LAUNCHED("k_tangent");
   if (!W) return;
+  Transposes turns;
+  int64_t ldt = 0, ldr = 0, ldo = 0;
+  Operand dUt, Qt, dVt, Pt, Wt;
   if (dW) {
-    int64_t ldq = 0, ldr = 0;
-    const Operand dUt = make_transposed(dU, GIFT_F32, nq, dout, ldq, sc, s);
-    const Operand Qt = make_transposed(q, dtype, nq, din, ldq, sc, s);
-    gemm_tc(dUt.hi, dUt.lo, dout, dUt.rows_alloc, ldq, Qt.hi, Qt.lo, din, Qt.rows_alloc, ldq, (int)ldq, dW, din, 0,
+    dUt = turns.add(dU, GIFT_F32, nq, dout, ldt, sc);
+    Qt = turns.add(q, dtype, nq, din, ldt, sc);
+    dVt = turns.add(dV, GIFT_F32, nr, dout, ldr, sc);
+    Pt = turns.add(p, dtype, nr, din, ldr, sc);
+  }
+  if (dQ || dP) Wt = turns.add(W, dtype, dout, din, ldo, sc);  // [din, ldo], K = dout
+  turns.launch(s);
+  if (dW) {
+    gemm_tc(dUt.hi, dUt.lo, dout, dUt.rows_alloc, ldt, Qt.hi, Qt.lo, din, Qt.rows_alloc, ldt, (int)ldt, dW, din, 0,
             err, s, &sc);
-    const Operand dVt = make_transposed(dV, GIFT_F32, nr, dout, ldr, sc, s);
-    const Operand Pt = make_transposed(p, dtype, nr, din, ldr, sc, s);
     gemm_tc(dVt.hi, dVt.lo, dout, dVt.rows_alloc, ldr, Pt.hi, Pt.lo, din, Pt.rows_alloc, ldr, (int)ldr, dW, din, 1,
             err, s, &sc);
   }
-  if (dQ || dP) {
-    int64_t ldo = 0;
-    const Operand Wt = make_transposed(W, dtype, dout, din, ldo, sc, s);  // [din, ldo], K = dout
-    if (dQ) {
-      const Operand dUo = make_operand(dU, GIFT_F32, nq, dout, true, sc, s);
-      gemm_tc(dUo.hi, dUo.lo, nq, dUo.rows_alloc, dout, Wt.hi, Wt.lo, din, Wt.rows_alloc, ldo, dout, dQ, din, 0, err,
-              s);
-    }
-    if (dP) {
-      const Operand dVo = make_operand(dV, GIFT_F32, nr, dout, true, sc, s);
-      gemm_tc(dVo.hi, dVo.lo, nr, dVo.rows_alloc, dout, Wt.hi, Wt.lo, din, Wt.rows_alloc, ldo, dout, dP, din, 0, err,
-              s);
-    }
-  }
+  if (dQ)
+    gemm_tc(dUo.hi, dUo.lo, nq, dUo.rows_alloc, dout, Wt.hi, Wt.lo, din, Wt.rows_alloc, ldo, dout, dQ, din, 0, err, s);
+  if (dP)
+    gemm_tc(dVo.hi, dVo.lo, nr, dVo.rows_alloc, dout, Wt.hi, Wt.lo, din, Wt.rows_alloc, ldo, dout, dP, din, 0, err, s);
 }
 
 }  // namespace gift
