@@ -421,8 +421,14 @@ def _autograd_function():
 
 
 class _Lazy:
+    """The autograd function, made on first use (torch is imported then) and kept."""
+
+    _fn = None
+
     def __getattr__(self, item):
-        return getattr(_autograd_function(), item)
+        if _Lazy._fn is None:
+            _Lazy._fn = _autograd_function()
+        return getattr(_Lazy._fn, item)
 
 
 GiftMatch = _Lazy()

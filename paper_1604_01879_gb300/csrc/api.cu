@@ -484,8 +484,25 @@ Scratch::~Scratch() {
 }
 
 void* Scratch::raw(size_t bytes) {
+  bytes = std::max<size_t>((bytes + 255) / 256 * 256, 256);  // (pieces start as an allocation would)
+  if (bytes <= kSmall && bytes > slab_left) {
+    void* p = nullptr;
+    if (cudaMallocAsync(&p, kSlab, stream) == cudaSuccess) {
+      blocks.push_back(p);
+      slab = static_cast<uint8_t*>(p);
+      slab_left = kSlab;
+    } else {
+      cudaGetLastError();  // no room for a slab: the piece alone may fit
+    }
+  }
+  if (bytes <= kSmall && bytes <= slab_left) {
+    void* p = slab;
+    slab += bytes;
+    slab_left -= bytes;
+    return p;
+  }
   void* p = nullptr;
-  cudaError_t e = cudaMallocAsync(&p, std::max<size_t>(bytes, 16), stream);
+  cudaError_t e = cudaMallocAsync(&p, bytes, stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     fail(GIFT_ENOMEM, "scratch allocation of " + std::to_string(bytes) + " bytes failed");

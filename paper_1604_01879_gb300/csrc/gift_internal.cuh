@@ -36,9 +36,14 @@ void count_launch();
 // ---------------------------------------------------------------- scratch
 // Stream-ordered scratch: every allocation is released (stream-ordered) when
 // the Scratch object goes out of scope, so concurrent calls never share it.
+// Small pieces are cut from slabs: a call makes some forty of them, and an
+// allocation with its release costs the host about as much as a launch.
 struct Scratch {
+  static constexpr size_t kSlab = 4u << 20, kSmall = 512u << 10;
   cudaStream_t stream;
   std::vector<void*> blocks;
+  uint8_t* slab = nullptr;
+  size_t slab_left = 0;
   explicit Scratch(cudaStream_t s) : stream(s) {}
   ~Scratch();
   void* raw(size_t bytes);

@@ -1,4 +1,6 @@
 // Host helpers of the tcgen05 kernels: TMA tensor maps and device queries.
+#include <atomic>
+
 #include "tc_common.cuh"
 
 namespace gift {
@@ -63,9 +65,13 @@ CUtensorMap make_tmap_u8(const void* base, uint64_t rows, uint64_t cols, uint32_
 }
 
 int device_sm_count() {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices];  // a property of the device, asked once
   int dev = 0, n = 0;
   GIFT_CUDA(cudaGetDevice(&dev));
+  if (dev < kDevices && (n = known[dev].load()) > 0) return n;
   GIFT_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+  if (dev < kDevices) known[dev].store(n);
   return n;
 }
 
