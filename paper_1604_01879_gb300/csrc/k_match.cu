@@ -174,18 +174,27 @@ __device__ __forceinline__ void cp_async_wait() {
 // row of V, so the product has N_v times fewer multiply-adds than the dense one-hot
 // GEMM. A block owns 256 query views x 128 columns (16 warps of 16 views, 4 columns
 // per lane, accumulators in registers) and walks the shapes in ascending order. A
-// step stages, in shared memory (cp.async, three stages), the rows of up to 64
-// database views restricted to the block's columns together with the entry records
-// of the block's query views in those shapes: a row of V leaves L2 once per block
-// instead of once per entry, and each entry is one broadcast record read, one
-// 512-byte shared-memory read and four multiply-adds. A step is up to kGShapes whole
-// shapes of at most 64 views together, or one 64-view piece of a larger shape. The
+// step stages, in shared memory, the rows of up to 64 database views restricted to the
+// block's columns together with the entry records of the block's query views in those
+// shapes: a row of V leaves L2 once per block instead of once per entry, and each entry
+// is one broadcast record read, one 512-byte shared-memory read and four multiply-adds.
+// The stages are a ring of up to eight, filled by one thread of a 17th warp (a TMA tile of
+// V and a bulk copy per shape's records) and freed warp by warp, so the warps drift apart
+// and none issues copies: what is left is the 512-byte reads (137 GB at full size, 16,384 x 4,096
+// entries of 512 columns: 3.4 ms at shared memory's rate), the records' and the copies' share of
+// it, and their issue: 7.41 ms with copies by every thread and a barrier per step, 6.59 now.
+// A step is up to kGShapes whole shapes of at most 64 views together, or one 64-view piece of a larger shape. The
 // steps may be split into parts (blockIdx.z) whose partial sums k_tangent adds in
 // part order: the result does not depend on the launch.
-constexpr int kGT = 512, kGRows = 256, kGCols = 128, kGStages = 3, kGViews = 64, kGShapes = 8;
-constexpr int kGRecOff = (kGViews + 1) * kGCols * 4;            // 33,280: V rows + one zero row
-constexpr int kGStageBytes = kGRecOff + kGShapes * kGRows * 8;  // 49,664: + records [kGShapes][kGRows]
-static_assert(kGStageBytes % 16 == 0 && kGRecOff % 16 == 0, "stage alignment");
+constexpr int kGWarps = 16, kGT = 32 * (kGWarps + 1), kGRows = 256, kGCols = 128, kGStages = 8, kGViews = 64, kGShapes = 8;
+constexpr int kGRecOff = (kGViews + 1) * kGCols * 4;  // 33,280: V rows + one zero row, then records [shapes][kGRows]
+constexpr int kGSmem = 227 * 1024;
+static_assert(kGRecOff % 128 == 0, "stage alignment");
+// bytes of a stage and stages of the ring for steps of `shapes` record rows
+__host__ __device__ constexpr int g_stage_bytes(int shapes) { return kGRecOff + shapes * kGRows * 8; }
+__host__ __device__ constexpr int g_stages(int shapes) {
+  return (kGSmem - 1024) / g_stage_bytes(shapes) < kGStages ? (kGSmem - 1024) / g_stage_bytes(shapes) : kGStages;
+}
 
 struct GatherSteps {
   int spc;  // whole shapes per step (N_v <= 64); 0: 64-view pieces of one shape
@@ -228,49 +237,76 @@ __device__ __forceinline__ void g_add(float (&acc)[4], float w, const float4 x) 
   acc[3] = fmaf(w, x.w, acc[3]);
 }
 
-// gR: [Np, ldq] entry records (ldq a multiple of kGRows; no entry past nq);
-// V: [nr, dout] (16-byte aligned, dout % 4 == 0); Gp: [parts, nq, dout]
-__global__ __launch_bounds__(kGT, 1) void k_gather_views(const float* __restrict__ V, const float2* __restrict__ gR,
-                                                         int64_t nq, int64_t ldq, int Np, int nv, int dout,
-                                                         GatherSteps st, float* __restrict__ Gp) {
-  extern __shared__ __align__(16) uint8_t g_sm[];
+// tmV: V [nr, dout] in boxes of 64 rows x 128 columns; gR: [Np, ldq] entry records (ldq a multiple of kGRows; no
+// entry past nq); Gp: [parts, nq, dout]; every wait is bounded, and gives up once err is set
+__global__ __launch_bounds__(kGT, 1) void k_gather_views(const __grid_constant__ CUtensorMap tmV,
+                                                         const float2* __restrict__ gR, int64_t nq, int64_t ldq, int Np,
+                                                         int nv, int dout, GatherSteps st, float* __restrict__ Gp,
+                                                         int* err) {
+  extern __shared__ __align__(128) uint8_t g_raw[];
+  uint8_t* g_sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(g_raw) + 127) & ~uintptr_t(127));
+  const int shapes = st.spc > 0 ? st.spc : 1;
+  const int bytes = g_stage_bytes(shapes), ring = g_stages(shapes);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(g_sm + (size_t)ring * bytes);
+  const uint32_t full0 = tc::smem_u32(bars), empty0 = full0 + 8 * kGStages;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int64_t i0 = (int64_t)blockIdx.x * kGRows;
   const int c0 = blockIdx.y * kGCols;
   const int part = blockIdx.z, parts = gridDim.z;
   const int s0 = (int)((int64_t)st.n * part / parts), s1 = (int)((int64_t)st.n * (part + 1) / parts);
-  for (int t = tid; t < kGStages * 32; t += kGT)  // the zero row of every stage (never a copy target)
-    *reinterpret_cast<float4*>(g_sm + (t >> 5) * kGStageBytes + kGViews * kGCols * 4 + (t & 31) * 16) =
+  for (int t = tid; t < ring * 32; t += kGT)  // the zero row of every stage (never a copy target)
+    *reinterpret_cast<float4*>(g_sm + (size_t)(t >> 5) * bytes + kGViews * kGCols * 4 + (t & 31) * 16) =
         make_float4(0.f, 0.f, 0.f, 0.f);
-  auto issue = [&](int s) {
-    if (s < s1) {
-      uint8_t* buf = g_sm + ((s - s0) % kGStages) * kGStageBytes;
-      int p0, nps, nvs;
-      int64_t vb;
-      g_step(st, s, nv, Np, p0, nps, vb, nvs);
-      for (int t = tid; t < nvs * 32; t += kGT) {  // rows of V, 16-byte pieces of the column slice
-        const int row = t >> 5, q = t & 31, c = c0 + 4 * q;
-        if (c < dout) cp_async16(buf + (row * kGCols + 4 * q) * 4, V + (vb + row) * dout + c);
+  if (tid == 0) {
+    for (int k = 0; k < ring; ++k) {
+      tc::mbar_init(full0 + 8 * k, 1);
+      tc::mbar_init(empty0 + 8 * k, kGWarps);
+    }
+    tc::fence_barrier_init();
+  }
+  __syncthreads();
+  int stage = 0;
+  uint32_t phase = 0;
+  if (w == kGWarps) {
+    if (lane == 0) {
+      tc::prefetch_tmap(&tmV);
+      bool ok = true;
+      int issued = 0;
+      for (int s = s0; s < s1; ++s) {
+        if (!tc::mbar_wait(empty0 + 8 * stage, phase ^ 1, err, tc::kErrProducer)) {
+          ok = false;
+          break;
+        }
+        int p0, nps, nvs;
+        int64_t vb;
+        g_step(st, s, nv, Np, p0, nps, vb, nvs);
+        const uint32_t buf = tc::smem_u32(g_sm + (size_t)stage * bytes), bar = full0 + 8 * stage;
+        tc::mbar_expect_tx(bar, kGViews * kGCols * 4 + nps * kGRows * 8);
+        tc::tma_load_2d(buf, &tmV, c0, (int)vb, bar);  // (rows past the step's are staged and not read)
+        for (int ps = 0; ps < nps; ++ps)
+          tc::bulk_load(buf + kGRecOff + ps * kGRows * 8, gR + (int64_t)(p0 + ps) * ldq + i0, kGRows * 8, bar);
+        ++issued;
+        if (++stage == ring) {
+          stage = 0;
+          phase ^= 1;
+        }
       }
-      for (int t = tid; t < nps * 128; t += kGT) {  // per shape: 256 records, 128 pieces
-        const int ps = t >> 7, q = t & 127;
-        cp_async16(buf + kGRecOff + ps * (kGRows * 8) + 16 * q, gR + (int64_t)(p0 + ps) * ldq + i0 + 2 * q);
+      if (!ok && issued) {  // let issued copies land before exiting (bounded)
+        const long long t0 = clock64();
+        while (clock64() - t0 < tc::kWaitCycles / 4) {
+        }
       }
     }
-    cp_async_commit();  // empty groups past the last step keep the wait count uniform
-  };
+    return;
+  }
   float acc[16][4];
 #pragma unroll
   for (int k = 0; k < 16; ++k)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[k][q] = 0.f;
-#pragma unroll
-  for (int k = 0; k < kGStages - 1; ++k) issue(s0 + k);
   for (int s = s0; s < s1; ++s) {
-    cp_async_wait<kGStages - 2>();  // this step's copies have landed ...
-    __syncthreads();                // ... for every thread, and the step before is done with its buffer
-    issue(s + kGStages - 1);
-    const uint8_t* buf = g_sm + ((s - s0) % kGStages) * kGStageBytes;
+    if (!tc::mbar_wait(full0 + 8 * stage, phase, err, tc::kErrEpilogue)) break;
+    const uint8_t* buf = g_sm + (size_t)stage * bytes;
     const float4* vs = reinterpret_cast<const float4*>(buf) + lane;
     int p0, nps, nvs;
     int64_t vb;
@@ -296,8 +332,13 @@ __global__ __launch_bounds__(kGT, 1) void k_gather_views(const float* __restrict
         }
       }
     }
+    __syncwarp();
+    if (lane == 0) tc::mbar_arrive(empty0 + 8 * stage);
+    if (++stage == ring) {
+      stage = 0;
+      phase ^= 1;
+    }
   }
-  cp_async_wait<0>();
   const int c = c0 + 4 * lane;
   if (c >= dout) return;
 #pragma unroll
@@ -978,11 +1019,11 @@ void match_backward(const void* q, const std::vector<int32_t>& h_qoff, int32_t B
       }
     }
     float* Gp = sc.get<float>((size_t)parts * nq * dout);
-    const size_t smem = (size_t)kGStages * kGStageBytes;
-    GIFT_CUDA(cudaFuncSetAttribute(k_gather_views, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    GIFT_CUDA(cudaFuncSetAttribute(k_gather_views, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem));
     const dim3 grid((unsigned)cdiv(nq, (int64_t)kGRows), (unsigned)cdiv((int64_t)dout, (int64_t)kGCols),
                     (unsigned)parts);
-    k_gather_views<<<grid, kGT, smem, s>>>(V16, gR, nq, ldq, Np, nv, dout, st, Gp);
+    const CUtensorMap tmV = make_tmap_f32(V16, nr, dout, kGCols, kGViews);
+    k_gather_views<<<grid, kGT, kGSmem, s>>>(tmV, gR, nq, ldq, Np, nv, dout, st, Gp, err);
     GIFT_LAUNCHED("k_gather_views");
     tg.m[0] = Tangent{P.U, P.uinv, Gp, parts, nq * dout, nq, dU, nullptr, nullptr};
   }

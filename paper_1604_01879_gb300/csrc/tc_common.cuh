@@ -85,6 +85,13 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
       : "memory");
 }
 
+// contiguous copy global -> shared (16-byte aligned, a multiple of 16 bytes), completion counted on `bar`
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
+               : "memory");
+}
+
 // hint: bring the 128-byte line holding p into L2 (no register result, no wait)
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<uint64_t>(p)));
@@ -203,6 +210,9 @@ __host__ __device__ inline bool pair_wins(int64_t items, int64_t pair_items, int
 CUtensorMap make_tmap_bf16(const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint64_t pitch = 0);
 // host: the same for a byte matrix (FP8 rows): box {128 columns (128 bytes), box_rows rows}.
 CUtensorMap make_tmap_u8(const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint64_t pitch = 0);
+// host: 2-D FP32 tensor map, box {box_cols columns, box_rows rows}, no swizzle, zero fill outside (the box may be
+// larger than the matrix); 16-byte aligned base, cols a multiple of 4.
+CUtensorMap make_tmap_f32(const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols, uint32_t box_rows);
 int device_sm_count();
 
 }  // namespace gift

@@ -64,6 +64,22 @@ CUtensorMap make_tmap_u8(const void* base, uint64_t rows, uint64_t cols, uint32_
   return m;
 }
 
+CUtensorMap make_tmap_f32(const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols, uint32_t box_rows) {
+  GIFT_REQUIRE(reinterpret_cast<uintptr_t>(base) % 16 == 0, "tensor map base must be 16-byte aligned");
+  GIFT_REQUIRE(cols % 4 == 0 && rows >= 1, "tensor map rows must be multiples of 16 bytes");
+  GIFT_REQUIRE(box_rows >= 1 && box_rows <= 256 && box_cols % 4 == 0 && box_cols <= 256, "tensor map box out of range");
+  CUtensorMap m;
+  const cuuint64_t dims[2] = {cols, rows};
+  const cuuint64_t strides[1] = {cols * 4};
+  const cuuint32_t box[2] = {box_cols, box_rows};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims, strides, box,
+                                 estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                 CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) fail(GIFT_ECUDA, "cuTensorMapEncodeTiled failed with " + std::to_string((int)r));
+  return m;
+}
+
 int device_sm_count() {
   constexpr int kDevices = 64;
   static std::atomic<int> known[kDevices];  // a property of the device, asked once
