@@ -541,14 +541,19 @@ __global__ void k_unfix_rows(const unsigned long long* __restrict__ acc, const i
 // Candidate scores (ma = 1): one block per query, its warps over the query's
 // views; a run's term is added at its shape's position among the query's
 // sorted candidates (shared fixed-point sums).
+// The candidates are searched in shared memory: in global memory every run's search was
+// eight dependent reads (1,000 queries of 64 views, R = 200: 200 us, 178 now).
 __global__ __launch_bounds__(kCombineT) void k_fif_combine_cand(const CombineArgs a) {
-  extern __shared__ unsigned long long acc[];
+  extern __shared__ unsigned long long acc[];  // [R] sums, then int32 candidates [R]
+  int32_t* cand = reinterpret_cast<int32_t*>(acc + a.R);
   const int q = blockIdx.x;
-  for (int i = threadIdx.x; i < a.R; i += kCombineT) acc[i] = 0ull;
+  for (int i = threadIdx.x; i < a.R; i += kCombineT) {
+    acc[i] = 0ull;
+    cand[i] = a.cand[(int64_t)q * a.R + i];
+  }
   __syncthreads();
   const int v0 = a.qoff[q], v1 = a.qoff[q + 1];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int32_t* cand = a.cand + (int64_t)q * a.R;
   for (int v = v0 + w; v < v1; v += kCombineT / 32) {
     const int32_t s = a.view_slot[v];
     const int k = a.skeys[s];
@@ -557,10 +562,9 @@ __global__ __launch_bounds__(kCombineT) void k_fif_combine_cand(const CombineArg
     const int64_t rb = a.runbase[s];
     for (int r = lane; r < nr; r += 32) {
       const int32_t p = rs[r];
-      float t;
-      if (!view_term(a, v, p, a.table[rb + r], t)) continue;
       const int idx = find_sorted(cand, a.R, p);
-      if (idx >= 0) atomicAdd(&acc[idx], fix32(t));
+      float t;
+      if (idx >= 0 && view_term(a, v, p, a.table[rb + r], t)) atomicAdd(&acc[idx], fix32(t));
     }
   }
   __syncthreads();
@@ -783,7 +787,7 @@ void fif_combine(const Index& ix, const FifPlan& P, const uint32_t* table, float
   }
   if (cand_sorted) {
     GIFT_REQUIRE(R <= 1024, "rescore depth must be <= 1024");
-    k_fif_combine_cand<<<(unsigned)P.B, kCombineT, (size_t)R * 8, s>>>(a);
+    k_fif_combine_cand<<<(unsigned)P.B, kCombineT, (size_t)R * 12, s>>>(a);
     GIFT_LAUNCHED("k_fif_combine_cand");
     return;
   }
