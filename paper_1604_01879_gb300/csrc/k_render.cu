@@ -189,20 +189,37 @@ __device__ __forceinline__ f2x f2x_fma(f2x a, f2x b, f2x c) {
   return r;
 }
 
+// Every triangle's corners, centred and scaled, as nine planes of one float per triangle: the blocks of a mesh's
+// images read them in whole lines, instead of three indices and nine gathered coordinates per triangle and band
+__global__ __launch_bounds__(kRenderT) void k_tri_planes(const float* __restrict__ V, const int32_t* __restrict__ T,
+                                                         const int64_t* __restrict__ voff,
+                                                         const int64_t* __restrict__ toff, int M,
+                                                         const float* __restrict__ cs, float* __restrict__ C) {
+  const int64_t total = toff[M], t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= total) return;
+  const int m = find_mesh(toff, M, t);
+  float p[3][3];
+  tri_corners(V + voff[m] * 3, T + t * 3, cs[m * 4], cs[m * 4 + 1], cs[m * 4 + 2], cs[m * 4 + 3], p);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) C[k * total + t] = p[k / 3][k % 3];
+}
+
 // Images by bands in shared memory: a block takes some rows of one (mesh, view) image, draws every triangle of
 // the mesh that meets them with shared-memory minima, and writes the band once, background included. Triangles
 // are set up one per thread and queued; once the queue is filled, the pixels of their boxes are dealt out in
 // units of kUnit horizontal pairs, so triangles of any size load all threads alike, and warps take their next
 // 32 units from a counter. What bounds it is the issue rate of the edge tests (a box has about three pixels per
 // covered one), not memory, so a pair is tested with two-wide FP32 instructions. 64 meshes of 2,208 triangles,
-// 64 views of 224 x 224: 1,549 us (setting up 29%, dealing out 14%, pixels 46%) where a thread per triangle with
-// minima in global memory took 1,865 and a separate fill 405. Two blocks of
+// 64 views of 224 x 224: 1,395 us where a thread per triangle with minima in global memory took 1,865 and a separate
+// fill 405; 1,549 with corners gathered per band and a ten-step search per unit. Units of whole rows, clipped to
+// the columns between the edges, halve the tested pairs but take 1,484: a warp waits for its longest row. Two blocks of
 // 512 threads share an SM, so one's set-up and write-out overlap the other's pixels; the price is that each of
 // an image's bands (three at 224 x 224) sets up the mesh again, up to the first test of its y range.
 constexpr int kBandT = 512, kUnit = 8;
 constexpr int kQueue = 768, kQueueRun = 256;  // the queue is drawn once it holds more than kQueueRun
 constexpr int kBandSmem = 112 * 1024;         // two blocks per SM
 constexpr int kMostBands = 16;
+constexpr int kStep = kQueue / 32;            // a queue's search: 32 parts of kStep, then one of kStep
 struct BandQueue {
   float x[3][kQueue], y[3][kQueue], z[3][kQueue], inv[kQueue];
   int box[kQueue];   // first column and width, 16 bits each
@@ -212,6 +229,7 @@ struct BandQueue {
   int next;
 };
 static_assert(kQueueRun + kBandT <= kQueue, "a round of set-ups fits");
+static_assert(kStep * 32 == kQueue && kStep <= 32, "the search ends in two steps");
 
 // row pitch in shared memory: 16-byte rows, an odd multiple of four apart in the 32 banks, so that pixels below one
 // another fall in different banks (224 is a multiple of 32)
@@ -221,12 +239,10 @@ __host__ __device__ constexpr size_t band_bytes(int rows, int W) {
   return sizeof(BandQueue) + (size_t)(band_pitch(W) + rows + 4) * 4 + (size_t)rows * band_pitch(W) * 4;
 }
 
-__global__ __launch_bounds__(kBandT, 2) void k_render_bands(const float* __restrict__ V, const int32_t* __restrict__ T,
-                                                            const int64_t* __restrict__ voff,
-                                                            const int64_t* __restrict__ toff,
-                                                            const float* __restrict__ cs,
-                                                            const float* __restrict__ frames, int Nv, int H, int W,
-                                                            int band_rows, int bands, float* __restrict__ depth) {
+__global__ __launch_bounds__(kBandT, 2) void k_render_bands(const float* __restrict__ C, const int64_t* __restrict__ toff,
+                                                            int M, const float* __restrict__ frames, int Nv, int H,
+                                                            int W, int band_rows, int bands,
+                                                            float* __restrict__ depth) {
   extern __shared__ __align__(16) uint8_t band_sm[];
   const int pitch = band_pitch(W);
   int* img = reinterpret_cast<int*>(band_sm);                          // [band_rows][pitch], 16-byte rows
@@ -238,16 +254,16 @@ __global__ __launch_bounds__(kBandT, 2) void k_render_bands(const float* __restr
   const int64_t mv = blockIdx.x / bands;
   const int v = (int)(mv % Nv), m = (int)(mv / Nv);
   const int r0 = band * band_rows, r1 = min(H, r0 + band_rows);
-  for (int i = tid; i < (r1 - r0) * pitch; i += kBandT) img[i] = __float_as_int(2.f);
+  const int far = __float_as_int(2.f);
+  for (int i = tid; i < (r1 - r0) * pitch / 4; i += kBandT)  // whole 16-byte pieces
+    reinterpret_cast<int4*>(img)[i] = make_int4(far, far, far, far);
   for (int j = tid; j < W; j += kBandT) pxs[j] = -1.f + (float)(2 * j + 1) / (float)W;
   for (int i = r0 + tid; i < r1; i += kBandT) pys[i - r0] = 1.f - (float)(2 * i + 1) / (float)H;
   const float* fr = frames + v * 9;
   float f[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) f[k] = fr[k];
-  const float c0 = cs[m * 4], c1 = cs[m * 4 + 1], c2 = cs[m * 4 + 2], sc = cs[m * 4 + 3];
-  const float* Vm = V + voff[m] * 3;
-  const int64_t t1 = toff[m + 1];
+  const int64_t t1 = toff[m + 1], plane = toff[M];
   int kept = 0, total = 0;  // queued triangles and their units (the same in every thread)
   if (tid == 0) q.next = 0;
   __syncthreads();
@@ -256,7 +272,8 @@ __global__ __launch_bounds__(kBandT, 2) void k_render_bands(const float* __restr
     int i0 = 0, i1 = -1, j0 = 0, j1 = -1;
     if (t0 + tid < t1) {
       float p[3][3];
-      tri_corners(Vm, T + (t0 + tid) * 3, c0, c1, c2, sc, p);
+#pragma unroll
+      for (int k = 0; k < 9; ++k) p[k / 3][k % 3] = C[k * plane + t0 + tid];
 #pragma unroll
       for (int k = 0; k < 3; ++k) t.y[k] = tri_coord(p[k], f + 3);
       const float ymin = fminf(t.y[0], fminf(t.y[1], t.y[2])), ymax = fmaxf(t.y[0], fmaxf(t.y[1], t.y[2]));
@@ -322,19 +339,27 @@ __global__ __launch_bounds__(kBandT, 2) void k_render_bands(const float* __restr
       if (lane == 0) u = atomicAdd(&q.next, 32);
       u = __shfl_sync(0xffffffffu, u, 0);
       if (u >= total) break;
+      // the triangle of each of the warp's 32 units: u's by two 32-way steps, then the others' by a bit at each
+      // unit that begins a triangle (every queued triangle has one, so 32 of them reach past the last unit)
+      int at = lane * kStep;
+      uint32_t have = __ballot_sync(0xffffffffu, at < kept && q.pre[at] <= u);
+      const int part = (__popc(have) - 1) * kStep;
+      at = part + lane;
+      have = __ballot_sync(0xffffffffu, lane < kStep && at < kept && q.pre[at] <= u);
+      int lo = part + __popc(have) - 1;
+      at = lo + 1 + lane;
+      const int begins = at < kept ? q.pre[at] - u : 32;
+      const uint32_t marks = __reduce_or_sync(0xffffffffu, begins < 32 ? 1u << begins : 0u);
+      lo += __popc(marks & (0xffffffffu >> (31 - lane)));
       u += lane;
       if (u >= total) continue;
-      int lo = 0, hi = kept;  // pre[lo] <= u < pre[hi]
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (q.pre[mid] <= u) lo = mid;
-        else hi = mid;
-      }
       const int box = q.box[lo], rw = q.rows[lo];
       const int wd = box >> 16, jf = box & 0xffff, jl = jf + wd - 1, wp = (wd + 1) >> 1;
       const int first = (u - q.pre[lo]) * kUnit;
       const int n = min(kUnit, wp * (rw >> 16) - first);
-      const int di = first / wp;
+      // first / wp: both are below 2^15 (a band's pixels), so half a pair keeps the quotient off whole numbers by
+      // far more than its error
+      const int di = (int)__fdividef((float)first + 0.5f, (float)wp);
       int i = (rw & 0xffff) + di, j = jf + 2 * (first - di * wp);
       const float x0 = q.x[0][lo], x1 = q.x[1][lo], x2 = q.x[2][lo];
       const float y0 = q.y[0][lo], y1 = q.y[1][lo], y2 = q.y[2][lo];
@@ -499,8 +524,13 @@ void render_views(const float* V, const int32_t* T, const std::vector<int64_t>& 
   int rows = 0, bands = 0;
   if (band_plan(images, h_toff[M], M, H, W, rows, bands)) {
     GIFT_CUDA(cudaFuncSetAttribute(k_render_bands, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmem));
-    k_render_bands<<<(unsigned)(images * bands), kBandT, band_bytes(rows, W), s>>>(V, T, voff, toff, cs, d_fr, Nv, H, W,
-                                                                                  rows, bands, depth);
+    float* corners = sc.get<float>((size_t)h_toff[M] * 9);
+    if (h_toff[M] > 0) {
+      k_tri_planes<<<(unsigned)cdiv(h_toff[M], kRenderT), kRenderT, 0, s>>>(V, T, voff, toff, M, cs, corners);
+      GIFT_LAUNCHED("k_tri_planes");
+    }
+    k_render_bands<<<(unsigned)(images * bands), kBandT, band_bytes(rows, W), s>>>(corners, toff, M, d_fr, Nv, H, W, rows,
+                                                                                  bands, depth);
     GIFT_LAUNCHED("k_render_bands");
     return;
   }
