@@ -212,9 +212,9 @@ __global__ __launch_bounds__(kRenderT) void k_tri_planes(const float* __restrict
 // covered one), not memory, so a pair is tested with two-wide FP32 instructions. 64 meshes of 2,208 triangles,
 // 64 views of 224 x 224: 1,395 us where a thread per triangle with minima in global memory took 1,865 and a separate
 // fill 405; 1,549 with corners gathered per band and a ten-step search per unit. Units of whole rows, clipped to
-// the columns between the edges, halve the tested pairs but take 1,484: a warp waits for its longest row. Two blocks of
-// 512 threads share an SM, so one's set-up and write-out overlap the other's pixels; the price is that each of
-// an image's bands (three at 224 x 224) sets up the mesh again, up to the first test of its y range.
+// the columns between the edges, halve the tested pairs but take 1,484: a warp waits for its longest row. Two
+// blocks of 512 threads share an SM, so one's set-up and write-out overlap the other's pixels; the price is that
+// each of an image's bands (three at 224 x 224) sets up the mesh again, up to the first test of its y range.
 constexpr int kBandT = 512, kUnit = 8;
 constexpr int kQueue = 768, kQueueRun = 256;  // the queue is drawn once it holds more than kQueueRun
 constexpr int kBandSmem = 112 * 1024;         // two blocks per SM
