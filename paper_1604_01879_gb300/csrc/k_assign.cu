@@ -30,6 +30,8 @@ constexpr unsigned kFull = 0xffffffffu;
 // coarse scores kept per row and chunk of tn codewords: the best 16, or all 32 (which spares the epilogue its
 // insertions, most of a small item's time)
 __host__ __device__ constexpr int kept_scores(int tn) { return tn == 32 ? 32 : 16; }
+constexpr int kMaxParts = 8;   // parts of the reduction
+constexpr int kPartsK = 1024;  // codewords of a vocabulary whose reduction is taken in parts
 
 // TN_: codewords per chunk. 256 where the (row tile, chunk) items fill the SMs; with few rows 64 or 32, whose more
 // items run on more SMs at once with more stages in flight: an item's time is a chain of D / 64 k-blocks, 1.7 us each
@@ -46,21 +48,28 @@ struct AssignPolicy {
   int K;
   int nch;            // codeword chunks of TN
   int nkb;
+  int parts = 1;      // parts of the reduction, each an item of its own (kAll only)
   const float* half_sq;
-  float* cval;        // [n, nch, kT] best coarse scores of each chunk, descending
+  float* cval;        // [n, nch, kT] best coarse scores of each chunk, descending; parts > 1: [parts, n, nch, kT] products
   int32_t* cidx;      // [n, nch, kT] their codewords (0x7fffffff: none)
   struct Item {
     int64_t r0;
     int nr;
     int c;
+    int part;
   };
   struct Ctx {
     float val[kT];
     int idx[kT];
   };
-  __device__ __forceinline__ int64_t total() const { return cdiv(n, tc::kTM) * nch; }
+  __device__ __forceinline__ int64_t total() const { return cdiv(n, tc::kTM) * nch * (kAll ? parts : 1); }
   __device__ __forceinline__ Item decode(int64_t item) const {
     Item it;
+    it.part = 0;
+    if constexpr (kAll) {
+      it.part = (int)(item % parts);
+      item /= parts;
+    }
     it.r0 = (item / nch) * tc::kTM;
     it.c = (int)(item % nch);
     it.nr = (int)min((int64_t)tc::kTM, n - it.r0);
@@ -69,8 +78,8 @@ struct AssignPolicy {
   __device__ __forceinline__ int nchunks(const Item&) const { return 1; }
   __device__ __forceinline__ void chunk(const Item& it, int, int& br, int& kb0, int& kb1) const {
     br = it.c * TN;
-    kb0 = 0;
-    kb1 = nkb;
+    kb0 = kAll ? nkb * it.part / parts : 0;
+    kb1 = kAll ? nkb * (it.part + 1) / parts : nkb;
   }
   __device__ __forceinline__ int a_row(const Item& it) const { return (int)it.r0; }
   __device__ __forceinline__ void epi_begin(const Item&, Ctx& x, int, int, uint8_t*) const {
@@ -95,7 +104,7 @@ struct AssignPolicy {
       tc::tmem_wait_ld();
 #pragma unroll
       for (int j = 0; j < 32; ++j) {
-        x.val[j] = __uint_as_float(r[j]) - hs[j];
+        x.val[j] = __uint_as_float(r[j]) - (parts > 1 ? 0.f : hs[j]);
         x.idx[j] = c * TN + j < K ? c * TN + j : 0x7fffffff;
       }
       __syncwarp();
@@ -130,7 +139,16 @@ struct AssignPolicy {
   }
   __device__ __forceinline__ void epi_end(const Item& it, Ctx& x, int m, uint8_t*) const {
     if (m >= it.nr) return;
-    const int64_t o = ((it.r0 + m) * nch + it.c) * kT;
+    const int64_t o = (((kAll ? it.part * n : 0) + it.r0 + m) * nch + it.c) * kT;
+    if constexpr (kAll) {
+#pragma unroll
+      for (int t = 0; t < kT; t += 4) {
+        *reinterpret_cast<float4*>(cval + o + t) = make_float4(x.val[t], x.val[t + 1], x.val[t + 2], x.val[t + 3]);
+        if (parts == 1)
+          *reinterpret_cast<int4*>(cidx + o + t) = make_int4(x.idx[t], x.idx[t + 1], x.idx[t + 2], x.idx[t + 3]);
+      }
+      return;
+    }
 #pragma unroll
     for (int t = 0; t < kT; ++t) {
       cval[o + t] = x.val[t];
@@ -334,9 +352,12 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
                                                        const float* __restrict__ cval,
                                                        const int32_t* __restrict__ cidx, int nch, int tn, int kT,
                                                        const float* __restrict__ x_inv, float bmax_host,
-                                                       const float* __restrict__ bmax_dev,
+                                                       const float* __restrict__ bmax_dev, int parts,
+                                                       const float* __restrict__ half_sq,
                                                        int32_t* __restrict__ codes) {
   __shared__ DfPart part[8];
+  __shared__ float sval[WPR > 1 ? kPartsK : 1];
+  __shared__ int32_t sidx[WPR > 1 ? kPartsK : 1];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = w % WPR;
   const int64_t r = (int64_t)blockIdx.x * (8 / WPR) + w / WPR;
   if (r >= n) return;  // (with a block per row every warp decides everything alike)
@@ -344,6 +365,23 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
   const int tot = nch * kT;
   const float* v = cval + r * tot;
   const int32_t* id = cidx + r * tot;
+  if constexpr (WPR > 1) {
+    if (parts > 1) {  // the scores of all codewords (tot <= kPartsK), from their products' parts in order
+      for (int k = threadIdx.x; k < tot; k += 256) {
+        float p[kMaxParts];
+#pragma unroll
+        for (int i = 0; i < kMaxParts; ++i) p[i] = i < parts ? v[i * n * tot + k] : 0.f;
+        float x = p[0];
+#pragma unroll
+        for (int i = 1; i < kMaxParts; ++i) x += p[i];
+        sval[k] = k < K ? x - half_sq[k] : -INFINITY;
+        sidx[k] = k < K ? k : 0x7fffffff;
+      }
+      __syncthreads();
+      v = sval;
+      id = sidx;
+    }
+  }
   // the ma-th best coarse score over all chunks
   float thr = INFINITY;
   int tp = -1, found = 0;
@@ -612,7 +650,14 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
     if (pair) tn = 128;  // chunks of kept scores
   }
   const int nch = (int)cdiv(K, tn), kT = kept_scores(tn);
-  float* cval = sc.get<float>((size_t)chunk * nch * kT);
+  // Few items: their chains of k-blocks in parts, as long as a part keeps four k-blocks and finds a free SM; the
+  // refine's block of a row adds the parts up (108 rows, D = 4096, K = 512: 16 items in 44 us, in eight parts 10;
+  // the refine, which then reads its scores from shared memory, 30 and 27)
+  const int nkb = (int)cdiv(D, tc::kTK);
+  int cuts = 1;
+  if (tn == 32 && n <= chunk && n < 8 * sms && nch * tn <= kPartsK)
+    cuts = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)kMaxParts, nkb / 4, sms / (row_tiles * nch)}));
+  float* cval = sc.get<float>((size_t)chunk * nch * kT * cuts);
   int32_t* cidx = sc.get<int32_t>((size_t)chunk * nch * kT);
   float* inv = nullptr;
   if (!x_inv) {
@@ -627,12 +672,13 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
     if (!parts) split_rows_bf16(X + r0 * D, m, D, hi, lo, s);
     const CUtensorMap tA = make_tmap_bf16(hi, rows_alloc, D, tc::kTM);
     const CUtensorMap tA2 = make_tmap_bf16(lo, rows_alloc, D, tc::kTM);
-    const int grid = (int)std::min<int64_t>(sms, cdiv(m, tc::kTM) * nch);
+    const int grid = (int)std::min<int64_t>(sms, cdiv(m, tc::kTM) * nch * cuts);
     auto coarse = [&](auto p, auto launch) {
       p.n = m;
       p.K = K;
       p.nch = nch;
-      p.nkb = (int)cdiv(D, tc::kTK);
+      p.nkb = nkb;
+      p.parts = cuts;
       p.half_sq = ix.cb_half_sq;
       p.cval = cval;
       p.cidx = cidx;
@@ -653,10 +699,12 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
     }
     if (m >= 8 * sms)
       k_assign_refine<1><<<(unsigned)cdiv(m, 8), 256, 0, s>>>(X + r0 * D, m, D, ix.codebook, K, ma, cval, cidx, nch,
-                                                              tn, kT, x_inv + r0, ix.cb_max_norm, cb_max, codes + r0 * ma);
+                                                              tn, kT, x_inv + r0, ix.cb_max_norm, cb_max, 1, nullptr,
+                                                              codes + r0 * ma);
     else
       k_assign_refine<8><<<(unsigned)m, 256, 0, s>>>(X + r0 * D, m, D, ix.codebook, K, ma, cval, cidx, nch, tn, kT,
-                                                     x_inv + r0, ix.cb_max_norm, cb_max, codes + r0 * ma);
+                                                     x_inv + r0, ix.cb_max_norm, cb_max, cuts, ix.cb_half_sq,
+                                                     codes + r0 * ma);
     GIFT_LAUNCHED("k_assign_refine");
   }
 }

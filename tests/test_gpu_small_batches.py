@@ -23,6 +23,23 @@ def test_codes_at_tile_edges(gpu_lib, K, n, ma):
     assert np.array_equal(got, np.argsort(dist, axis=1, kind="stable")[:, :ma])
 
 
+# few rows: the reduction in one to eight parts (D = 256 is one, 512 two, 4096 eight; 1025 codewords keep one)
+@pytest.mark.parametrize("K", [1, 31, 32, 33, 512, 1000, 1024, 1025])
+@pytest.mark.parametrize("n,ma,D", [(1, 1, 256), (3, 2, 512), (54, 2, 4096), (127, 3, 1024), (128, 1, 1104),
+                                    (129, 2, 2048), (1215, 2, 528)])
+def test_codes_from_parts_of_the_reduction(gpu_lib, K, n, ma, D):
+    import torch
+    g = np.random.default_rng(K * 17 + n)
+    ma = min(ma, K)
+    cb = g.standard_normal((K, D)).astype(np.float32)
+    x = (cb[g.integers(0, K, n)] + 0.7 * g.standard_normal((n, D))).astype(np.float32)
+    ix = gpu_lib.Index(torch.from_numpy(x[:1].copy()).cuda(), torch.from_numpy(cb).cuda(), 1, 1, K, keep_exact=False)
+    got = ix.assign(torch.from_numpy(x).cuda(), ma).cpu().numpy()
+    cb64, x64 = cb.astype(np.float64), x.astype(np.float64)
+    dist = (cb64 ** 2).sum(1)[None] - 2 * x64 @ cb64.T  # less |x|^2; gaps are of order D, the rounding 1e-12
+    assert np.array_equal(got, np.argsort(dist, axis=1, kind="stable")[:, :ma])
+
+
 # one list (K = 1) makes every (slot, entry) tile of the FP32 scan: entries and slots at and around 64
 @pytest.mark.parametrize("D", [16, 32, 48, 80])
 @pytest.mark.parametrize("N,nv,vq", [(1, 1, 1), (9, 7, 64), (13, 5, 65), (16, 8, 3)])
