@@ -355,6 +355,7 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
                                                        const float* __restrict__ bmax_dev, int parts,
                                                        const float* __restrict__ half_sq,
                                                        int32_t* __restrict__ codes) {
+  dep_begin();
   __shared__ DfPart part[8];
   __shared__ float sval[WPR > 1 ? kPartsK : 1];
   __shared__ int32_t sidx[WPR > 1 ? kPartsK : 1];
@@ -698,13 +699,11 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
       kc->assign_rows += m;
     }
     if (m >= 8 * sms)
-      k_assign_refine<1><<<(unsigned)cdiv(m, 8), 256, 0, s>>>(X + r0 * D, m, D, ix.codebook, K, ma, cval, cidx, nch,
-                                                              tn, kT, x_inv + r0, ix.cb_max_norm, cb_max, 1, nullptr,
-                                                              codes + r0 * ma);
+      launch_dep(k_assign_refine<1>, dim3((unsigned)cdiv(m, 8)), dim3(256), 0, s, X + r0 * D, m, D, ix.codebook, K, ma,
+                 cval, cidx, nch, tn, kT, x_inv + r0, ix.cb_max_norm, cb_max, 1, nullptr, codes + r0 * ma);
     else
-      k_assign_refine<8><<<(unsigned)m, 256, 0, s>>>(X + r0 * D, m, D, ix.codebook, K, ma, cval, cidx, nch, tn, kT,
-                                                     x_inv + r0, ix.cb_max_norm, cb_max, cuts, ix.cb_half_sq,
-                                                     codes + r0 * ma);
+      launch_dep(k_assign_refine<8>, dim3((unsigned)m), dim3(256), 0, s, X + r0 * D, m, D, ix.codebook, K, ma, cval,
+                 cidx, nch, tn, kT, x_inv + r0, ix.cb_max_norm, cb_max, cuts, ix.cb_half_sq, codes + r0 * ma);
     GIFT_LAUNCHED("k_assign_refine");
   }
 }

@@ -93,6 +93,7 @@ __global__ __launch_bounds__(kPlanT) void k_plan_work(const int64_t* __restrict_
                                                       const int64_t* __restrict__ list_off, int K,
                                                       const WorkSpecs specs, int64_t fold,
                                                       int64_t* __restrict__ woff) {
+  dep_begin();
   __shared__ int64_t wsum[kPlanT / 32 + 1];
   __shared__ unsigned s_items;
   __shared__ int s_most;
@@ -182,6 +183,7 @@ __global__ __launch_bounds__(kPlanT) void k_slots_small(const int32_t* __restric
                                                         int32_t* __restrict__ slot_view,
                                                         int32_t* __restrict__ view_slot,
                                                         int64_t* __restrict__ runbase) {
+  dep_begin();
   __shared__ unsigned long long key[kSmallSlots];
   __shared__ uint32_t id[kSmallSlots];
   __shared__ int64_t wsum[kPlanT / 32 + 1];
@@ -268,6 +270,7 @@ struct ScanArgs {
 constexpr int kScanBK = 32;
 template <bool RESCORE>
 __global__ __launch_bounds__(256) void k_fif_scan(const ScanArgs a) {
+  dep_begin();
   __shared__ __align__(16) float stage[2 * 2 * kScanBK * kScanTS];  // Q and F, two buffers; then the cosines
   __shared__ int32_t e_run[kScanTE], e_shape[kScanTE];
   __shared__ float e_scale[kScanTE];
@@ -499,6 +502,7 @@ __device__ __forceinline__ bool view_term(const CombineArgs& a, int64_t v, int32
 // reached through several of the view's lists counts once, with the largest
 // maximum, added by the lowest assignment that reaches it.
 __global__ __launch_bounds__(kCombineT) void k_fif_combine_views(const CombineArgs a) {
+  dep_begin();
   const int64_t item = ((int64_t)blockIdx.x * kCombineT + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (item >= a.nv * a.ma) return;
@@ -532,6 +536,7 @@ __global__ __launch_bounds__(kCombineT) void k_fif_combine_views(const CombineAr
 // fixed-point sums -> scores (1/|V(x_q)|) sum (Eq. 4), n = row width
 __global__ void k_unfix_rows(const unsigned long long* __restrict__ acc, const int32_t* __restrict__ qoff, int B,
                              int64_t n, float* __restrict__ out) {
+  dep_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (int64_t)B * n) return;
   const int q = (int)(i / n);
@@ -544,6 +549,7 @@ __global__ void k_unfix_rows(const unsigned long long* __restrict__ acc, const i
 // The candidates are searched in shared memory: in global memory every run's search was
 // eight dependent reads (1,000 queries of 64 views, R = 200: 200 us, 178 now).
 __global__ __launch_bounds__(kCombineT) void k_fif_combine_cand(const CombineArgs a) {
+  dep_begin();
   extern __shared__ unsigned long long acc[];  // [R] sums, then int32 candidates [R]
   int32_t* cand = reinterpret_cast<int32_t*>(acc + a.R);
   const int q = blockIdx.x;
@@ -582,6 +588,7 @@ __global__ __launch_bounds__(kCombineT) void k_fif_combine_cand(const CombineArg
 // directly).
 constexpr int kCombineWarps = kCombineT / 32;
 __global__ __launch_bounds__(kCombineT) void k_fif_combine_ma_cand(const CombineArgs a) {
+  dep_begin();
   extern __shared__ unsigned long long acc[];  // [R] sums, then int32 cand[R], then uint32 [warps][R] view maxima
   const int q = blockIdx.x / a.groups, g = blockIdx.x % a.groups, R = a.R;
   int32_t* cs = reinterpret_cast<int32_t*>(acc + R);
@@ -647,6 +654,7 @@ __global__ __launch_bounds__(kCombineT) void k_fif_combine_ma_cand(const Combine
 
 // zero the first *n cells (n read on the device)
 __global__ void k_zero_cells(uint32_t* __restrict__ t, const int64_t* __restrict__ n_dev) {
+  dep_begin();
   const int64_t n = *n_dev;
   const int64_t n4 = n >> 2;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -660,7 +668,7 @@ __global__ void k_zero_cells(uint32_t* __restrict__ t, const int64_t* __restrict
 
 void fif_zero_table(const FifPlan& P, uint32_t* table, cudaStream_t s) {
   if (P.nslots <= 0) return;
-  k_zero_cells<<<1216, 256, 0, s>>>(table, P.runbase + P.nslots);  // 8 blocks per SM of a GB300
+  launch_dep(k_zero_cells, dim3(1216), dim3(256), 0, s, table, P.runbase + P.nslots);  // 8 blocks per SM of a GB300
   GIFT_LAUNCHED("k_zero_cells");
 }
 
@@ -668,7 +676,7 @@ int64_t* plan_work(const Index& ix, const FifPlan& P, const WorkSpecs& specs, in
                    cudaStream_t s) {
   const int K = ix.prm.n_codewords;
   int64_t* woff = sc.get<int64_t>((size_t)specs.n * (K + 1));
-  k_plan_work<<<(unsigned)specs.n, kPlanT, 0, s>>>(P.boff, ix.list_off, K, specs, fold, woff);
+  launch_dep(k_plan_work, dim3((unsigned)specs.n), dim3(kPlanT), 0, s, P.boff, ix.list_off, K, specs, fold, woff);
   GIFT_LAUNCHED("k_plan_work");
   return woff;
 }
@@ -683,8 +691,8 @@ void fif_plan(const Index& ix, FifPlan& P, Scratch& sc, cudaStream_t s) {
   P.view_slot = sc.get<int32_t>(n);
   P.runbase = sc.get<int64_t>(n + 1);
   if (n <= kSmallSlots) {
-    k_slots_small<<<1, kPlanT, 0, s>>>(P.q_code, (int)n, P.ma, K, ix.nruns, P.skeys, P.boff, P.slot_view, P.view_slot,
-                                       P.runbase);
+    launch_dep(k_slots_small, dim3(1), dim3(kPlanT), 0, s, P.q_code, (int)n, P.ma, K, ix.nruns, P.skeys, P.boff,
+               P.slot_view, P.view_slot, P.runbase);
     GIFT_LAUNCHED("k_slots_small");
   } else {
     int32_t* perm = sc.get<int32_t>(n);
@@ -733,12 +741,12 @@ void fif_scan(const Index& ix, const FifPlan& P, uint32_t* table, bool rescore,
   if (rescore) {
     a.feat = ix.master;
     a.scale = ix.row_inv;
-    k_fif_scan<true><<<grid, 256, 0, s>>>(a);
+    launch_dep(k_fif_scan<true>, dim3(grid), dim3(256), 0, s, a);
   } else {
     GIFT_REQUIRE(ix.prm.storage == GIFT_F32, "reduced stores are scanned on the tensor cores");
     a.feat = ix.list_feat;
     a.scale = ix.list_scale;
-    k_fif_scan<false><<<grid, 256, 0, s>>>(a);
+    launch_dep(k_fif_scan<false>, dim3(grid), dim3(256), 0, s, a);
   }
   GIFT_LAUNCHED("k_fif_scan");
 }
@@ -779,15 +787,16 @@ void fif_combine(const Index& ix, const FifPlan& P, const uint32_t* table, float
     GIFT_CUDA(cudaMemsetAsync(a.acc, 0, (size_t)P.B * R * 8, s));
     const size_t smem = (size_t)R * (8 + 4 + 4 * kCombineWarps);
     GIFT_CUDA(cudaFuncSetAttribute(k_fif_combine_ma_cand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_fif_combine_ma_cand<<<(unsigned)(P.B * a.groups), kCombineT, smem, s>>>(a);
+    launch_dep(k_fif_combine_ma_cand, dim3((unsigned)(P.B * a.groups)), dim3(kCombineT), smem, s, a);
     GIFT_LAUNCHED("k_fif_combine_ma_cand");
-    k_unfix_rows<<<(unsigned)cdiv((int64_t)P.B * R, 256), 256, 0, s>>>(a.acc, P.qoff, P.B, R, cand_score);
+    launch_dep(k_unfix_rows, dim3((unsigned)cdiv((int64_t)P.B * R, 256)), dim3(256), 0, s, a.acc, P.qoff, P.B, R,
+               cand_score);
     GIFT_LAUNCHED("k_unfix_rows");
     return;
   }
   if (cand_sorted) {
     GIFT_REQUIRE(R <= 1024, "rescore depth must be <= 1024");
-    k_fif_combine_cand<<<(unsigned)P.B, kCombineT, (size_t)R * 12, s>>>(a);
+    launch_dep(k_fif_combine_cand, dim3((unsigned)P.B), dim3(kCombineT), (size_t)R * 12, s, a);
     GIFT_LAUNCHED("k_fif_combine_cand");
     return;
   }
@@ -796,10 +805,10 @@ void fif_combine(const Index& ix, const FifPlan& P, const uint32_t* table, float
   GIFT_CUDA(cudaMemsetAsync(a.acc, 0, (size_t)n * 8, s));
   const int64_t warps = P.nv * P.ma;
   if (warps > 0) {
-    k_fif_combine_views<<<(unsigned)cdiv(warps * 32, (int64_t)kCombineT), kCombineT, 0, s>>>(a);
+    launch_dep(k_fif_combine_views, dim3((unsigned)cdiv(warps * 32, (int64_t)kCombineT)), dim3(kCombineT), 0, s, a);
     GIFT_LAUNCHED("k_fif_combine_views");
   }
-  k_unfix_rows<<<(unsigned)cdiv(n, 256), 256, 0, s>>>(a.acc, P.qoff, P.B, a.N, S_dense);
+  launch_dep(k_unfix_rows, dim3((unsigned)cdiv(n, 256)), dim3(256), 0, s, a.acc, P.qoff, P.B, a.N, S_dense);
   GIFT_LAUNCHED("k_unfix_rows");
 }
 

@@ -437,6 +437,7 @@ __global__ __launch_bounds__(kSlotT) void k_slot_rows(const float* __restrict__ 
                                                       const int32_t* __restrict__ view_slot, int ma, int D,
                                                       __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                                                       uint32_t* __restrict__ out8, float* __restrict__ scale) {
+  dep_begin();
   __shared__ float red[kSlotT / 32];
   const int64_t v = blockIdx.x;
   const float4* src = reinterpret_cast<const float4*>(q + v * D);
@@ -557,6 +558,7 @@ __global__ __launch_bounds__(256) void k_resc_flags(const ListSched ls, const Cl
                                                     const int32_t* __restrict__ cand, int R,
                                                     uint8_t* __restrict__ masks,
                                                     unsigned long long* __restrict__ stats) {
+  dep_begin();
   __shared__ uint8_t s_hit[8];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const ClassItem ci = class_item(cw, ls.K, first_class, (int64_t)blockIdx.x * 8 + w);
@@ -621,6 +623,7 @@ __global__ __launch_bounds__(kCompactT) void k_resc_compact(const ListSched ls, 
                                                             const uint8_t* __restrict__ masks, int64_t nmasks,
                                                             ListItem* __restrict__ items,
                                                             int64_t* __restrict__ base) {
+  dep_begin();
   __shared__ int part[kCompactT / 32], own[kCompactT / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int64_t m0 = (int64_t)blockIdx.x * (kCompactT / 8), g = (int64_t)blockIdx.x * kCompactT + tid;
@@ -702,9 +705,8 @@ void fif_rescore_stats(const Index& ix, const FifPlan& P, const int32_t* cand_so
   cw.woff[kClasses - 1] = plan_work(ix, P, specs, 0, sc, s);
   const int64_t upper = std::max<int64_t>(P.upper_items, 1);
   for (int c = 0; c < kClasses; ++c) cw.woff[c] = cw.woff[kClasses - 1];  // (only the last class's items are counted)
-  k_resc_flags<<<(unsigned)cdiv(upper, 8), 256, 0, s>>>(list_sched(ix, P, nullptr, 0), cw, kClasses - 1, P.slot_view,
-                                                        P.vquery, ix.entry_run, ix.list_shape, cand_sorted, R, nullptr,
-                                                        P.stats);
+  launch_dep(k_resc_flags, dim3((unsigned)cdiv(upper, 8)), dim3(256), 0, s, list_sched(ix, P, nullptr, 0), cw,
+             kClasses - 1, P.slot_view, P.vquery, ix.entry_run, ix.list_shape, cand_sorted, R, nullptr, P.stats);
   GIFT_LAUNCHED("k_resc_flags");
 }
 
@@ -735,8 +737,8 @@ void fif_scan_tc(const Index& ix, const FifPlan& P, uint32_t* table, bool rescor
     }
     if (!fp8 || parts) qhi = sc.get<__nv_bfloat16>((size_t)qrows * D);
     if (parts) qlo = sc.get<__nv_bfloat16>((size_t)qrows * D);
-    k_slot_rows<<<(unsigned)P.nv, kSlotT, 0, s>>>(P.q, P.view_slot, P.ma, D, qhi, qlo, reinterpret_cast<uint32_t*>(q8),
-                                                  q8s);
+    launch_dep(k_slot_rows, dim3((unsigned)P.nv), dim3(kSlotT), 0, s, P.q, P.view_slot, P.ma, D, qhi, qlo,
+               reinterpret_cast<uint32_t*>(q8), q8s);
     GIFT_LAUNCHED("k_slot_rows");
     P.slot_hi = qhi;
     P.slot_lo = qlo;
@@ -837,10 +839,11 @@ void fif_scan_tc(const Index& ix, const FifPlan& P, uint32_t* table, bool rescor
     ListItem* items = sc.get<ListItem>(upper);
     int64_t* base = sc.get<int64_t>(kClasses + 1);
     const ListSched ls = list_sched(ix, P, nullptr, (int)cdiv((int64_t)D, (int64_t)64));
-    k_resc_flags<<<(unsigned)nmasks, 256, 0, s>>>(ls, cw, 0, P.slot_view, P.vquery, ix.entry_run, ix.list_shape,
-                                                  cand_sorted, R, masks, P.stats);
+    launch_dep(k_resc_flags, dim3((unsigned)nmasks), dim3(256), 0, s, ls, cw, 0, P.slot_view, P.vquery, ix.entry_run,
+               ix.list_shape, cand_sorted, R, masks, P.stats);
     GIFT_LAUNCHED("k_resc_flags");
-    k_resc_compact<<<(unsigned)(8 * nmasks / kCompactT + 1), kCompactT, 0, s>>>(ls, cw, masks, nmasks, items, base);
+    launch_dep(k_resc_compact, dim3((unsigned)(8 * nmasks / kCompactT + 1)), dim3(kCompactT), 0, s, ls, cw, masks,
+               nmasks, items, base);
     GIFT_LAUNCHED("k_resc_compact");
     const CUtensorMap tA = make_tmap_bf16(bhi, ix.list_rows_alloc, D, tc::kTM);
     const CUtensorMap tA2 = make_tmap_bf16(ix.list_lo, ix.list_rows_alloc, D, tc::kTM);

@@ -36,6 +36,7 @@ struct ScoreRow {
 
 __global__ __launch_bounds__(1024) void k_topk(const float* __restrict__ scores, int64_t n, int k,
                                                int32_t* __restrict__ ids_out, float* __restrict__ val_out) {
+  dep_begin();
   __shared__ sel::Smem sm;
   const int64_t b = blockIdx.x;
   const int take = sel::select(sm, ScoreRow{scores + b * n}, n, n, k);
@@ -110,6 +111,7 @@ __global__ __launch_bounds__(1024) void k_sort_candidates(const int32_t* __restr
                                                           const float* __restrict__ scores, int r, int k,
                                                           int32_t* __restrict__ ids_out,
                                                           float* __restrict__ scores_out, int mode_ids) {
+  dep_begin();
   __shared__ unsigned long long s_key[kMaxK];
   __shared__ uint32_t s_id[kMaxK];
   const int64_t b = blockIdx.x;
@@ -146,7 +148,7 @@ void topk_rows_f32(const float* scores, int32_t B, int64_t n, int32_t k, int32_t
   if (B <= 0 || k <= 0) return;
   GIFT_REQUIRE(k <= kMaxK, "top-k is limited to 1024");
   GIFT_REQUIRE(n < (int64_t)INT32_MAX, "row too long for top-k");
-  k_topk<<<(unsigned)B, row_threads(n, B), 0, s>>>(scores, n, k, ids_out, val_out);
+  launch_dep(k_topk, dim3((unsigned)B), dim3(row_threads(n, B)), 0, s, scores, n, k, ids_out, val_out);
   GIFT_LAUNCHED("k_topk");
 }
 
@@ -164,14 +166,15 @@ void sort_candidates(const int32_t* ids, const float* scores, int32_t B, int32_t
                      int32_t* ids_out, float* scores_out, cudaStream_t s) {
   if (B <= 0 || k <= 0) return;
   GIFT_REQUIRE(r <= kMaxK, "candidate rows are limited to 1024");
-  k_sort_candidates<<<(unsigned)B, row_threads(r, B), 0, s>>>(ids, scores, r, k, ids_out, scores_out, 0);
+  launch_dep(k_sort_candidates, dim3((unsigned)B), dim3(row_threads(r, B)), 0, s, ids, scores, r, k, ids_out,
+             scores_out, 0);
   GIFT_LAUNCHED("k_sort_candidates");
 }
 
 void sort_ids_rows(const int32_t* ids, int32_t B, int32_t r, int32_t* out, cudaStream_t s) {
   if (B <= 0 || r <= 0) return;
   GIFT_REQUIRE(r <= kMaxK, "candidate rows are limited to 1024");
-  k_sort_candidates<<<(unsigned)B, row_threads(r, B), 0, s>>>(ids, nullptr, r, r, out, nullptr, 1);
+  launch_dep(k_sort_candidates, dim3((unsigned)B), dim3(row_threads(r, B)), 0, s, ids, nullptr, r, r, out, nullptr, 1);
   GIFT_LAUNCHED("k_sort_ids");
 }
 

@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(engine_threads<P>::value, 1)
   constexpr bool kGen = gen_a_of<P>::value;
   constexpr int kGenWarps = kGen ? gen_warps_of<P>::value : 1;
   static_assert(kGenWarps >= 1 && kGenWarps <= 4, "one to four generator warps");
+  dep_begin();
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* tiles = smem;
@@ -491,7 +492,7 @@ void launch_engine(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap
                    const P& p, int* err, int grid, cudaStream_t s) {
   using L = EngineLayout<P>;
   GIFT_CUDA(cudaFuncSetAttribute(tc_engine<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kSmem));
-  tc_engine<P><<<grid, engine_threads<P>::value, L::kSmem, s>>>(a, b, a2, b2, p, err);
+  launch_dep(tc_engine<P>, dim3(grid), dim3(engine_threads<P>::value), L::kSmem, s, a, b, a2, b2, p, err);
   GIFT_LAUNCHED("tc_engine");
 }
 
