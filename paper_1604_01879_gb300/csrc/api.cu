@@ -206,6 +206,7 @@ __global__ void k_list_runs(const int64_t* __restrict__ list_off, const int64_t*
 
 // out = raise * max_k ||b_k||
 __global__ void k_cb_maxnorm(const float* __restrict__ half_sq, int K, float* __restrict__ out, float raise) {
+  dep_begin();
   float m = 0.f;
   for (int k = threadIdx.x; k < K; k += blockDim.x) m = fmaxf(m, half_sq[k]);
 #pragma unroll
@@ -235,7 +236,7 @@ const float* prepare_codebook_async(Index& ix, Scratch& sc, cudaStream_t s) {
   launch_half_sq_norm(ix.codebook, K, D, ix.cb_half_sq, s);
   split_rows_bf16(ix.codebook, K, D, ix.cb_hi, ix.cb_lo, s);
   float* d_cbmax = sc.get<float>(1);
-  k_cb_maxnorm<<<1, 1024, 0, s>>>(ix.cb_half_sq, K, d_cbmax, 1.0001f);
+  launch_dep(k_cb_maxnorm, dim3(1), dim3(1024), 0, s, ix.cb_half_sq, K, d_cbmax, 1.0001f);
   GIFT_LAUNCHED("k_cb_maxnorm");
   return d_cbmax;
 }

@@ -557,6 +557,7 @@ __global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__
 // hi = bf16(x), lo = bf16(x - hi), row-major [n, D]
 __global__ void k_split_rows(const float* __restrict__ X, int64_t n, int D, __nv_bfloat16* __restrict__ hi,
                              __nv_bfloat16* __restrict__ lo) {
+  dep_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;  // index of a float4
   if (i >= n * (D / 4)) return;
   const float4 v = reinterpret_cast<const float4*>(X)[i];
@@ -613,7 +614,7 @@ __global__ __launch_bounds__(256) void k_split_norm(const float* __restrict__ X,
 void split_rows_bf16(const float* X, int64_t n, int D, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t s) {
   if (n <= 0) return;
   const int64_t n4 = n * (D / 4);
-  k_split_rows<<<(unsigned)cdiv(n4, 256), 256, 0, s>>>(X, n, D, hi, lo);
+  launch_dep(k_split_rows, dim3((unsigned)cdiv(n4, 256)), dim3(256), 0, s, X, n, D, hi, lo);
   GIFT_LAUNCHED("k_split_rows");
 }
 

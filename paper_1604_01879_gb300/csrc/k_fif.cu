@@ -36,6 +36,7 @@ __global__ void k_slot_setup(const int32_t* __restrict__ perm, int64_t nslots, i
                              const int32_t* __restrict__ skeys, const int32_t* __restrict__ nruns,
                              int32_t* __restrict__ slot_view, int32_t* __restrict__ view_slot,
                              int64_t* __restrict__ run_cnt) {
+  dep_begin();
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s == nslots) run_cnt[s] = 0;  // so that the scan's last element is the table size
   if (s >= nslots) return;
@@ -699,8 +700,8 @@ void fif_plan(const Index& ix, FifPlan& P, Scratch& sc, cudaStream_t s) {
     stable_sort_by_key(P.q_code, n, K, perm, P.skeys, sc, s);
     bin_offsets(P.skeys, n, K, P.boff, s);
     int64_t* run_cnt = sc.get<int64_t>(n + 1);
-    k_slot_setup<<<(unsigned)cdiv(n + 1, 256), 256, 0, s>>>(perm, n, P.ma, P.skeys, ix.nruns, P.slot_view,
-                                                              P.view_slot, run_cnt);
+    launch_dep(k_slot_setup, dim3((unsigned)cdiv(n + 1, 256)), dim3(256), 0, s, perm, n, P.ma, P.skeys, ix.nruns,
+               P.slot_view, P.view_slot, run_cnt);
     GIFT_LAUNCHED("k_slot_setup");
     scan_exclusive_i64(run_cnt, P.runbase, n + 1, sc, s);  // runbase[n] = table cells in use
   }

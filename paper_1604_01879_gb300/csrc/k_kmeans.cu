@@ -26,6 +26,7 @@ __global__ __launch_bounds__(kMeanT) void k_km_mean(const float* __restrict__ X,
                                                     const int32_t* __restrict__ perm,
                                                     const int64_t* __restrict__ off, const float* __restrict__ C_old,
                                                     float* __restrict__ C_new) {
+  dep_begin();
   const int c = blockIdx.x;
   const int d = (blockIdx.y * kMeanT + threadIdx.x) * 4;
   if (d >= D) return;
@@ -127,8 +128,8 @@ void kmeans(const float* X, int64_t n, int D, int K, const std::vector<int32_t>&
     assign_codes(tmp, X, n, 1, lab, isc, s, x_inv, nullptr, parts.hi ? &parts : nullptr, cb_max);
     stable_sort_by_key(lab, n, K, perm, skeys, isc, s);
     bin_offsets(skeys, n, K, off, s);
-    k_km_mean<<<dim3((unsigned)K, (unsigned)cdiv(D, 4 * kMeanT)), kMeanT, 0, s>>>(X, D, perm, off, tmp.codebook,
-                                                                                C_new);
+    launch_dep(k_km_mean, dim3((unsigned)K, (unsigned)cdiv(D, 4 * kMeanT)), dim3(kMeanT), 0, s, X, D, perm, off,
+               tmp.codebook, C_new);
     GIFT_LAUNCHED("k_km_mean");
     GIFT_CUDA(cudaMemcpyAsync(h_off.data(), off, ((size_t)K + 1) * 8, cudaMemcpyDeviceToHost, s));
     GIFT_CUDA(cudaStreamSynchronize(s));

@@ -34,6 +34,7 @@ __global__ void k_row_invnorm(const float* __restrict__ X, int64_t n, int D, flo
 
 // one warp per row: 0.5 * ||x||^2 accumulated in two-float precision
 __global__ void k_half_sq_norm(const float* __restrict__ X, int64_t n, int D, float* __restrict__ out) {
+  dep_begin();
   const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= n) return;
@@ -68,6 +69,7 @@ constexpr int kScanPerBlock = kScanT * kScanItems;
 __global__ __launch_bounds__(kScanT) void k_scan_blocks(const int64_t* __restrict__ in,
                                                          int64_t* __restrict__ out, int64_t n,
                                                          int64_t* __restrict__ block_sums) {
+  dep_begin();
   __shared__ int64_t wtot[kScanT / 32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int64_t base = (int64_t)blockIdx.x * kScanPerBlock + (int64_t)tid * kScanItems;
@@ -115,6 +117,7 @@ __global__ void k_scan_shift(int64_t* __restrict__ out, int64_t n, const int64_t
 // out[i] += the sums of the blocks before i's: each block adds them up itself
 __global__ __launch_bounds__(kScanT) void k_scan_add(int64_t* __restrict__ out, int64_t n,
                                                      const int64_t* __restrict__ sums) {
+  dep_begin();
   __shared__ int64_t part[kScanT / 32];
   const int tid = threadIdx.x, lane = tid & 31;
   const int64_t b = blockIdx.x + 1;  // block 0 has none before it
@@ -140,6 +143,7 @@ constexpr int kRadixT = 1024;
 __global__ __launch_bounds__(kRadixT) void k_radix_hist(const int32_t* __restrict__ keys, int64_t n,
                                                          int shift, int64_t* __restrict__ hist,
                                                          int64_t ntiles) {
+  dep_begin();
   __shared__ int h[256];
   const int tid = threadIdx.x;
   if (tid < 256) h[tid] = 0;
@@ -154,6 +158,7 @@ __global__ __launch_bounds__(kRadixT) void k_radix_scatter(
     const int32_t* __restrict__ keys_in, const int32_t* __restrict__ vals_in, int64_t n, int shift,
     const int64_t* __restrict__ offs, int64_t ntiles, int32_t* __restrict__ keys_out,
     int32_t* __restrict__ vals_out) {
+  dep_begin();
   __shared__ int wcnt[32][257];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   for (int i = tid; i < 32 * 257; i += kRadixT) (&wcnt[0][0])[i] = 0;
@@ -185,6 +190,7 @@ __global__ __launch_bounds__(kRadixT) void k_radix_scatter(
 
 __global__ void k_bin_offsets(const int32_t* __restrict__ sk, int64_t n, int nbins,
                               int64_t* __restrict__ off) {
+  dep_begin();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i > n) return;
   const int prev = (i == 0) ? -1 : sk[i - 1];
@@ -207,7 +213,7 @@ void launch_row_invnorm(const float* X, int64_t n, int D, float* inv, cudaStream
 
 void launch_half_sq_norm(const float* X, int64_t n, int D, float* out, cudaStream_t s) {
   if (n <= 0) return;
-  k_half_sq_norm<<<(unsigned)cdiv(n, 8), 256, 0, s>>>(X, n, D, out);
+  launch_dep(k_half_sq_norm, dim3((unsigned)cdiv(n, 8)), dim3(256), 0, s, X, n, D, out);
   GIFT_LAUNCHED("k_half_sq_norm");
 }
 
@@ -223,11 +229,11 @@ void scan_exclusive_i64(const int64_t* in, int64_t* out, int64_t n, Scratch& sc,
   if (n <= 0) return;
   const int64_t nb = cdiv(n, kScanPerBlock);
   int64_t* sums = sc.get<int64_t>(nb);
-  k_scan_blocks<<<(unsigned)nb, kScanT, 0, s>>>(in, out, n, sums);
+  launch_dep(k_scan_blocks, dim3((unsigned)nb), dim3(kScanT), 0, s, in, out, n, sums);
   GIFT_LAUNCHED("k_scan_blocks");
   if (nb <= 1) return;
   if (nb <= 8192) {
-    k_scan_add<<<(unsigned)(nb - 1), kScanT, 0, s>>>(out, n, sums);
+    launch_dep(k_scan_add, dim3((unsigned)(nb - 1)), dim3(kScanT), 0, s, out, n, sums);
     GIFT_LAUNCHED("k_scan_add");
     return;
   }
@@ -255,10 +261,10 @@ void stable_sort_by_key(const int32_t* keys, int64_t n, int32_t nbins, int32_t* 
     const bool last = p == passes - 1;
     int32_t* ko = last ? keys_out : kbuf[p & 1];
     int32_t* vo = last ? perm_out : vbuf[p & 1];
-    k_radix_hist<<<(unsigned)ntiles, kRadixT, 0, s>>>(kin, n, 8 * p, hist, ntiles);
+    launch_dep(k_radix_hist, dim3((unsigned)ntiles), dim3(kRadixT), 0, s, kin, n, 8 * p, hist, ntiles);
     GIFT_LAUNCHED("k_radix_hist");
     scan_exclusive_i64(hist, offs, 256 * ntiles, sc, s);
-    k_radix_scatter<<<(unsigned)ntiles, kRadixT, 0, s>>>(kin, vin, n, 8 * p, offs, ntiles, ko, vo);
+    launch_dep(k_radix_scatter, dim3((unsigned)ntiles), dim3(kRadixT), 0, s, kin, vin, n, 8 * p, offs, ntiles, ko, vo);
     GIFT_LAUNCHED("k_radix_scatter");
     kin = ko;
     vin = vo;
@@ -266,7 +272,7 @@ void stable_sort_by_key(const int32_t* keys, int64_t n, int32_t nbins, int32_t* 
 }
 
 void bin_offsets(const int32_t* sorted_keys, int64_t n, int32_t nbins, int64_t* off, cudaStream_t s) {
-  k_bin_offsets<<<(unsigned)cdiv(n + 1, 256), 256, 0, s>>>(sorted_keys, n, nbins, off);
+  launch_dep(k_bin_offsets, dim3((unsigned)cdiv(n + 1, 256)), dim3(256), 0, s, sorted_keys, n, nbins, off);
   GIFT_LAUNCHED("k_bin_offsets");
 }
 
