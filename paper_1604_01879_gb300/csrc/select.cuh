@@ -211,15 +211,21 @@ __device__ int select(Smem& sm, const Get& get, int64_t n, int64_t valid, int k)
   auto remains = [&](unsigned long long key, uint32_t id) {
     return (!binned || score_bin(Get::score(key)) == bin0) && (key & mk) == pk && (~id & ml) == pl;
   };
-  // counts d (-1: none) of the warp's lanes: one atomic for the first counted lane's bin, where most pairs
-  // of a row that few shapes reach fall, and one each for the rest
+  // counts d (-1: none) of the warp's lanes: lanes that share a bin by one atomic as long as the groups found are of
+  // four or more (scores of a few bins, or a row that few shapes reach), and the rest one each (256 rows of 200,000
+  // scores of 400 classes: 775 us with one group, 738)
   auto count_bin = [&](int d) {
-    const unsigned m = __ballot_sync(kAll, d >= 0);
+    unsigned m = __ballot_sync(kAll, d >= 0);
     if (!m) return;
-    const int lead = __ffs(m) - 1, d0 = __shfl_sync(kAll, d, lead);
-    const unsigned same = __ballot_sync(kAll, d == d0);
-    if (lane == lead) atomicAdd(&sm.hist[d0], __popc(same));
-    if (d >= 0 && d != d0) atomicAdd(&sm.hist[d], 1);
+    int group;
+    do {
+      const int lead = __ffs(m) - 1, d0 = __shfl_sync(kAll, d, lead);
+      const unsigned same = __ballot_sync(kAll, d == d0);
+      group = __popc(same);
+      if (lane == lead) atomicAdd(&sm.hist[d0], group);
+      m &= ~same;
+    } while (m && group >= 4);
+    if (m >> lane & 1u) atomicAdd(&sm.hist[d], 1);
   };
   // the bin of the k-th best (threads own runs of bins, best bin first) -> sm.bin, sm.above, sm.in_bin
   auto find_bin = [&]() {
