@@ -1265,7 +1265,7 @@ gift_status gift_index_info(const gift_index* index, gift_index_info_t* out) {
     out->max_list_len = ix.max_list;
     out->n_runs = ix.n_runs;
     out->max_runs = ix.max_runs;
-    out->max_sif_entry = ix.max_sif_entry;
+    out->max_sif_entry = ix.sif_walks.longest;
     out->sif_shapes = ix.sif_off ? ix.sif_n : 0;
     out->sif_k1 = ix.sif_off ? ix.k1 : 0;
   });

@@ -96,6 +96,14 @@ constexpr double kScoreFix = 4294967296.0;  // 2^32
 constexpr double kMemberFix = 2147483648.0;  // 2^31
 
 // ---------------------------------------------------------------- index
+// The walk of a query through an inverted file, estimated at its build from rows of its own shapes (means)
+struct WalkStats {
+  double coords = 0.;  // coordinates of a row
+  double met = 0.;     // shapes in the entry of a coordinate
+  double reach = 0.;   // distinct shapes of a row's entries
+  int longest = 0;     // shapes of the longest entry (exact)
+};
+
 // State of a streamed build (gift_build_begin / add / end_pass).
 struct StreamBuild {
   int stage = 1;               // pass accepting chunks: 1 codes, 2 stores, 3 S-IF; 4 = complete
@@ -159,7 +167,7 @@ struct Index {
   int32_t* sif_ids = nullptr;    // [N*k1]
   uint32_t* sif_mem = nullptr;   // [N*k1]
   uint64_t* sif_card = nullptr;  // [N]
-  int32_t max_sif_entry = 0;
+  WalkStats sif_walks;
   int32_t* row_ids = nullptr;    // [N*k1] N_k1(p) of every database shape, ranked (score desc, id asc)
   float* row_sc = nullptr;       // [N*k1] their scores S(x_p, x_i): the rows of F_p (Eq. 7)
 
@@ -190,6 +198,9 @@ size_t dtype_bytes(int storage);
 // scan constants: entries and query slots per work item of the scan kernel
 constexpr int kScanTE = 64;
 constexpr int kScanTS = 64;
+
+// tc_host.cu
+int device_sm_count();
 
 // k_util.cu
 void launch_row_invnorm(const float* X, int64_t n, int D, float* inv, cudaStream_t s);
@@ -287,7 +298,7 @@ struct Aca {
   uint32_t* mem = nullptr;             // [pairs] round(F_p[i] * 2^31)
   unsigned long long* card = nullptr;  // [N] ||F_p||_1 in the same fixed point
   int64_t pairs = 0;
-  int32_t max_entry = 0;
+  WalkStats walks;
   std::vector<void*> owned;
   size_t device_bytes = 0;
   template <class T> T* alloc(size_t n);

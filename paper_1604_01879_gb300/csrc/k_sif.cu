@@ -25,6 +25,8 @@
 // mean of Eq. 9. The database activations are transposed into a second
 // inverted file of their own; a query's activation is walked through it as in
 // the one-measure re-rank.
+#include <cmath>
+
 #include "gift_internal.cuh"
 #include "select.cuh"
 
@@ -69,65 +71,83 @@ __global__ void k_sif_card(const float* __restrict__ nbr_scores, int32_t N, int 
   card[p] = c;
 }
 
-__global__ void k_max_entry(const int64_t* __restrict__ off, int32_t N, int* __restrict__ out) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  atomicMax(out, (int)(off[i + 1] - off[i]));
-}
+// ---------------------------------------------------------------- what a query's walk will take
+// Found when an inverted file is built, by walking it from some of its own shapes, whose rows are what queries bring
+constexpr int kSamples = 64;
+constexpr int kSampleBits = 1 << 18;
+struct Sample {
+  unsigned long long pairs;   // shapes in the entries of the row's coordinates
+  unsigned long long coords;  // coordinates
+  int blank;                  // bits that no shape's hash sets
+};
 
-// ||F_q||_1 per query and the dense S row of the candidates (-inf elsewhere)
-__global__ void k_rerank_prep(const int32_t* __restrict__ cand_ids, const float* __restrict__ cand_scores,
-                              int n_cand, int k1, int32_t N, float* __restrict__ Srow,
-                              unsigned long long* __restrict__ fq_norm) {
-  const int b = blockIdx.x;
-  __shared__ unsigned long long tot;
-  if (threadIdx.x == 0) tot = 0;
+// block j: row j N / samples of `rows` [N, ld], cnt[.] (null: ld) coordinates; longest[0]: the longest entry (zeroed)
+__global__ __launch_bounds__(512) void k_walk_sample(const int32_t* __restrict__ rows, int ld,
+                                                     const int32_t* __restrict__ cnt, int32_t N, int samples,
+                                                     const int64_t* __restrict__ off, const int32_t* __restrict__ ids,
+                                                     Sample* __restrict__ out, int* __restrict__ longest) {
+  __shared__ uint32_t bits[kSampleBits / 32];
+  __shared__ unsigned long long pairs, coords;
+  __shared__ int blank;
+  const int t = threadIdx.x, T = blockDim.x, lane = t & 31;
+  if (t == 0) {
+    pairs = coords = 0ull;
+    blank = 0;
+  }
+  for (int i = t; i < kSampleBits / 32; i += T) bits[i] = 0u;
   __syncthreads();
-  for (int t = threadIdx.x; t < n_cand; t += blockDim.x) {
-    const int32_t id = cand_ids[(int64_t)b * n_cand + t];
-    const float sc = cand_scores[(int64_t)b * n_cand + t];
-    if (id >= 0 && id < N) {
-      Srow[(int64_t)b * N + id] = sc;
-      if (t < k1) atomicAdd(&tot, (unsigned long long)member_fix(sc));
+  int most = 0;
+  for (int64_t i = (int64_t)blockIdx.x * T + t; i < N; i += (int64_t)gridDim.x * T)
+    most = max(most, (int)(off[i + 1] - off[i]));
+  most = __reduce_max_sync(0xffffffffu, most);
+  if (lane == 0) atomicMax(longest, most);
+  const int64_t p = (int64_t)blockIdx.x * N / samples;
+  const int n = cnt ? cnt[p] : ld;
+  for (int r = t >> 5; r < n; r += T >> 5) {
+    const int32_t i = rows[p * ld + r];
+    if (i < 0 || i >= N) continue;
+    const int64_t e0 = off[i], e1 = off[i + 1];
+    if (lane == 0) {
+      atomicAdd(&pairs, (unsigned long long)(e1 - e0));
+      atomicAdd(&coords, 1ull);
+    }
+    for (int64_t e = e0 + lane; e < e1; e += 32) {
+      const uint32_t h = (uint32_t)ids[e] * 2654435761u >> 14;
+      atomicOr(bits + (h >> 5), 1u << (h & 31u));
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0) fq_norm[b] = tot;
+  int own = 0;
+  for (int i = t; i < kSampleBits / 32; i += T) own += 32 - __popc(bits[i]);
+  own = __reduce_add_sync(0xffffffffu, own);
+  if (lane == 0) atomicAdd(&blank, own);
+  __syncthreads();
+  if (t == 0) out[blockIdx.x] = Sample{pairs, coords, blank};
 }
 
-// one block per (query, neighbour i): walk S-IF entry i
-__global__ void k_rerank_walk(const int32_t* __restrict__ cand_ids, const float* __restrict__ cand_scores,
-                              int n_cand, int k1, int32_t N, const int64_t* __restrict__ sif_off,
-                              const int32_t* __restrict__ sif_ids, const uint32_t* __restrict__ sif_mem,
-                              unsigned long long* __restrict__ num) {
-  const int b = blockIdx.x, r = blockIdx.y;
-  const int32_t i = cand_ids[(int64_t)b * n_cand + r];
-  if (i < 0 || i >= N) return;
-  const uint32_t fq = member_fix(cand_scores[(int64_t)b * n_cand + r]);
-  if (fq == 0) return;
-  const int64_t e0 = sif_off[i], e1 = sif_off[i + 1];
-  for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const uint32_t m = sif_mem[e];
-    if (m == 0) continue;
-    atomicAdd(num + (int64_t)b * N + sif_ids[e], (unsigned long long)min(fq, m));
+WalkStats walk_stats(const int32_t* rows, int ld, const int32_t* cnt, int32_t N, const int64_t* off, const int32_t* ids,
+                     Scratch& sc, cudaStream_t s) {
+  const int n = std::min(N, kSamples);
+  Sample* d = sc.get<Sample>(kSamples);
+  int* longest = sc.get<int>(1);
+  GIFT_CUDA(cudaMemsetAsync(longest, 0, sizeof(int), s));
+  k_walk_sample<<<(unsigned)n, 512, 0, s>>>(rows, ld, cnt, N, n, off, ids, d, longest);
+  GIFT_LAUNCHED("k_walk_sample");
+  Sample h[kSamples];
+  WalkStats w;
+  GIFT_CUDA(cudaMemcpyAsync(h, d, n * sizeof(Sample), cudaMemcpyDeviceToHost, s));
+  GIFT_CUDA(cudaMemcpyAsync(&w.longest, longest, sizeof(int), cudaMemcpyDeviceToHost, s));
+  GIFT_CUDA(cudaStreamSynchronize(s));
+  double pairs = 0., coords = 0., reach = 0.;
+  for (int j = 0; j < n; ++j) {
+    pairs += (double)h[j].pairs;
+    coords += (double)h[j].coords;
+    reach += std::min<double>(N, -(double)kSampleBits * std::log(std::max(h[j].blank, 1) / (double)kSampleBits));
   }
-}
-
-__global__ void k_rerank_keys(const unsigned long long* __restrict__ num,
-                              const unsigned long long* __restrict__ fq_norm,
-                              const unsigned long long* __restrict__ card, const float* __restrict__ Srow,
-                              int32_t B, int32_t N, unsigned long long* __restrict__ keys) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (int64_t)B * N) return;
-  const int b = (int)(idx / N);
-  const int p = (int)(idx % N);
-  const unsigned long long nm = num[idx];
-  float sp = 0.f;
-  if (nm > 0) {
-    const unsigned long long den = fq_norm[b] + card[p] - nm;
-    sp = __fdiv_rn(__ull2float_rn(nm), __ull2float_rn(den));
-  }
-  keys[idx] = ((unsigned long long)f2key(sp) << 32) | (unsigned long long)f2key(Srow[idx]);
+  w.coords = coords / n;
+  w.met = coords > 0. ? pairs / coords : 0.;
+  w.reach = reach / n;
+  return w;
 }
 
 // ---------------------------------------------------------------- re-rank of one query per block
@@ -144,8 +164,12 @@ __global__ void k_rerank_keys(const unsigned long long* __restrict__ num,
 //
 // Unreached shapes all have the key (S' = 0, S = -inf). Where they are needed (fewer reached
 // shapes than the top-k) they follow in id order. A hash table that overflows (a query that
-// reaches more shapes than its slots) is given up, and the block goes over the database in
-// ranges of as many shapes as its table holds, merging each range's best with those before.
+// reaches more shapes than its slots) is given up, and the block walks again into a row of
+// the whole database in global memory. Without such a row (no memory for one, or entries too short
+// to fill the slots but unluckily placed) it goes over the database in ranges of as many shapes
+// as its table holds, merging each range's best with those before. (Ranges alone, after a walk that went
+// on in a full table, took 29.7 ms where rows take 5.5 now and dense rows 8.9: 256 queries, 200,000 shapes,
+// k1 = 1,000.)
 struct ReachArgs {
   int32_t N;                     // shapes
   const int32_t* cand_ids;       // [B, n_cand]
@@ -165,10 +189,23 @@ struct ReachArgs {
   int32_t* out_ids;              // [B, topk]
   float* out_sprime;
   int table_bytes;               // dynamic shared memory
-  int hash;                      // 1: hash table first; 0: ranges of shapes (one range when all fit)
+  int hash;                      // 1: hash table first; 0: one range when all shapes fit, else as after an overflow
   unsigned long long* win_key;   // [B, topk] the best of the ranges gone over so far
   uint32_t* win_id;
+  unsigned long long* num;       // [B, N] numerators and tie-break scores of queries that no table holds,
+  float* S;                      //   or null (ranges of shapes)
 };
+__host__ __device__ __forceinline__ int reach_coords(const ReachArgs& a) { return a.act_ids ? a.act_ld : a.k1; }
+
+// coordinate r of query b's activation: its shape (-1: none) and fixed-point value (0: nothing to add)
+__device__ __forceinline__ int32_t reach_coord(const ReachArgs& a, int b, int r, uint32_t& fq) {
+  const int64_t at = (int64_t)b * (a.act_ids ? a.act_ld : a.n_cand) + r;
+  const int32_t i = a.act_ids ? a.act_ids[at] : a.cand_ids[at];
+  fq = 0;
+  if (i < 0 || i >= a.N) return -1;
+  fq = a.act_ids ? a.act_mem[at] : member_fix(a.cand_scores[at]);
+  return i;
+}
 
 constexpr int kReachProbes = 64;  // slots tried before a hash table counts as full
 constexpr uint32_t kNoKey = 0u;   // high key word of a row that is not reached (a real one is >= 0x80000000)
@@ -199,12 +236,10 @@ __device__ __forceinline__ void reach_walk(const ReachArgs& a, int b, const F& f
     int len = 0;
     uint32_t fq = 0;
     if (r < cnt) {
-      const int64_t at = (int64_t)b * (a.act_ids ? a.act_ld : a.n_cand) + r;
-      const int32_t i = a.act_ids ? a.act_ids[at] : a.cand_ids[at];
-      if (i >= 0 && i < a.N) {
-        fq = a.act_ids ? a.act_mem[at] : member_fix(a.cand_scores[at]);
+      const int32_t i = reach_coord(a, b, r, fq);
+      if (fq) {
         e0 = a.off[i];
-        len = fq ? (int)(a.off[i + 1] - e0) : 0;
+        len = (int)(a.off[i + 1] - e0);
       }
     }
     for (int j = 0; j < 32 && r0 + nw * j < cnt; ++j) {
@@ -257,6 +292,20 @@ struct ReachRows {
     key = ((unsigned long long)h << 32) | lo[i];
     id = hid ? (uint32_t)hid[i] : (uint32_t)(r0 + reach_row((int)i));
     return h != kNoKey;
+  }
+};
+
+struct DenseRows {  // a query's row of every shape, in global memory
+  static constexpr int kAhead = 4;
+  static __device__ __forceinline__ uint32_t score(unsigned long long key) { return (uint32_t)(key >> 32); }
+  const unsigned long long* num;
+  const float* S;
+  const unsigned long long* card;
+  unsigned long long fq_norm;
+  __device__ __forceinline__ bool operator()(int64_t i, unsigned long long& key, uint32_t& id) const {
+    key = reach_key(__ldcg(num + i), fq_norm, card, (int32_t)i, __ldcg(S + i));
+    id = (uint32_t)i;
+    return true;
   }
 };
 
@@ -320,15 +369,18 @@ __global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
       hid[i] = -1;
     }
     __syncthreads();
+    int probes = kReachProbes;  // a lane that found none tries no further (stopping the whole walk, asked for at every
+                                // entry, cost walks of 1,000 entries 7%)
     auto slot_of = [&](int32_t id) {  // the shape's slot, taken if it has none; -1: none left near
       uint32_t h = reach_slot(id, rows);
-      for (int n = 0; n < kReachProbes; ++n) {
+      for (int n = 0; n < probes; ++n) {
         int32_t cur = *reinterpret_cast<volatile int32_t*>(hid + h);
         if (cur == -1) cur = atomicCAS(hid + h, -1, id);
         if (cur == -1 || cur == id) return (int)h;
         if (++h == (uint32_t)rows) h = 0;
       }
       s_flag = 1;
+      probes = 1;
       return -1;
     };
     for (int c = t; c < a.n_cand; c += T)
@@ -342,14 +394,28 @@ __global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
     });
     __syncthreads();
     hashed = s_flag == 0;
-    if (!hashed) {  // the table overflowed: ranges of shapes
+    if (!hashed) {  // the table overflowed
       rows = W;
       hi = lo + rows;
       S = reinterpret_cast<float*>(hi + rows);
     }
   }
-  const bool ranges = !hashed && !one;
-  for (int64_t r0 = 0; !hashed && r0 < a.N; r0 += W) {
+  const bool dense = !hashed && a.num, ranges = !hashed && !one && !dense;
+  if (dense) {  // a row of every shape
+    unsigned long long* num = a.num + (int64_t)b * a.N;
+    float* Sg = a.S + (int64_t)b * a.N;
+    for (int64_t i = t; i < a.N; i += T) {
+      num[i] = 0ull;
+      Sg[i] = -INFINITY;
+    }
+    __syncthreads();
+    for (int c = t; c < a.n_cand; c += T)
+      if (cid[c] >= 0 && cid[c] < a.N) Sg[cid[c]] = csc[c];
+    reach_walk(a, b, [&](int32_t id, uint32_t v) { atomicAdd(num + id, (unsigned long long)v); });
+    __syncthreads();
+    take = sel::select(sm, DenseRows{num, Sg, a.card, s_norm}, a.N, a.N, need);
+  }
+  for (int64_t r0 = 0; !hashed && !dense && r0 < a.N; r0 += W) {
     const int n = (int)min((int64_t)W, a.N - r0);
     __syncthreads();
     for (int i = t; i < rows; i += T) {
@@ -384,7 +450,7 @@ __global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
     __syncthreads();
   }
 
-  if (!ranges) {
+  if (!ranges && !dense) {
     // the reached rows, listed first, so that their keys' reads of the norms go out together
     const int lane = t & 31;
     for (int base = 0; base < rows; base += T) {
@@ -454,30 +520,60 @@ __global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
   }
 }
 
-// Table and block of a launch. Two blocks of 512 threads share an SM while a table takes at
-// most 78 KB: all N up to 6,656 shapes, or 4,992 hash slots, which a query's pairs (n_cand
-// candidates, k1 entries of `mean` shapes) should leave a quarter empty. Heavier walks (`heavy`:
-// many entries per query) take a whole SM's table of up to 15,700 shapes, which spares them the probing.
-void launch_reach(ReachArgs& a, int B, int64_t mean, bool heavy, Scratch& sc, cudaStream_t s) {
-  constexpr int kHalf = 71680, kWhole = 188416;
-  int threads = 512;
-  const int64_t rows = reach_rows_bytes(a.N);
-  if (rows <= kHalf || (heavy && rows <= kWhole)) {
-    a.hash = 0;
-    a.table_bytes = (int)rows;
-    threads = a.N <= 1024 ? 256 : rows <= kHalf ? 512 : 1024;
-  } else {
-    const int64_t pairs = (int64_t)a.n_cand + mean * (a.act_ids ? a.act_ld : a.k1);
-    a.hash = 1;
-    a.table_bytes = !heavy && pairs * 16 * 4 / 3 <= kHalf ? kHalf : kWhole;
-    threads = a.table_bytes == kHalf ? 512 : 1024;
+// ---------------------------------------------------------------- re-rank on dense rows
+// Five kernels over [B, N] rows in global memory: a query's walk spreads over as many blocks as it has
+// coordinates.
+inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
+size_t dense_bytes(int32_t B, int32_t N, int32_t topk) {
+  const size_t BN = (size_t)B * (size_t)N;
+  return align256(BN * 8) + align256(BN * 4) + align256((size_t)B * 8) + align256(BN * 8) +
+         align256((size_t)B * (size_t)topk * 8);
+}
+
+// ||F_q||_1 per query and the dense S row of the candidates (-inf elsewhere)
+__global__ void k_rerank_prep(const ReachArgs a, float* __restrict__ Srow, unsigned long long* __restrict__ fq_norm) {
+  const int b = blockIdx.x;
+  __shared__ unsigned long long tot;
+  if (threadIdx.x == 0) tot = 0;
+  __syncthreads();
+  for (int t = threadIdx.x; t < a.n_cand; t += blockDim.x) {
+    const int32_t id = a.cand_ids[(int64_t)b * a.n_cand + t];
+    const float sc = a.cand_scores[(int64_t)b * a.n_cand + t];
+    if (id >= 0 && id < a.N) {
+      Srow[(int64_t)b * a.N + id] = sc;
+      if (t < a.k1) atomicAdd(&tot, (unsigned long long)member_fix(sc));
+    }
   }
-  a.win_key = sc.get<unsigned long long>((size_t)B * a.topk);
-  a.win_id = sc.get<uint32_t>((size_t)B * a.topk);
-  // the largest table, whatever this call takes: calls of several threads set the same value
-  GIFT_CUDA(cudaFuncSetAttribute(k_rerank_reach, cudaFuncAttributeMaxDynamicSharedMemorySize, kWhole));
-  k_rerank_reach<<<(unsigned)B, threads, a.table_bytes, s>>>(a);
-  GIFT_LAUNCHED("k_rerank_reach");
+  __syncthreads();
+  if (threadIdx.x == 0) fq_norm[b] = a.act_ids ? a.act_norm[b] : tot;
+}
+
+// a block per (query, coordinate): walk its entry
+constexpr int kWalkBlocks = 4096;  // per query (then each takes every so many)
+__global__ __launch_bounds__(128) void k_rerank_walk(const ReachArgs a, unsigned long long* __restrict__ num) {
+  const int b = blockIdx.x, cnt = a.act_ids ? a.act_cnt[b] : a.k1;
+  unsigned long long* row = num + (int64_t)b * a.N;
+  for (int r = blockIdx.y; r < cnt; r += gridDim.y) {
+    uint32_t fq;
+    const int32_t i = reach_coord(a, b, r, fq);
+    if (fq == 0) continue;
+    const int64_t e1 = a.off[i + 1];
+    for (int64_t e = a.off[i] + threadIdx.x; e < e1; e += blockDim.x) {
+      const uint32_t m = a.mem[e];
+      if (m) atomicAdd(row + a.ids[e], (unsigned long long)min(fq, m));
+    }
+  }
+}
+
+__global__ void k_rerank_keys(const unsigned long long* __restrict__ num,
+                              const unsigned long long* __restrict__ fq_norm,
+                              const unsigned long long* __restrict__ card, const float* __restrict__ Srow,
+                              int32_t B, int32_t N, unsigned long long* __restrict__ keys) {
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (int64_t)B * N) return;
+  const int b = (int)(idx / N);
+  const int p = (int)(idx % N);
+  keys[idx] = reach_key(num[idx], fq_norm[b], card, p, Srow[idx]);
 }
 
 __global__ void k_keys_to_sprime(const unsigned long long* __restrict__ keys, int64_t n,
@@ -490,6 +586,127 @@ __global__ void k_keys_to_sprime(const unsigned long long* __restrict__ keys, in
 __global__ void k_fill_f32(float* p, int64_t n, float v) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) p[i] = v;
+}
+
+// scratch: dense_bytes(B, N, topk), cleared and filled here, so nothing depends on what it held before
+void dense_rerank(const ReachArgs& a, int32_t B, uint8_t* p, cudaStream_t s) {
+  const int64_t BN = (int64_t)B * a.N;
+  unsigned long long* num = reinterpret_cast<unsigned long long*>(p);
+  p += align256((size_t)BN * 8);
+  float* Srow = reinterpret_cast<float*>(p);
+  p += align256((size_t)BN * 4);
+  unsigned long long* fqn = reinterpret_cast<unsigned long long*>(p);
+  p += align256((size_t)B * 8);
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(p);
+  p += align256((size_t)BN * 8);
+  unsigned long long* kout = reinterpret_cast<unsigned long long*>(p);
+  GIFT_CUDA(cudaMemsetAsync(num, 0, BN * 8, s));
+  k_fill_f32<<<(unsigned)cdiv(BN, 256), 256, 0, s>>>(Srow, BN, -INFINITY);
+  GIFT_LAUNCHED("k_fill_f32");
+  k_rerank_prep<<<(unsigned)B, 256, 0, s>>>(a, Srow, fqn);
+  GIFT_LAUNCHED("k_rerank_prep");
+  k_rerank_walk<<<dim3((unsigned)B, (unsigned)std::min(reach_coords(a), kWalkBlocks)), 128, 0, s>>>(a, num);
+  GIFT_LAUNCHED("k_rerank_walk");
+  k_rerank_keys<<<(unsigned)cdiv(BN, 256), 256, 0, s>>>(num, fqn, a.card, Srow, B, a.N, keys);
+  GIFT_LAUNCHED("k_rerank_keys");
+  topk_rows_u64(reinterpret_cast<const uint64_t*>(keys), B, a.N, a.topk, a.out_ids, reinterpret_cast<uint64_t*>(kout), s);
+  k_keys_to_sprime<<<(unsigned)cdiv((int64_t)B * a.topk, 256), 256, 0, s>>>(kout, (int64_t)B * a.topk, a.out_sprime);
+  GIFT_LAUNCHED("k_keys_to_sprime");
+}
+
+// ---------------------------------------------------------------- which of the two
+constexpr int kHalf = 71680, kWhole = 188416;  // bytes of a table: two blocks share an SM, or one has it
+
+// Re-rank of B queries whose activations have `coords` coordinates; w: what a walk from the inverted file's own shapes
+// takes (their number of coordinates is w.coords). heavy: many entries per query whatever w says.
+//
+// Table and block: two blocks of 512 threads share an SM while a table takes at most kHalf (70 KB): all N up to 5,952
+// shapes, or 4,480 hash slots, which the shapes a query reaches should leave a quarter empty. Heavier walks (of more
+// than twice those slots of pairs) take a whole SM's table of up to 15,680 shapes, which spares them the probing.
+//
+// One block's walk takes 0.24 to 0.6 ns a pair by its threads, however many SMs stand idle; on dense rows a query's coordinates spread over
+// the SMs, at a price in launches and in passes over all N shapes: they take over where the walks are long and the
+// queries few (both sides in microseconds, from the figures below), and where a query reaches more shapes than a table
+// holds, unless every SM has a query to walk. Measured, whole calls in us (one block, dense rows; neighbours drawn from
+// all shapes unless said):
+//   200,000 shapes, k1 =    50, 1 query     62   187        12,000 shapes, k1 = 1,000,     1 query     267    115
+//   200,000, k1 = 200 in classes, 64        61   316        12,000, k1 = 1,000,           64           278    357
+//   200,000, k1 = 1,000,          1      1,034   276        12,000, two measures, k2 = 40, 1         2,811    337
+//   200,000, k1 = 1,000,        256      5,264 8,853        12,000, two measures, k2 = 40, 64        2,471  2,203
+void rerank_queries(ReachArgs& a, int B, double coords, const WalkStats& w, bool heavy, Scratch& sc, cudaStream_t s) {
+  const int sms = device_sm_count();
+  const int64_t rows = reach_rows_bytes(a.N);
+  const double pairs = a.n_cand + coords * w.met;
+  const double reach = std::min<double>(a.N, a.n_cand + w.reach * std::max(1., coords / std::max(1., w.coords)));
+  heavy = heavy || pairs > 2 * (kHalf / 16);
+  int threads = 512;
+  if (rows <= kHalf || (heavy && rows <= kWhole)) {
+    a.hash = 0;
+    a.table_bytes = (int)rows;
+    threads = a.N <= 1024 ? 256 : rows <= kHalf ? 512 : 1024;
+  } else {
+    a.hash = 1;
+    a.table_bytes = !heavy && reach * 16 * 4 / 3 <= kHalf ? kHalf : kWhole;
+    threads = a.table_bytes == kHalf ? 512 : 1024;
+  }
+  bool dense = false;
+  const bool over = a.hash && rows > a.table_bytes && reach * 16 * 4 / 3 > a.table_bytes;  // more than a table holds
+  if (over) {
+    a.hash = 0;
+    dense = B < sms;
+  } else {
+    const double one = (double)cdiv(B, (int64_t)sms * (a.table_bytes <= kHalf ? 2 : 1)) *
+                       (25 + (threads == 1024 ? 0.24e-3 : threads == 512 ? 0.29e-3 : 0.6e-3) * pairs);
+    // (a pair's sum is in DRAM where the rows are larger than L2)
+    const double pair = (double)B * a.N * 8 > 100e6 ? 24e-6 : 3.4e-6;
+    dense = 50 + 0.75e-3 * a.N + B * (1e-5 * a.N + pair * pairs) < one;
+  }
+  if (dense) {
+    uint8_t* p = nullptr;
+    try {
+      p = sc.get<uint8_t>(dense_bytes(B, a.N, a.topk));
+    } catch (const Error&) {  // no memory for them: a block per query
+    }
+    if (p) {
+      dense_rerank(a, B, p, s);
+      return;
+    }
+  }
+  // Rows for queries that no table holds, at most 2 GB of them at a time. Where entries are too short for a walk to
+  // overflow a hash table by much, and the ranges that would follow are few, none are kept ready.
+  a.num = nullptr;
+  int per = B;
+  const double most = a.n_cand + (double)reach_coords(a) * w.longest;
+  const int slots = a.table_bytes / 16, range = a.table_bytes / 12;
+  if (rows > a.table_bytes && (over || most > 8 * slots || (most > slots / 2 && a.N > 64 * range))) {
+    per = (int)std::min<int64_t>(B, std::max<int64_t>(1, ((int64_t)2 << 30) / ((int64_t)a.N * 12)));
+    try {
+      a.num = sc.get<unsigned long long>((size_t)per * a.N + ((size_t)per * a.N + 1) / 2);
+      a.S = reinterpret_cast<float*>(a.num + (size_t)per * a.N);
+    } catch (const Error&) {  // no memory for them: ranges of shapes
+      per = B;
+    }
+  }
+  if (!a.num) {
+    a.win_key = sc.get<unsigned long long>((size_t)B * a.topk);
+    a.win_id = sc.get<uint32_t>((size_t)B * a.topk);
+  }
+  // the largest table, whatever this call takes: calls of several threads set the same value
+  GIFT_CUDA(cudaFuncSetAttribute(k_rerank_reach, cudaFuncAttributeMaxDynamicSharedMemorySize, kWhole));
+  for (int b0 = 0; b0 < B; b0 += per) {
+    k_rerank_reach<<<(unsigned)std::min(per, B - b0), threads, a.table_bytes, s>>>(a);
+    GIFT_LAUNCHED("k_rerank_reach");
+    a.cand_ids += (int64_t)per * a.n_cand;
+    a.cand_scores += (int64_t)per * a.n_cand;
+    if (a.act_ids) {
+      a.act_ids += (int64_t)per * a.act_ld;
+      a.act_mem += (int64_t)per * a.act_ld;
+      a.act_cnt += per;
+      a.act_norm += per;
+    }
+    a.out_ids += (int64_t)per * a.topk;
+    a.out_sprime += (int64_t)per * a.topk;
+  }
 }
 
 // ---------------------------------------------------------------- two measures
@@ -717,12 +934,7 @@ void aca_build(Aca& a, Scratch& sc, cudaStream_t s) {
     k_aca_fill<<<(unsigned)cdiv(pairs, 256), 256, 0, s>>>(perm, pairs, r.cap, r.out_mem, a.ids, a.mem);
     GIFT_LAUNCHED("k_aca_fill");
   }
-  int* mx = sc.get<int>(1);
-  GIFT_CUDA(cudaMemsetAsync(mx, 0, sizeof(int), s));
-  k_max_entry<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(a.off, N, mx);
-  GIFT_LAUNCHED("k_max_entry");
-  GIFT_CUDA(cudaMemcpyAsync(&a.max_entry, mx, sizeof(int), cudaMemcpyDeviceToHost, s));
-  GIFT_CUDA(cudaStreamSynchronize(s));
+  a.walks = walk_stats(r.out_ids, r.cap, r.out_cnt, N, a.off, a.ids, sc, s);
 }
 
 void aca_rerank(const Aca& a, const int32_t* cand1, const float* sc1, const int32_t* cand2, const float* sc2,
@@ -769,7 +981,7 @@ void aca_rerank(const Aca& a, const int32_t* cand1, const float* sc1, const int3
   g.topk = topk;
   g.out_ids = out_ids;
   g.out_sprime = out_sprime;
-  launch_reach(g, B, cdiv(a.pairs, (int64_t)N), true, sc, s);
+  rerank_queries(g, B, a.walks.coords, a.walks, true, sc, s);
 }
 
 void sif_build(Index& ix, const int32_t* nbr_ids, const float* nbr_scores, Scratch& sc, cudaStream_t s) {
@@ -790,20 +1002,17 @@ void sif_build(Index& ix, const int32_t* nbr_ids, const float* nbr_scores, Scrat
   k_sif_card<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(nbr_scores, N, k1,
                                                       reinterpret_cast<unsigned long long*>(ix.sif_card));
   GIFT_LAUNCHED("k_sif_card");
-  int* mx = sc.get<int>(1);
-  GIFT_CUDA(cudaMemsetAsync(mx, 0, sizeof(int), s));
-  k_max_entry<<<(unsigned)cdiv(N, 256), 256, 0, s>>>(ix.sif_off, N, mx);
-  GIFT_LAUNCHED("k_max_entry");
-  int h[2] = {0, 0};
-  GIFT_CUDA(cudaMemcpyAsync(&h[0], bad, sizeof(int), cudaMemcpyDeviceToHost, s));
-  GIFT_CUDA(cudaMemcpyAsync(&h[1], mx, sizeof(int), cudaMemcpyDeviceToHost, s));
-  GIFT_CUDA(cudaStreamSynchronize(s));
-  if (h[0]) fail(GIFT_EINVAL, "S-IF build: a database shape has fewer than k1 neighbours");
-  ix.max_sif_entry = h[1];
+  int h_bad = 0;
+  GIFT_CUDA(cudaMemcpyAsync(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+  const WalkStats w = walk_stats(nbr_ids, k1, nullptr, N, ix.sif_off, ix.sif_ids, sc, s);
+  if (h_bad) fail(GIFT_EINVAL, "S-IF build: a database shape has fewer than k1 neighbours");
+  ix.sif_walks = w;
 }
 
-void sif_rerank(const Index& ix, const int32_t* cand_ids, const float* cand_scores, int32_t B, int32_t n_cand,
-                int32_t k1, int32_t topk, int32_t* out_ids, float* out_sprime, Scratch& sc, cudaStream_t s) {
+namespace {
+
+ReachArgs sif_args(const Index& ix, const int32_t* cand_ids, const float* cand_scores, int32_t n_cand, int32_t k1,
+                   int32_t topk, int32_t* out_ids, float* out_sprime) {
   ReachArgs g{};
   g.N = ix.sif_n;
   g.cand_ids = cand_ids;
@@ -817,53 +1026,26 @@ void sif_rerank(const Index& ix, const int32_t* cand_ids, const float* cand_scor
   g.topk = topk;
   g.out_ids = out_ids;
   g.out_sprime = out_sprime;
-  launch_reach(g, B, ix.k1, false, sc, s);
+  return g;
 }
 
-namespace {
-inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 }  // namespace
 
-size_t sif_rerank_scratch_bytes(int32_t B, int32_t N, int32_t topk) {
-  const size_t BN = (size_t)B * (size_t)N;
-  return align256(BN * 8) + align256(BN * 4) + align256((size_t)B * 8) + align256(BN * 8) +
-         align256((size_t)B * (size_t)topk * 8);
+void sif_rerank(const Index& ix, const int32_t* cand_ids, const float* cand_scores, int32_t B, int32_t n_cand,
+                int32_t k1, int32_t topk, int32_t* out_ids, float* out_sprime, Scratch& sc, cudaStream_t s) {
+  ReachArgs g = sif_args(ix, cand_ids, cand_scores, n_cand, k1, topk, out_ids, out_sprime);
+  rerank_queries(g, B, k1, ix.sif_walks, false, sc, s);
 }
 
-// The re-rank of sif_rerank on scratch the caller provides (no allocation):
-// the same kernels, with the numerator cleared and the candidate row filled
-// before use, so nothing depends on what the scratch held before.
+size_t sif_rerank_scratch_bytes(int32_t B, int32_t N, int32_t topk) { return dense_bytes(B, N, topk); }
+
+// The re-rank on scratch the caller provides (no allocation): the dense rows, whatever the walks are
 void sif_rerank_into(const Index& ix, const int32_t* cand_ids, const float* cand_scores, int32_t B, int32_t n_cand,
                      int32_t k1, int32_t topk, int32_t* out_ids, float* out_sprime, void* scratch,
                      size_t scratch_bytes, cudaStream_t s) {
-  const int32_t N = ix.sif_n;
-  const int64_t BN = (int64_t)B * N;
-  GIFT_REQUIRE(sif_rerank_scratch_bytes(B, N, topk) <= scratch_bytes, "re-rank scratch too small");
-  uint8_t* p = static_cast<uint8_t*>(scratch);
-  unsigned long long* num = reinterpret_cast<unsigned long long*>(p);
-  p += align256((size_t)BN * 8);
-  float* Srow = reinterpret_cast<float*>(p);
-  p += align256((size_t)BN * 4);
-  unsigned long long* fqn = reinterpret_cast<unsigned long long*>(p);
-  p += align256((size_t)B * 8);
-  unsigned long long* keys = reinterpret_cast<unsigned long long*>(p);
-  p += align256((size_t)BN * 8);
-  unsigned long long* kout = reinterpret_cast<unsigned long long*>(p);
-  GIFT_CUDA(cudaMemsetAsync(num, 0, BN * 8, s));
-  k_fill_f32<<<(unsigned)cdiv(BN, 256), 256, 0, s>>>(Srow, BN, -INFINITY);
-  GIFT_LAUNCHED("k_fill_f32");
-  k_rerank_prep<<<(unsigned)B, 256, 0, s>>>(cand_ids, cand_scores, n_cand, k1, N, Srow, fqn);
-  GIFT_LAUNCHED("k_rerank_prep");
-  k_rerank_walk<<<dim3((unsigned)B, (unsigned)k1), 128, 0, s>>>(cand_ids, cand_scores, n_cand, k1, N, ix.sif_off,
-                                                             ix.sif_ids, ix.sif_mem, num);
-  GIFT_LAUNCHED("k_rerank_walk");
-  k_rerank_keys<<<(unsigned)cdiv(BN, 256), 256, 0, s>>>(num, fqn,
-                                                          reinterpret_cast<const unsigned long long*>(ix.sif_card),
-                                                          Srow, B, N, keys);
-  GIFT_LAUNCHED("k_rerank_keys");
-  topk_rows_u64(reinterpret_cast<const uint64_t*>(keys), B, N, topk, out_ids, reinterpret_cast<uint64_t*>(kout), s);
-  k_keys_to_sprime<<<(unsigned)cdiv((int64_t)B * topk, 256), 256, 0, s>>>(kout, (int64_t)B * topk, out_sprime);
-  GIFT_LAUNCHED("k_keys_to_sprime");
+  GIFT_REQUIRE(dense_bytes(B, ix.sif_n, topk) <= scratch_bytes, "re-rank scratch too small");
+  dense_rerank(sif_args(ix, cand_ids, cand_scores, n_cand, k1, topk, out_ids, out_sprime), B,
+               static_cast<uint8_t*>(scratch), s);
 }
 
 }  // namespace gift

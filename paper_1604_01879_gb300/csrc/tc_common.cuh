@@ -213,6 +213,5 @@ CUtensorMap make_tmap_u8(const void* base, uint64_t rows, uint64_t cols, uint32_
 // host: 2-D FP32 tensor map, box {box_cols columns, box_rows rows}, no swizzle, zero fill outside (the box may be
 // larger than the matrix); 16-byte aligned base, cols a multiple of 4.
 CUtensorMap make_tmap_f32(const void* base, uint64_t rows, uint64_t cols, uint32_t box_cols, uint32_t box_rows);
-int device_sm_count();
 
 }  // namespace gift
