@@ -13,6 +13,7 @@
 // atomicMin on the float bits (non-negative floats order like their bit patterns):
 // in shared memory, band by band of the image, or in global memory (band_plan).
 #include <cmath>
+#include <cstring>
 
 #include "gift_internal.cuh"
 #include "tc_common.cuh"
@@ -97,16 +98,100 @@ __global__ __launch_bounds__(kRenderT) void k_mesh_scale(const float* __restrict
   }
 }
 
-// every vertex index must address its own mesh's vertices
-__global__ void k_check_tris(const int32_t* __restrict__ T, const int64_t* __restrict__ voff,
-                             const int64_t* __restrict__ toff, int M, int* __restrict__ bad) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= toff[M]) return;
-  const int m = find_mesh(toff, M, t);
-  const int64_t nv = voff[m + 1] - voff[m];
-  for (int k = 0; k < 3; ++k) {
-    const int32_t i = T[t * 3 + k];
-    if (i < 0 || i >= nv) atomicExch(bad, 1);
+// host: the float of an f2key (0: -infinity)
+inline float key_value(uint32_t k) {
+  const uint32_t u = k & 0x80000000u ? k & 0x7fffffffu : ~k;
+  float f;
+  memcpy(&f, &u, 4);
+  return k ? f : -INFINITY;
+}
+
+// A mesh's triangles, as the host needs them to choose how to draw it (all zero: none). The box of a triangle
+// shows, on average over all directions, a third of dx dy + dy dz + dz dx.
+struct MeshFacts {
+  float boxes;                // the triangles' sum
+  float largest;              // and their largest
+  uint32_t high[3], low[3];   // f2key of the largest coordinates, and of the largest of the negated ones
+};
+
+// every vertex index must address its own mesh's vertices; facts [M] (zeroed)
+__global__ __launch_bounds__(kRenderT) void k_check_tris(const float* __restrict__ V, const int32_t* __restrict__ T,
+                                                         const int64_t* __restrict__ voff,
+                                                         const int64_t* __restrict__ toff, int M,
+                                                         MeshFacts* __restrict__ facts, int* __restrict__ bad) {
+  __shared__ MeshFacts part[kRenderT / 32];
+  __shared__ int s_first;
+  const int64_t t = (int64_t)blockIdx.x * kRenderT + threadIdx.x;
+  const int m = t < toff[M] ? find_mesh(toff, M, t) : -1;
+  MeshFacts f{};
+  if (m >= 0) {
+    const int64_t nv = voff[m + 1] - voff[m];
+    const float* Vm = V + voff[m] * 3;
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    bool ok = true;
+    for (int k = 0; k < 3; ++k) {
+      const int32_t i = T[t * 3 + k];
+      if (i < 0 || i >= nv) {
+        ok = false;
+        continue;
+      }
+      for (int d = 0; d < 3; ++d) {
+        const float x = Vm[(int64_t)i * 3 + d];
+        lo[d] = fminf(lo[d], x);
+        hi[d] = fmaxf(hi[d], x);
+      }
+    }
+    if (ok) {
+      const float d0 = hi[0] - lo[0], d1 = hi[1] - lo[1], d2 = hi[2] - lo[2];
+      f.boxes = f.largest = d0 * d1 + d1 * d2 + d2 * d0;
+      for (int d = 0; d < 3; ++d) {
+        f.high[d] = f2key(hi[d]);
+        f.low[d] = f2key(-lo[d]);
+      }
+    } else {
+      atomicExch(bad, 1);
+    }
+  }
+  auto add = [&](MeshFacts& to) {
+    atomicAdd(&to.boxes, f.boxes);
+    atomicMax(reinterpret_cast<int*>(&to.largest), __float_as_int(f.largest));  // (not negative)
+    for (int d = 0; d < 3; ++d) {
+      atomicMax(&to.high[d], f.high[d]);
+      atomicMax(&to.low[d], f.low[d]);
+    }
+  };
+  auto join = [&](const MeshFacts& o) {
+    f.boxes += o.boxes;
+    f.largest = fmaxf(f.largest, o.largest);
+    for (int d = 0; d < 3; ++d) {
+      f.high[d] = max(f.high[d], o.high[d]);
+      f.low[d] = max(f.low[d], o.low[d]);
+    }
+  };
+  // one thread adds for a block whose triangles are all of one mesh, else one for each such warp
+  const int lane = threadIdx.x & 31;
+  const bool warp_one = __all_sync(0xffffffffu, m == __shfl_sync(0xffffffffu, m, 0) || m < 0);
+  if (warp_one) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      MeshFacts y;
+      y.boxes = __shfl_xor_sync(0xffffffffu, f.boxes, o);
+      y.largest = __shfl_xor_sync(0xffffffffu, f.largest, o);
+      for (int d = 0; d < 3; ++d) {
+        y.high[d] = __shfl_xor_sync(0xffffffffu, f.high[d], o);
+        y.low[d] = __shfl_xor_sync(0xffffffffu, f.low[d], o);
+      }
+      join(y);
+    }
+    if (lane == 0) part[threadIdx.x >> 5] = f;
+  }
+  if (threadIdx.x == 0) s_first = m;
+  __syncthreads();
+  if (!__syncthreads_and(m == s_first || m < 0)) {
+    if (m >= 0 && (lane == 0 || !warp_one)) add(facts[m]);
+  } else if (threadIdx.x == 0) {
+    for (int i = 1; i < kRenderT / 32; ++i) join(part[i]);
+    add(facts[m]);
   }
 }
 
@@ -158,10 +243,8 @@ __device__ __forceinline__ int py_first(float hi, int n) { return max(0, (int)ce
 __device__ __forceinline__ int py_last(float lo, int n) {
   return min(n - 1, (int)floorf((1.f - lo) * 0.5f * n - 0.5f) + 1);
 }
-// an edge function dx (py - y) - dy (px - x), the first product (the same along a row) rounded by itself
-__device__ __forceinline__ float edge(float dx, float pyy, float dy, float px, float x) {
-  return __fmaf_rn(-dy, px - x, __fmul_rn(dx, pyy));
-}
+// an edge function dx (py - y) - dy (px - x) from the first product (the same along a row), rounded by itself
+__device__ __forceinline__ float edge(float row, float dy, float px, float x) { return __fmaf_rn(-dy, px - x, row); }
 // two FP32 values in one 64-bit register: add, multiply and fused multiply-add of both by one instruction
 // each, rounded as the scalar ones are
 typedef unsigned long long f2x;
@@ -439,12 +522,15 @@ __global__ __launch_bounds__(kRenderT) void k_render(const float* __restrict__ V
   for (int i = i0; i <= i1; ++i) {
     const float py = 1.f - (float)(2 * i + 1) / (float)H;
     if (py < ymin || py > ymax) continue;
+    const float ra = __fmul_rn(tr.x[2] - tr.x[1], py - tr.y[1]);
+    const float rb = __fmul_rn(tr.x[0] - tr.x[2], py - tr.y[2]);
+    const float rc = __fmul_rn(tr.x[1] - tr.x[0], py - tr.y[0]);
     for (int j = j0; j <= j1; ++j) {
       const float px = -1.f + (float)(2 * j + 1) / (float)W;
       if (px < xmin || px > xmax) continue;
-      const float ea = edge(tr.x[2] - tr.x[1], py - tr.y[1], tr.y[2] - tr.y[1], px, tr.x[1]);
-      const float eb = edge(tr.x[0] - tr.x[2], py - tr.y[2], tr.y[0] - tr.y[2], px, tr.x[2]);
-      const float ec = edge(tr.x[1] - tr.x[0], py - tr.y[0], tr.y[1] - tr.y[0], px, tr.x[0]);
+      const float ea = edge(ra, tr.y[2] - tr.y[1], px, tr.x[1]);
+      const float eb = edge(rb, tr.y[0] - tr.y[2], px, tr.x[2]);
+      const float ec = edge(rc, tr.y[1] - tr.y[0], px, tr.x[0]);
       if (ea < 0.f || eb < 0.f || ec < 0.f) continue;
       const float z = fminf(fmaxf((ea * tr.z[0] + eb * tr.z[1] + ec * tr.z[2]) * inv_area, 0.f), 2.f);
       atomicMin(reinterpret_cast<int*>(img + (int64_t)i * W + j), __float_as_int(z));
@@ -453,11 +539,17 @@ __global__ __launch_bounds__(kRenderT) void k_render(const float* __restrict__ V
 }
 
 // Rows of a band and bands of an image: as many rows as shared memory holds, fewer where the images would not
-// give every SM two blocks (but at least 16). False: the images are drawn in global memory, which is better for
-// images of more than kMostBands bands (each band sets the whole mesh up) and for few images of large meshes
-// (a block walks its mesh alone: from 8,192 triangles on, with less than a block per SM).
-bool band_plan(int64_t images, int64_t tris, int M, int H, int W, int& rows, int& bands) {
-  const int64_t sms = device_sm_count();
+// give every SM two blocks (but at least 16). False: the images are drawn in global memory. That is for images of more
+// than kMostBands bands, and for meshes of many small triangles, which every band sets up anew: 13 ps a triangle,
+// image and band, or a block's 2.9 us per 512 triangles where few blocks run, against 26 ps a triangle and image. Global
+// memory costs 1.7 ps more per pixel of a triangle's box (beyond the first few), 80 ns a pixel for the largest one's
+// thread, and the fill. Measured, closed surfaces, whole calls in us (bands, global): 512 images of 224 x 224 in
+// 3 bands, 1,680 triangles 451 and 609, 9,408: 707 and 728, 28,560: 1,250 and 999; of 512 x 512 in 14 bands, 9,408:
+// 1,789 and 1,955, 98,000: 8,868 and 3,458; 64 of 224 x 224, 1,680: 304 and 323, 9,408: 381 and 326, 397,000: 3,220 and
+// 1,375.
+bool band_plan(const std::vector<int64_t>& toff, int M, int Nv, int H, int W, const std::vector<MeshFacts>& facts,
+               int& rows, int& bands) {
+  const int64_t sms = device_sm_count(), images = (int64_t)M * Nv;
   int fit = 0;
   while (fit < H && band_bytes(fit + 1, W) <= (size_t)kBandSmem) ++fit;
   if (fit == 0) return false;
@@ -467,7 +559,28 @@ bool band_plan(int64_t images, int64_t tris, int M, int H, int W, int& rows, int
   bands = std::max(bands, (int)std::min<int64_t>(want, kMostBands));
   rows = (int)cdiv(H, bands);
   bands = (int)cdiv(H, rows);
-  return !(images * bands < sms && tris / M >= 8192) && images * bands < INT32_MAX;
+  if (images * bands >= INT32_MAX) return false;
+  int64_t most = 0;  // triangles of the largest mesh
+  double boxes = 0., largest = 0.;  // of meshes scaled to radius 1
+  for (int m = 0; m < M; ++m) {
+    most = std::max(most, toff[m + 1] - toff[m]);
+    double r2 = 0.;  // the radius squared: a third of this for a ball's extents, all of it for a box's or a rod's
+    for (int d = 0; d < 3; ++d) {
+      const double e = key_value(facts[m].high[d]) + key_value(facts[m].low[d]);
+      r2 += e * e / 4;
+    }
+    r2 *= 0.4;
+    if (toff[m + 1] == toff[m] || r2 <= 0.) continue;
+    boxes += facts[m].boxes / r2;
+    largest = std::max(largest, facts[m].largest / r2);
+  }
+  const double seen = (double)toff[M] * Nv, image = (double)H * W;  // (the image spans 2 x 2)
+  const double tested = boxes / 3 / std::max<int64_t>(toff[M], 1) * image / 4;
+  const double band_us = std::max(13e-6 * bands * seen, 2.9 / 512 * most);
+  const double global_us = 26e-6 * seen +
+                           std::max(1.7e-6 * seen * std::max(0., tested - 5), 80e-3 * largest / 3 * image / 4) +
+                           1.35e-6 * images * image + 2;
+  return band_us < global_us;
 }
 
 }  // namespace
@@ -505,15 +618,18 @@ void render_views(const float* V, const int32_t* T, const std::vector<int64_t>& 
   GIFT_CUDA(cudaMemcpyAsync(voff, head.data(), head.size() * 8, cudaMemcpyHostToDevice, s));
   const int64_t* toff = voff + n_off;
   const float* d_fr = reinterpret_cast<const float*>(voff + 2 * n_off);
+  std::vector<MeshFacts> h_facts((size_t)M + 1);  // the last one's first word: an index was out of range
   if (h_toff[M] > 0) {
-    int* bad = sc.get<int>(1);
-    GIFT_CUDA(cudaMemsetAsync(bad, 0, sizeof(int), s));
-    k_check_tris<<<(unsigned)cdiv(h_toff[M], 256), 256, 0, s>>>(T, voff, toff, M, bad);
+    MeshFacts* facts = sc.get<MeshFacts>(h_facts.size());
+    GIFT_CUDA(cudaMemsetAsync(facts, 0, h_facts.size() * sizeof(MeshFacts), s));
+    k_check_tris<<<(unsigned)cdiv(h_toff[M], kRenderT), kRenderT, 0, s>>>(V, T, voff, toff, M, facts,
+                                                                          reinterpret_cast<int*>(facts + M));
     GIFT_LAUNCHED("k_check_tris");
-    int h_bad = 0;
-    GIFT_CUDA(cudaMemcpyAsync(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
+    GIFT_CUDA(cudaMemcpyAsync(h_facts.data(), facts, h_facts.size() * sizeof(MeshFacts), cudaMemcpyDeviceToHost, s));
     GIFT_CUDA(cudaStreamSynchronize(s));
-    if (h_bad) fail(GIFT_EINVAL, "a triangle addresses a vertex outside its mesh");
+    int bad;
+    memcpy(&bad, &h_facts[M], sizeof(int));
+    if (bad) fail(GIFT_EINVAL, "a triangle addresses a vertex outside its mesh");
   }
   float* cs = sc.get<float>((size_t)M * 4);
   k_mesh_centre<<<(unsigned)M, kRenderT, 0, s>>>(V, T, voff, toff, cs);
@@ -522,7 +638,7 @@ void render_views(const float* V, const int32_t* T, const std::vector<int64_t>& 
   GIFT_LAUNCHED("k_mesh_scale");
   const int64_t images = (int64_t)M * Nv;
   int rows = 0, bands = 0;
-  if (band_plan(images, h_toff[M], M, H, W, rows, bands)) {
+  if (band_plan(h_toff, M, Nv, H, W, h_facts, rows, bands)) {
     GIFT_CUDA(cudaFuncSetAttribute(k_render_bands, cudaFuncAttributeMaxDynamicSharedMemorySize, kBandSmem));
     float* corners = sc.get<float>((size_t)h_toff[M] * 9);
     if (h_toff[M] > 0) {
