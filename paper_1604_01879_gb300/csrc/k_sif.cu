@@ -323,6 +323,7 @@ constexpr int kReachList = 2048;
 // table of N shapes in one range, rows rounded up to the 32 that reach_row mixes
 __host__ __device__ __forceinline__ int64_t reach_rows_bytes(int64_t N) { return (N + 31) / 32 * 32 * 12; }
 
+template <bool ROWS>
 __global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
   extern __shared__ __align__(16) uint32_t table[];
   __shared__ sel::Smem sm;
@@ -400,8 +401,8 @@ __global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
       S = reinterpret_cast<float*>(hi + rows);
     }
   }
-  const bool dense = !hashed && a.num, ranges = !hashed && !one && !dense;
-  if (dense) {  // a row of every shape
+  const bool dense = ROWS && !hashed, ranges = !hashed && !one && !dense;
+  if (ROWS && dense) {  // a row of every shape
     unsigned long long* num = a.num + (int64_t)b * a.N;
     float* Sg = a.S + (int64_t)b * a.N;
     for (int64_t i = t; i < a.N; i += T) {
@@ -692,9 +693,10 @@ void rerank_queries(ReachArgs& a, int B, double coords, const WalkStats& w, bool
     a.win_id = sc.get<uint32_t>((size_t)B * a.topk);
   }
   // the largest table, whatever this call takes: calls of several threads set the same value
-  GIFT_CUDA(cudaFuncSetAttribute(k_rerank_reach, cudaFuncAttributeMaxDynamicSharedMemorySize, kWhole));
+  const auto kernel = a.num ? k_rerank_reach<true> : k_rerank_reach<false>;  // (without rows: less code to fetch)
+  GIFT_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWhole));
   for (int b0 = 0; b0 < B; b0 += per) {
-    k_rerank_reach<<<(unsigned)std::min(per, B - b0), threads, a.table_bytes, s>>>(a);
+    kernel<<<(unsigned)std::min(per, B - b0), threads, a.table_bytes, s>>>(a);
     GIFT_LAUNCHED("k_rerank_reach");
     a.cand_ids += (int64_t)per * a.n_cand;
     a.cand_scores += (int64_t)per * a.n_cand;
