@@ -640,17 +640,28 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
   __nv_bfloat16* hi = parts ? parts->hi : sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
   __nv_bfloat16* lo = parts ? parts->lo : sc.get<__nv_bfloat16>((size_t)rows_alloc * D);
   const int sms = device_sm_count();
-  // codewords per item: as many as leave an item for every SM (one pass over the rows)
-  const int64_t row_tiles = cdiv(chunk, (int64_t)tc::kTM);
-  // (a vocabulary of more than 1,024 keeps 64: the refine reads kT scores per chunk and row)
-  int tn = row_tiles * cdiv(K, 256) >= sms ? 256 : K > 1024 || row_tiles * cdiv(K, 64) >= sms ? 64 : 32;
-  // full SMs: pairs of them, where their rounds, each 0.85 of the others' time (measured), take less
+  // Codewords per item: 256 where that leaves an item for every SM (one pass over the rows), fewer otherwise.
+  const int64_t row_tiles = cdiv(chunk, (int64_t)tc::kTM), full = row_tiles * cdiv(K, 256);
+  int tn = 256;
   bool pair = false;
-  if (tn == 256) {
+  if (full >= sms || K > 16384) {
+    // Full SMs: pairs of them, where their rounds, each 0.85 of the others' time (measured), take less; for vocabularies
+    // of 1,025 to 16,384 in any case, whose items keep their best scores sooner from 128 columns (1,300 rows, D = 256, K =
+    // 16,384: 277 us in pairs, 342 one SM per item). Beyond, the refine's read of twice as many kept scores costs more.
     const int64_t items = cdiv(chunk, (int64_t)256) * cdiv(K, 256);
-    pair = 0.85 * cdiv(items, (int64_t)tc::pair_clusters<PairAssignPolicy>()) < cdiv(row_tiles * cdiv(K, 256), (int64_t)sms);
-    if (pair) tn = 128;  // chunks of kept scores
+    pair = (K > 1024 && K <= 16384) ||
+           0.85 * cdiv(items, (int64_t)tc::pair_clusters<PairAssignPolicy>()) < cdiv(full, (int64_t)sms);
+  } else if (K > 4096 || (K > 192 && 3 * full >= sms)) {
+    // Pairs too where a third of the SMs has items or the vocabulary is large: the refine reads 16 scores of every 64
+    // codewords otherwise, which takes longer than the narrower items save (130 rows, D = 256, K = 16,384: 96 us in pairs,
+    // 116 in items of 256, 183 of 64; 3,000 rows, D = 64, K = 1,100: 76, 96, 101; 20 rows, K = 4,096: 74, 85, 64)
+    pair = true;
+  } else {
+    // all scores of items of 32 go to the refine: for small vocabularies, or one round of them (700 rows, D = 4096,
+    // K = 1,024: 166 us in two rounds of 32, 120 in items of 64)
+    tn = K > 1024 || row_tiles * cdiv(K, 64) >= sms || (K > 512 && row_tiles * cdiv(K, 32) > sms) ? 64 : 32;
   }
+  if (pair) tn = 128;  // chunks of kept scores
   const int nch = (int)cdiv(K, tn), kT = kept_scores(tn);
   // Few items: their chains of k-blocks in parts, as long as a part keeps four k-blocks and finds a free SM; the
   // refine's block of a row adds the parts up (108 rows, D = 4096, K = 512: 16 items in 44 us, in eight parts 10;
@@ -699,12 +710,20 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
       kc->end(0);
       kc->assign_rows += m;
     }
-    if (m >= 8 * sms)
-      launch_dep(k_assign_refine<1>, dim3((unsigned)cdiv(m, 8)), dim3(256), 0, s, X + r0 * D, m, D, ix.codebook, K, ma,
-                 cval, cidx, nch, tn, kT, x_inv + r0, ix.cb_max_norm, cb_max, 1, nullptr, codes + r0 * ma);
-    else
-      launch_dep(k_assign_refine<8>, dim3((unsigned)m), dim3(256), 0, s, X + r0 * D, m, D, ix.codebook, K, ma, cval,
-                 cidx, nch, tn, kT, x_inv + r0, ix.cb_max_norm, cb_max, cuts, ix.cb_half_sq, codes + r0 * ma);
+    // A block that is resident while the coarse stage ends finds the SM's memory given to that stage's shared memory, and
+    // little of it left as L1: where a row's kept scores are more than fit there, which its warps go over several
+    // times, it waits for its launch instead (20 rows, D = 64, K = 65,536: 197 us so launched, 164 plainly).
+    auto refine = [&](auto kernel, int64_t blocks) {
+      const bool early = (int64_t)nch * kT * 8 <= 16 * 1024;
+      auto go = [&](auto... a) {
+        if (early) launch_dep(kernel, dim3((unsigned)blocks), dim3(256), 0, s, a...);
+        else kernel<<<(unsigned)blocks, 256, 0, s>>>(a...);
+      };
+      go(X + r0 * D, m, D, (const float*)ix.codebook, K, ma, (const float*)cval, (const int32_t*)cidx, nch, tn, kT,
+         x_inv + r0, ix.cb_max_norm, cb_max, cuts, (const float*)ix.cb_half_sq, codes + r0 * ma);
+    };
+    if (m >= 8 * sms) refine(k_assign_refine<1>, cdiv(m, 8));
+    else refine(k_assign_refine<8>, m);
     GIFT_LAUNCHED("k_assign_refine");
   }
 }
