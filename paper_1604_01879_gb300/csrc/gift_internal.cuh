@@ -100,7 +100,7 @@ constexpr double kMemberFix = 2147483648.0;  // 2^31
 struct WalkStats {
   double coords = 0.;  // coordinates of a row
   double met = 0.;     // shapes in the entry of a coordinate
-  double reach = 0.;   // distinct shapes of a row's entries
+  double reach = 0.;   // distinct shapes of a row's entries (of rows of very many, of some of them)
   int longest = 0;     // shapes of the longest entry (exact)
 };
 

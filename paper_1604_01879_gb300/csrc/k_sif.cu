@@ -75,9 +75,12 @@ __global__ void k_sif_card(const float* __restrict__ nbr_scores, int32_t N, int 
 // Found when an inverted file is built, by walking it from some of its own shapes, whose rows are what queries bring
 constexpr int kSamples = 64;
 constexpr int kSampleBits = 1 << 18;
+constexpr int kSampleCoords = 128;  // of a row, spread over it; and a warp walks so many pairs, which fill any table if their
+constexpr int kSamplePairs = 8192;  // shapes differ (a whole row of 1,000 long entries took 190 us)
 struct Sample {
-  unsigned long long pairs;   // shapes in the entries of the row's coordinates
-  unsigned long long coords;  // coordinates
+  unsigned long long pairs;   // shapes in the entries of the coordinates looked at
+  unsigned long long coords;  // those coordinates
+  int row;                    // all coordinates of the row
   int blank;                  // bits that no shape's hash sets
 };
 
@@ -103,15 +106,19 @@ __global__ __launch_bounds__(512) void k_walk_sample(const int32_t* __restrict__
   if (lane == 0) atomicMax(longest, most);
   const int64_t p = (int64_t)blockIdx.x * N / samples;
   const int n = cnt ? cnt[p] : ld;
-  for (int r = t >> 5; r < n; r += T >> 5) {
-    const int32_t i = rows[p * ld + r];
+  const int looked = min(n, kSampleCoords);
+  int64_t walked = 0;
+  for (int j = t >> 5; j < looked; j += T >> 5) {
+    const int32_t i = rows[p * ld + (int64_t)j * n / looked];
     if (i < 0 || i >= N) continue;
     const int64_t e0 = off[i], e1 = off[i + 1];
     if (lane == 0) {
       atomicAdd(&pairs, (unsigned long long)(e1 - e0));
       atomicAdd(&coords, 1ull);
     }
-    for (int64_t e = e0 + lane; e < e1; e += 32) {
+    const int64_t to = min(e1, e0 + max((int64_t)0, kSamplePairs - walked));
+    walked += e1 - e0;
+    for (int64_t e = e0 + lane; e < to; e += 32) {
       const uint32_t h = (uint32_t)ids[e] * 2654435761u >> 14;
       atomicOr(bits + (h >> 5), 1u << (h & 31u));
     }
@@ -122,7 +129,7 @@ __global__ __launch_bounds__(512) void k_walk_sample(const int32_t* __restrict__
   own = __reduce_add_sync(0xffffffffu, own);
   if (lane == 0) atomicAdd(&blank, own);
   __syncthreads();
-  if (t == 0) out[blockIdx.x] = Sample{pairs, coords, blank};
+  if (t == 0) out[blockIdx.x] = Sample{pairs, coords, n, blank};
 }
 
 WalkStats walk_stats(const int32_t* rows, int ld, const int32_t* cnt, int32_t N, const int64_t* off, const int32_t* ids,
@@ -138,13 +145,14 @@ WalkStats walk_stats(const int32_t* rows, int ld, const int32_t* cnt, int32_t N,
   GIFT_CUDA(cudaMemcpyAsync(h, d, n * sizeof(Sample), cudaMemcpyDeviceToHost, s));
   GIFT_CUDA(cudaMemcpyAsync(&w.longest, longest, sizeof(int), cudaMemcpyDeviceToHost, s));
   GIFT_CUDA(cudaStreamSynchronize(s));
-  double pairs = 0., coords = 0., reach = 0.;
+  double pairs = 0., coords = 0., rows_coords = 0., reach = 0.;
   for (int j = 0; j < n; ++j) {
     pairs += (double)h[j].pairs;
     coords += (double)h[j].coords;
+    rows_coords += h[j].row;
     reach += std::min<double>(N, -(double)kSampleBits * std::log(std::max(h[j].blank, 1) / (double)kSampleBits));
   }
-  w.coords = coords / n;
+  w.coords = rows_coords / n;
   w.met = coords > 0. ? pairs / coords : 0.;
   w.reach = reach / n;
   return w;
@@ -370,18 +378,18 @@ __global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
       hid[i] = -1;
     }
     __syncthreads();
-    int probes = kReachProbes;  // a lane that found none tries no further (stopping the whole walk, asked for at every
-                                // entry, cost walks of 1,000 entries 7%)
+    bool full = false;  // a lane that found none adds no more (a stop of the whole walk, asked for at every entry,
+                        // cost walks of 1,000 entries 7%)
     auto slot_of = [&](int32_t id) {  // the shape's slot, taken if it has none; -1: none left near
       uint32_t h = reach_slot(id, rows);
-      for (int n = 0; n < probes; ++n) {
+      for (int n = 0; n < kReachProbes; ++n) {
         int32_t cur = *reinterpret_cast<volatile int32_t*>(hid + h);
         if (cur == -1) cur = atomicCAS(hid + h, -1, id);
         if (cur == -1 || cur == id) return (int)h;
         if (++h == (uint32_t)rows) h = 0;
       }
       s_flag = 1;
-      probes = 1;
+      full = true;
       return -1;
     };
     for (int c = t; c < a.n_cand; c += T)
@@ -390,6 +398,7 @@ __global__ __launch_bounds__(1024) void k_rerank_reach(const ReachArgs a) {
         if (at >= 0) S[at] = csc[c];
       }
     reach_walk(a, b, [&](int32_t id, uint32_t v) {
+      if (full) return;
       const int at = slot_of(id);
       if (at >= 0) reach_add(lo, hi, at, v);
     });
@@ -983,7 +992,7 @@ void aca_rerank(const Aca& a, const int32_t* cand1, const float* sc1, const int3
   g.topk = topk;
   g.out_ids = out_ids;
   g.out_sprime = out_sprime;
-  rerank_queries(g, B, a.walks.coords, a.walks, true, sc, s);
+  rerank_queries(g, B, (double)a.pairs / N, a.walks, true, sc, s);
 }
 
 void sif_build(Index& ix, const int32_t* nbr_ids, const float* nbr_scores, Scratch& sc, cudaStream_t s) {
