@@ -21,6 +21,13 @@
  *    gift_last_error() gives a message for the last failing call of the
  *    calling thread. GIFT_ECUDA leaves the index usable unless the CUDA
  *    context itself was lost.
+ *  - Waits inside kernels are bounded. One that runs out ends its call's
+ *    kernels early; GIFT_ETIMEOUT is then returned by the call itself where it
+ *    waits for its work (builds, k-means, results to pageable host memory),
+ *    else by the next call on that index, or, for matching calls, which have
+ *    none, by the thread's next matching call. That call does nothing more, and
+ *    the results of the calls before it that were not yet waited for are not
+ *    valid; the calls after it work again.
  *  - A built index is read-only: calls on one index from several host threads
  *    or streams may run concurrently; each call has its own scratch.
  *  - D must be a positive multiple of 16 (16-byte rows for every storage type).
@@ -47,7 +54,7 @@ typedef enum {
   GIFT_EINVAL = 1,       /* an argument is out of range or inconsistent       */
   GIFT_ENOMEM = 2,       /* device or pinned host memory could not be reserved */
   GIFT_ECUDA = 3,        /* a CUDA runtime call or kernel launch failed        */
-  GIFT_ETIMEOUT = 4,     /* a bounded wait ran out (serving loop)             */
+  GIFT_ETIMEOUT = 4,     /* a bounded wait ran out (serving loop, kernels)    */
   GIFT_EUNSUPPORTED = 5, /* the index was built without what the call needs   */
   GIFT_ESTATE = 6        /* the object is in the wrong state for this call    */
 } gift_status;

@@ -423,7 +423,7 @@ void run_fif(Index& ix, const float* q, int64_t nv, const std::vector<int32_t>& 
 
   tm.mark(ST_TOPK);
   if (R <= 0) {
-    topk_rows_f32(S, B, N, topk, out_ids, out_scores, s);
+    topk_rows_f32(S, B, N, topk, out_ids, out_scores, s, ix.d_err);
     return;
   }
   const int Rr = std::min(R, N);
@@ -444,7 +444,7 @@ void run_fif(Index& ix, const float* q, int64_t nv, const std::vector<int32_t>& 
   float* cand_score = sc.get<float>((size_t)B * Rr);
   fif_combine(ix, P, fused ? table32 : table, nullptr, cand_sorted, Rr, cand_score, sc, s);
   tm.mark(ST_TOPK);
-  sort_candidates(cand_sorted, cand_score, B, Rr, topk, out_ids, out_scores, s);
+  sort_candidates(cand_sorted, cand_score, B, Rr, topk, out_ids, out_scores, s, ix.d_err);
 }
 
 }  // namespace
@@ -526,6 +526,13 @@ T* Index::alloc(size_t n) {
   return static_cast<T*>(p);
 }
 
+void Index::make_wait_flag(cudaStream_t s) {
+  wait_word = take_wait_word();
+  const WaitFlag f{0, 0, wait_word};
+  d_err = reinterpret_cast<int*>(alloc<WaitFlag>(1));
+  GIFT_CUDA(cudaMemcpyAsync(d_err, &f, sizeof(f), cudaMemcpyHostToDevice, s));  // (pageable: taken before the return)
+}
+
 Index::~Index() {
   delete sb;
   for (cudaEvent_t e : ev) cudaEventDestroy(e);
@@ -535,6 +542,7 @@ Index::~Index() {
   }
   if (stats_pinned) cudaFreeHost(stats_pinned);
   for (void* p : owned) cudaFree(p);
+  give_wait_word(wait_word);
 }
 
 size_t dtype_bytes(int storage) { return storage == GIFT_F32 ? 4 : storage == GIFT_BF16 ? 2 : 1; }
@@ -631,8 +639,7 @@ void build(const gift_index_params* prm, const float* db_feats, const float* cod
   const bool need_master = p.keep_exact || (p.rescore_r > 0 && !split_rescore);
   float* master = need_master ? ix->alloc<float>((size_t)n_rows * D) : sc.get<float>((size_t)n_rows * D);
   if (need_master) ix->master = master;
-  ix->d_err = ix->alloc<int>(1);
-  GIFT_CUDA(cudaMemsetAsync(ix->d_err, 0, sizeof(int), s));
+  ix->make_wait_flag(s);
   GIFT_CUDA(cudaMemcpyAsync(master, db_feats, (size_t)n_rows * D * 4, cudaMemcpyDefault, s));
   ix->row_inv = ix->alloc<float>(n_rows);
   launch_row_invnorm(master, n_rows, D, ix->row_inv, s);
@@ -721,6 +728,7 @@ void build(const gift_index_params* prm, const float* db_feats, const float* cod
     sif_build(*ix, nbr_ids, nbr_sc, sc, s);
   }
   GIFT_CUDA(cudaStreamSynchronize(s));
+  ix->check_waits(s);
   *out = reinterpret_cast<gift_index*>(ix.release());
 }
 
@@ -773,8 +781,7 @@ void stream_begin(const gift_index_params* prm, const float* codebook, cudaStrea
   GIFT_CUDA(cudaMemcpyAsync(&ix->cb_max_norm, d_cbmax, 4, cudaMemcpyDeviceToHost, s));
   ix->row_inv = ix->alloc<float>(n_rows);
   ix->db_codes = ix->alloc<int32_t>(n_rows * db_ma);
-  ix->d_err = ix->alloc<int>(1);
-  GIFT_CUDA(cudaMemsetAsync(ix->d_err, 0, sizeof(int), s));
+  ix->make_wait_flag(s);
   GIFT_CUDA(cudaStreamSynchronize(s));
   ix->cb_max_norm *= 1.0001f;
   ix->sb = new StreamBuild();
@@ -839,6 +846,7 @@ void stream_add(Index& ix, int pass, const float* feats, int32_t first, int32_t 
     }
   }
   GIFT_CUDA(cudaStreamSynchronize(s));  // the chunk buffer may be reused by the caller
+  ix.check_waits(s);                    // (then the chunk is not counted, and may be added again)
   std::fill(seen.begin() + first, seen.begin() + first + n, (uint8_t)1);
   ix.sb->rows_added += rows;
 }
@@ -904,6 +912,7 @@ void stream_end(Index& ix, int pass, cudaStream_t s) {
     delete ix.sb;
     ix.sb = nullptr;
   }
+  ix.check_waits(s);
 }
 
 }  // namespace
@@ -927,14 +936,17 @@ gift_status gift_build_add(gift_index* index, int32_t pass, const float* feats, 
                            int32_t n_shapes, cudaStream_t stream) {
   return gift::guard("gift_build_add", [&] {
     GIFT_REQUIRE(index, "NULL index");
-    gift::stream_add(*reinterpret_cast<Index*>(index), pass, feats, first_shape, n_shapes, stream);
+    Index& ix = *reinterpret_cast<Index*>(index);
+    gift::stream_add(ix, pass, feats, first_shape, n_shapes, stream);
   });
 }
 
 gift_status gift_build_end_pass(gift_index* index, int32_t pass, cudaStream_t stream) {
   return gift::guard("gift_build_end_pass", [&] {
     GIFT_REQUIRE(index, "NULL index");
-    gift::stream_end(*reinterpret_cast<Index*>(index), pass, stream);
+    Index& ix = *reinterpret_cast<Index*>(index);
+    ix.check_waits(stream);
+    gift::stream_end(ix, pass, stream);
   });
 }
 
@@ -957,6 +969,7 @@ gift_status gift_query(gift_index* index, const float* q_feats, const int32_t* q
     GIFT_REQUIRE(topk > 0 && topk <= 1024, "topk must be in [1, 1024]");
     Index& ix = *reinterpret_cast<Index*>(index);
     if (!ix.ready()) gift::fail(GIFT_ESTATE, "the streamed build of this index is not complete");
+    ix.check_waits(stream);
     std::vector<int32_t> h = gift::host_offsets(q_view_offsets, B);
     const int64_t nv = h[B];
     const int D = ix.prm.dim;
@@ -995,6 +1008,7 @@ gift_status gift_query(gift_index* index, const float* q_feats, const int32_t* q
       gift::fail(GIFT_EINVAL, "unknown matching mode");
     }
     gift::flush_out(outs, stream);
+    if (!outs.empty()) ix.check_waits(stream);  // (pageable results have been waited for)
     if (tm.on) {
       if (!ix.stats_pinned) GIFT_CUDA(cudaMallocHost(&ix.stats_pinned, 8 * sizeof(unsigned long long)));
       GIFT_CUDA(cudaMemcpyAsync(ix.stats_pinned, stats, 8 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
@@ -1015,6 +1029,7 @@ gift_status gift_rerank(gift_index* index, const int32_t* cand_ids, const float*
     if (!ix.sif_off) gift::fail(GIFT_EUNSUPPORTED, "index built without an S-IF (sif_k1 == 0)");
     GIFT_REQUIRE(B > 0 && n_cand > 0 && k1 > 0 && k1 <= n_cand, "need 0 < k1 <= n_cand and B > 0");
     GIFT_REQUIRE(topk > 0 && topk <= 1024, "topk must be in [1, 1024]");
+    ix.check_waits(stream);
     gift::Scratch sc(stream);
     gift::StageTimer tm(&ix, stream);
     std::vector<gift::OutBuf> outs;
@@ -1086,6 +1101,8 @@ gift_status gift_aca_build(const gift_index* measure1, const gift_index* measure
     GIFT_REQUIRE(mode == GIFT_ACA_NONE || (k2 >= 1 && k2 <= a.k1 && k2 * a.k1 <= 2048),
                  "need 1 <= k2 <= k1 and k2 * k1 <= 2048");
     GIFT_REQUIRE(mode != GIFT_ACA_NONE || a.k1 <= 1024, "k1 must be <= 1024");
+    a.check_waits(stream);
+    b.check_waits(stream);
     int dev = 0;
     GIFT_CUDA(cudaGetDevice(&dev));
     std::unique_ptr<gift::Aca> x(new gift::Aca());
@@ -1161,6 +1178,7 @@ gift_status gift_assign(gift_index* index, const float* feats, int64_t n, int32_
     GIFT_REQUIRE(index && feats && out_codes, "NULL argument");
     GIFT_REQUIRE(n >= 0, "n must be >= 0");
     Index& ix = *reinterpret_cast<Index*>(index);
+    ix.check_waits(stream);
     gift::Scratch sc(stream);
     gift::assign_codes(ix, feats, n, ma, out_codes, sc, stream);
   });
@@ -1179,6 +1197,7 @@ gift_status gift_export_fif(const gift_index* index, int32_t* db_codes, int64_t*
     if (list_rows)
       GIFT_CUDA(cudaMemcpyAsync(list_rows, ix.list_row, ix.n_entries * 4, cudaMemcpyDefault, stream));
     GIFT_CUDA(cudaStreamSynchronize(stream));
+    ix.check_waits(stream);
   });
 }
 
@@ -1189,6 +1208,7 @@ gift_status gift_sif_from_neighbours(gift_index* index, const int32_t* nbr_ids, 
     Index& ix = *reinterpret_cast<Index*>(index);
     if (!ix.ready()) gift::fail(GIFT_ESTATE, "the streamed build of this index is not complete");
     if (ix.sif_off) gift::fail(GIFT_ESTATE, "the index already has an S-IF");
+    ix.check_waits(stream);
     GIFT_REQUIRE(n_shapes_total >= 1, "n_shapes_total must be positive");
     GIFT_REQUIRE(k1 >= 1 && k1 <= std::min(1024, n_shapes_total), "k1 must be in [1, min(1024, n_shapes_total)]");
     int dev = 0;
@@ -1251,6 +1271,7 @@ gift_status gift_export_sif(const gift_index* index, int64_t* entry_offsets, int
     if (entry_members) GIFT_CUDA(cudaMemcpyAsync(entry_members, ix.sif_mem, n * 4, cudaMemcpyDefault, stream));
     if (card) GIFT_CUDA(cudaMemcpyAsync(card, ix.sif_card, N * 8, cudaMemcpyDefault, stream));
     GIFT_CUDA(cudaStreamSynchronize(stream));
+    ix.check_waits(stream);
   });
 }
 
@@ -1296,6 +1317,7 @@ gift_status gift_get_timing(gift_index* index, gift_timing_t* out) {
     Index& ix = *reinterpret_cast<Index*>(index);
     if (ix.ev.empty()) gift::fail(GIFT_ESTATE, "no timed call recorded");
     GIFT_CUDA(cudaEventSynchronize(ix.ev.back()));
+    ix.check_waits(nullptr);
     gift_timing_t t{};
     float* slot[gift::ST_END] = {&t.assign_ms, &t.bucket_ms, &t.scan_ms, &t.combine_ms,
                                  &t.topk_ms,   &t.rescore_ms, &t.rerank_ms};
@@ -1337,6 +1359,7 @@ gift_status gift_match_forward(const void* q, const int32_t* q_view_offsets, int
     GIFT_REQUIRE(d_in > 0 && d_in % 16 == 0 && d_out > 0 && d_out % 16 == 0, "dims must be multiples of 16");
     GIFT_REQUIRE(W || d_in == d_out, "d_out must equal d_in without a projection");
     GIFT_REQUIRE(dtype == GIFT_F32 || dtype == GIFT_BF16, "dtype must be GIFT_F32 or GIFT_BF16");
+    gift::check_wait_word(gift::thread_wait_word(), nullptr, stream);
     std::vector<int32_t> h = gift::host_offsets(q_view_offsets, Bq);
     gift::Scratch sc(stream);
     gift::match_forward(q, h, Bq, p, Np, nv_p, W, d_in, d_out, dtype, S, argmax, sc, stream);
@@ -1355,6 +1378,7 @@ gift_status gift_match_backward(const void* q, const int32_t* q_view_offsets, in
     GIFT_REQUIRE(W || !dW, "dW needs a projection");
     GIFT_REQUIRE(d_out <= 1024, "d_out must be at most 1024 for the backward");
     GIFT_REQUIRE(dtype == GIFT_F32 || dtype == GIFT_BF16, "dtype must be GIFT_F32 or GIFT_BF16");
+    gift::check_wait_word(gift::thread_wait_word(), nullptr, stream);
     std::vector<int32_t> h = gift::host_offsets(q_view_offsets, Bq);
     gift::Scratch sc(stream);
     gift::match_backward(q, h, Bq, p, Np, nv_p, W, d_in, d_out, dtype, grad_S, argmax, dW, dQ, dP, sc, stream);

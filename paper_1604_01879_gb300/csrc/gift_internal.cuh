@@ -33,6 +33,31 @@ void count_launch();
 #define GIFT_REQUIRE(cond, msg) \
   do { if (!(cond)) ::gift::fail(GIFT_EINVAL, msg); } while (0)
 
+// ---------------------------------------------------------------- bounded waits
+// Device flag of the waits of an index's calls, or of one call: the first that gives up writes its site here, which
+// ends the others. A kernel that comes after them passes it on into a word of host memory (report_wait; done by the
+// contractions' own kernels, even behind their loops, it took 3% of the FP32-level scan's time, although it never ran),
+// which the host looks at before the next call on the object (for calls without one, the thread's next) and wherever a
+// call waits for its stream. (tc_host.cu)
+struct WaitFlag {
+  int code;
+  int unused;
+  int* word;  // host; null: none
+};
+__device__ __forceinline__ void report_wait(int* err) {  // err optional
+  if (!err) return;
+  const int site = *reinterpret_cast<volatile int*>(err);
+  int* word = reinterpret_cast<WaitFlag*>(err)->word;
+  if (site == 0 || !word) return;
+  *reinterpret_cast<volatile int*>(word) = site;
+  __threadfence_system();
+}
+int* take_wait_word();            // a word of an object's own, zero
+void give_wait_word(int* word);
+int* thread_wait_word();          // the calling thread's, for calls without an object
+// ETIMEOUT when the word is set: it and the flag (optional; in the stream's order) are cleared
+void check_wait_word(int* word, int* flag, cudaStream_t s);
+
 // ---------------------------------------------------------------- dependent launches
 // A launch whose blocks may become resident while the kernel before it in the stream still ends: the device's part of
 // launching overlaps that. It is 1 to 2 us of every kernel in a chain of short ones (29 in a query of four against an
@@ -171,7 +196,8 @@ struct Index {
   int32_t* row_ids = nullptr;    // [N*k1] N_k1(p) of every database shape, ranked (score desc, id asc)
   float* row_sc = nullptr;       // [N*k1] their scores S(x_p, x_i): the rows of F_p (Eq. 7)
 
-  int* d_err = nullptr;          // device error flag set by bounded waits (0 = none)
+  int* d_err = nullptr;          // WaitFlag of its calls (0 = none gave up)
+  int* wait_word = nullptr;      // its host word
   StreamBuild* sb = nullptr;     // non-null while a streamed build is in progress
 
   size_t device_bytes = 0;
@@ -188,6 +214,10 @@ struct Index {
   bool stats_valid = false;
 
   template <class T> T* alloc(size_t n);
+  void make_wait_flag(cudaStream_t s);
+  void check_waits(cudaStream_t s) const {
+    if (wait_word) check_wait_word(wait_word, d_err, s);
+  }
   bool ready() const { return sb == nullptr; }
   ~Index();
 };
@@ -257,14 +287,14 @@ void exact_scores_lists(const Index& ix, const float* q, const float* q_inv, int
 // k_topk.cu
 // Per row b of `scores` [B, n] (or of keys64 when scores == nullptr): the k
 // largest by (value desc, index asc). ids_out/val_out [B, k] (val_out may be
-// null). When n < k the tail gets id -1 and -INF.
+// null). When n < k the tail gets id -1 and -INF. err (optional): the flag of the waits behind the scores, reported.
 void topk_rows_f32(const float* scores, int32_t B, int64_t n, int32_t k, int32_t* ids_out,
-                   float* val_out, cudaStream_t s);
+                   float* val_out, cudaStream_t s, int* err = nullptr);
 void topk_rows_u64(const uint64_t* keys, int32_t B, int64_t n, int32_t k, int32_t* ids_out,
                    uint64_t* key_out, cudaStream_t s);
-// Rows of (id, score) pairs of length r: sort by (score desc, id asc) and keep k.
+// Rows of (id, score) pairs of length r: sort by (score desc, id asc) and keep k (err as in topk_rows_f32).
 void sort_candidates(const int32_t* ids, const float* scores, int32_t B, int32_t r, int32_t k,
-                     int32_t* ids_out, float* scores_out, cudaStream_t s);
+                     int32_t* ids_out, float* scores_out, cudaStream_t s, int* err = nullptr);
 // Rows of ids of length r: ascending copy.
 void sort_ids_rows(const int32_t* ids, int32_t B, int32_t r, int32_t* out, cudaStream_t s);
 // Rows of (id, score) pairs of any length n (ids distinct per row, id < 0 =

@@ -345,17 +345,19 @@ __device__ __forceinline__ void next_best(const float* __restrict__ v, const int
 }
 
 // WPR: warps per row, 1, or 8 (a block per row) where the rows are few: a row's distances are then eight times
-// shorter chains of dependent reads
+// shorter chains of dependent reads. (A warp per row: four blocks on an SM, 64 registers; 76 without that bound, 1% of a
+// k-means call.)
 template <int WPR>
-__global__ __launch_bounds__(256) void k_assign_refine(const float* __restrict__ X, int64_t n, int D,
+__global__ __launch_bounds__(256, WPR == 1 ? 4 : 1) void k_assign_refine(const float* __restrict__ X, int64_t n, int D,
                                                        const float* __restrict__ cb, int K, int ma,
                                                        const float* __restrict__ cval,
                                                        const int32_t* __restrict__ cidx, int nch, int tn, int kT,
                                                        const float* __restrict__ x_inv, float bmax_host,
                                                        const float* __restrict__ bmax_dev, int parts,
                                                        const float* __restrict__ half_sq,
-                                                       int32_t* __restrict__ codes) {
+                                                       int32_t* __restrict__ codes, int* err) {
   dep_begin();
+  if (blockIdx.x == 0 && threadIdx.x == 0) report_wait(err);
   __shared__ DfPart part[8];
   __shared__ float sval[WPR > 1 ? kPartsK : 1];
   __shared__ int32_t sidx[WPR > 1 ? kPartsK : 1];
@@ -720,7 +722,8 @@ void assign_codes(const Index& ix, const float* X, int64_t n, int ma, int32_t* c
         else kernel<<<(unsigned)blocks, 256, 0, s>>>(a...);
       };
       go(X + r0 * D, m, D, (const float*)ix.codebook, K, ma, (const float*)cval, (const int32_t*)cidx, nch, tn, kT,
-         x_inv + r0, ix.cb_max_norm, cb_max, cuts, (const float*)ix.cb_half_sq, codes + r0 * ma);
+         x_inv + r0, ix.cb_max_norm, cb_max, cuts, (const float*)ix.cb_half_sq, codes + r0 * ma,
+         ix.d_err);
     };
     if (m >= 8 * sms) refine(k_assign_refine<1>, cdiv(m, 8));
     else refine(k_assign_refine<8>, m);

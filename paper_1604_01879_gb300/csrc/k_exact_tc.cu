@@ -378,7 +378,7 @@ void segmax_tc(const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int64_t a_r
       p.r_inv = b_inv;
       p.cell = cell;
       run_tiles(tA, tB, tA2, tB2, p, err, s);
-      segmax_reduce(cell, N, d_qoff, b0, b1 - b0, (int32_t)v0, S, argmax, s);
+      segmax_reduce(cell, N, d_qoff, b0, b1 - b0, (int32_t)v0, S, argmax, err, s);
       b0 = b1;
       continue;
     }
@@ -393,7 +393,7 @@ void segmax_tc(const __nv_bfloat16* a_hi, const __nv_bfloat16* a_lo, int64_t a_r
     p.r_inv = b_inv;
     p.cell = cell;
     run_tiles(tA, tB, tA2, tB2, p, err, s);
-    segmax_reduce(cell, N, d_qoff, b0, b1 - b0, (int32_t)v0, S, argmax, s);
+    segmax_reduce(cell, N, d_qoff, b0, b1 - b0, (int32_t)v0, S, argmax, err, s);
     b0 = b1;
   }
 }
@@ -453,7 +453,7 @@ void exact_scores_lists(const Index& ix, const float* q, const float* q_inv, int
     const CUtensorMap tA = make_tmap_bf16(hi + v0 * D, qrows - v0, D, tc::kTM);
     const CUtensorMap tA2 = make_tmap_bf16(lo + v0 * D, qrows - v0, D, tc::kTM);
     run_tiles(tA, tB, tA2, tB2, p, ix.d_err, s);
-    segmax_reduce(cell, N, d_qoff, b0, b1 - b0, (int32_t)v0, S, nullptr, s);
+    segmax_reduce(cell, N, d_qoff, b0, b1 - b0, (int32_t)v0, S, nullptr, ix.d_err, s);
     b0 = b1;
   }
 }

@@ -104,8 +104,7 @@ void kmeans(const float* X, int64_t n, int D, int K, const std::vector<int32_t>&
   tmp.prm.dim = D;
   GIFT_CUDA(cudaGetDevice(&tmp.device));
   tmp.codebook = tmp.alloc<float>((size_t)K * D);
-  tmp.d_err = tmp.alloc<int>(1);
-  GIFT_CUDA(cudaMemsetAsync(tmp.d_err, 0, sizeof(int), s));
+  tmp.make_wait_flag(s);
   int32_t* d_init = sc.get<int32_t>(K);
   GIFT_CUDA(cudaMemcpyAsync(d_init, init_rows.data(), (size_t)K * 4, cudaMemcpyHostToDevice, s));
   k_km_rows<<<(unsigned)K, 256, 0, s>>>(X, D, d_init, K, tmp.codebook);
@@ -133,6 +132,7 @@ void kmeans(const float* X, int64_t n, int D, int K, const std::vector<int32_t>&
     GIFT_LAUNCHED("k_km_mean");
     GIFT_CUDA(cudaMemcpyAsync(h_off.data(), off, ((size_t)K + 1) * 8, cudaMemcpyDeviceToHost, s));
     GIFT_CUDA(cudaStreamSynchronize(s));
+    tmp.check_waits(s);
     std::vector<int32_t> empty;
     for (int c = 0; c < K; ++c)
       if (h_off[c + 1] == h_off[c]) empty.push_back(c);

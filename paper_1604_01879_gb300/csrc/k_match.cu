@@ -17,6 +17,8 @@
 // memory and adds one staged row per (query view, shape) entry. Then
 //   dW = dU^T Q + dV^T P,  dQ = dU W,  dP = dV W
 // as engine GEMMs on transposed two-part operands.
+#include <cstring>
+
 #include "gift_internal.cuh"
 #include "segmax.cuh"
 #include "tc_gemm.cuh"
@@ -366,8 +368,12 @@ __global__ __launch_bounds__(kGT, 1) void k_gather_views(const __grid_constant__
   for (int k = 0; k < 16; ++k)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[k][q] = 0.f;
+  bool whole = true;
   for (int s = s0; s < s1; ++s) {
-    if (!tc::mbar_wait(full0 + 8 * stage, phase, err, tc::kErrEpilogue)) break;
+    if (!tc::mbar_wait(full0 + 8 * stage, phase, err, tc::kErrEpilogue)) {
+      whole = false;
+      break;
+    }
     const uint8_t* buf = g_sm + (size_t)stage * bytes;
     const float4* vs = reinterpret_cast<const float4*>(buf) + lane;
     int p0, nps, nvs;
@@ -401,8 +407,14 @@ __global__ __launch_bounds__(kGT, 1) void k_gather_views(const __grid_constant__
       phase ^= 1;
     }
   }
+  if (!whole && lane == 0) report_wait(err);
   const int c = c0 + 4 * lane;
   if (c >= dout) return;
+  if (!whole) {  // partial sums do not pass for whole ones
+    for (int64_t i = i0 + 16 * w; i < min(nq, i0 + 16 * w + 16); ++i)
+      *reinterpret_cast<float4*>(Gp + ((int64_t)part * nq + i) * dout + c) = make_float4(NAN, NAN, NAN, NAN);
+    return;
+  }
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const int64_t i = i0 + 16 * w + k;
@@ -997,16 +1009,17 @@ Proj project(const void* q, int64_t nq, const void* p, int64_t nr, const void* W
   return P;
 }
 
-int32_t* device_offsets(const std::vector<int32_t>& h_qoff, Scratch& sc, cudaStream_t s) {
-  int32_t* d = sc.get<int32_t>(h_qoff.size());
-  GIFT_CUDA(cudaMemcpyAsync(d, h_qoff.data(), h_qoff.size() * 4, cudaMemcpyHostToDevice, s));
+// the call's wait flag and its offsets behind it, in one copy
+int* device_head(const std::vector<int32_t>& h_qoff, int32_t*& d_qoff, Scratch& sc, cudaStream_t s) {
+  const WaitFlag f{0, 0, thread_wait_word()};
+  constexpr size_t n = sizeof(WaitFlag) / 4;
+  std::vector<int32_t> h(n + h_qoff.size());
+  memcpy(h.data(), &f, sizeof(f));
+  std::copy(h_qoff.begin(), h_qoff.end(), h.begin() + n);
+  int32_t* d = sc.get<int32_t>(h.size());
+  GIFT_CUDA(cudaMemcpyAsync(d, h.data(), h.size() * 4, cudaMemcpyHostToDevice, s));  // (pageable: taken before the return)
+  d_qoff = d + n;
   return d;
-}
-
-int* device_flag(Scratch& sc, cudaStream_t s) {
-  int* f = sc.get<int>(1);
-  GIFT_CUDA(cudaMemsetAsync(f, 0, sizeof(int), s));
-  return f;
 }
 
 }  // namespace
@@ -1016,9 +1029,9 @@ void match_forward(const void* q, const std::vector<int32_t>& h_qoff, int32_t Bq
                    Scratch& sc, cudaStream_t s) {
   const int64_t nq = h_qoff[Bq];
   const int64_t nr = (int64_t)Np * nv;
-  int* err = device_flag(sc, s);
+  int32_t* d_qoff = nullptr;
+  int* err = device_head(h_qoff, d_qoff, sc, s);
   const Proj P = project(q, nq, p, nr, W, din, dout, dtype, true, err, sc, s);
-  int32_t* d_qoff = device_offsets(h_qoff, sc, s);
   segmax_tc(P.Uo.hi, P.Uo.lo, P.Uo.rows_alloc, P.uinv, P.Vo.hi, P.Vo.lo, P.Vo.rows_alloc, P.vinv, nr, nv, dout, d_qoff, h_qoff,
             Bq, S, argmax, err, sc, s);
 }
@@ -1028,9 +1041,9 @@ void match_backward(const void* q, const std::vector<int32_t>& h_qoff, int32_t B
                     const int16_t* argmax, float* dW, float* dQ, float* dP, Scratch& sc, cudaStream_t s) {
   const int64_t nq = h_qoff[Bq];
   const int64_t nr = (int64_t)Np * nv;
-  int* err = device_flag(sc, s);
+  int32_t* d_qoff = nullptr;
+  int* err = device_head(h_qoff, d_qoff, sc, s);
   const Proj P = project(q, nq, p, nr, W, din, dout, dtype, false, err, sc, s);
-  int32_t* d_qoff = device_offsets(h_qoff, sc, s);
   int32_t* vquery = sc.get<int32_t>(nq);
   float* vcoef = sc.get<float>(nq);
   k_view_query<<<(unsigned)Bq, 128, 0, s>>>(d_qoff, vquery, vcoef);

@@ -84,6 +84,7 @@ extern "C" gift_status gift_rerank_noalloc(gift_index* index, const int32_t* can
     GIFT_REQUIRE(gift::on_device(cand_ids) && gift::on_device(cand_scores) && gift::on_device(out_ids) &&
                      gift::on_device(out_sprime),
                  "gift_rerank_noalloc takes device buffers only (host buffers would need staging memory)");
+    ix.check_waits(stream);
     const size_t need = gift::sif_rerank_scratch_bytes(B, ix.sif_n, topk);
     if (need > gift::kScratchBytes)
       gift::fail(GIFT_EINVAL, "gift_rerank_noalloc needs " + std::to_string(need) +

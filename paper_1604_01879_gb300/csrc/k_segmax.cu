@@ -11,8 +11,9 @@ namespace {
 
 __global__ void k_segmax_reduce(const unsigned long long* __restrict__ cell, int64_t n_shapes,
                                 const int32_t* __restrict__ qoff, int32_t qb0, int32_t nq,
-                                int32_t view0, float* __restrict__ S, int16_t* __restrict__ argmax) {
+                                int32_t view0, float* __restrict__ S, int16_t* __restrict__ argmax, int* err) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx == 0) report_wait(err);
   if (idx >= (int64_t)nq * n_shapes) return;
   const int32_t b = qb0 + (int32_t)(idx / n_shapes);
   const int64_t p = idx % n_shapes;
@@ -29,10 +30,10 @@ __global__ void k_segmax_reduce(const unsigned long long* __restrict__ cell, int
 }  // namespace
 
 void segmax_reduce(const unsigned long long* cell, int64_t n_shapes, const int32_t* d_qoff, int32_t b0, int32_t nq,
-                   int32_t view0, float* S, int16_t* argmax, cudaStream_t s) {
+                   int32_t view0, float* S, int16_t* argmax, int* err, cudaStream_t s) {
   const int64_t work = (int64_t)nq * n_shapes;
   if (work <= 0) return;
-  k_segmax_reduce<<<(unsigned)cdiv(work, 256), 256, 0, s>>>(cell, n_shapes, d_qoff, b0, nq, view0, S, argmax);
+  k_segmax_reduce<<<(unsigned)cdiv(work, 256), 256, 0, s>>>(cell, n_shapes, d_qoff, b0, nq, view0, S, argmax, err);
   GIFT_LAUNCHED("k_segmax_reduce");
 }
 

@@ -35,10 +35,11 @@ struct ScoreRow {
 };
 
 __global__ __launch_bounds__(1024) void k_topk(const float* __restrict__ scores, int64_t n, int k,
-                                               int32_t* __restrict__ ids_out, float* __restrict__ val_out) {
+                                               int32_t* __restrict__ ids_out, float* __restrict__ val_out, int* err) {
   dep_begin();
   __shared__ sel::Smem sm;
   const int64_t b = blockIdx.x;
+  if (b == 0 && threadIdx.x == 0) report_wait(err);
   const int take = sel::select(sm, ScoreRow{scores + b * n}, n, n, k);
   for (int t = threadIdx.x; t < k; t += blockDim.x) {
     const bool ok = t < take;
@@ -110,8 +111,9 @@ __global__ __launch_bounds__(1024) void k_merge_rows(const int32_t* __restrict__
 __global__ __launch_bounds__(1024) void k_sort_candidates(const int32_t* __restrict__ ids,
                                                           const float* __restrict__ scores, int r, int k,
                                                           int32_t* __restrict__ ids_out,
-                                                          float* __restrict__ scores_out, int mode_ids) {
+                                                          float* __restrict__ scores_out, int mode_ids, int* err) {
   dep_begin();
+  if (blockIdx.x == 0 && threadIdx.x == 0) report_wait(err);
   __shared__ unsigned long long s_key[kMaxK];
   __shared__ uint32_t s_id[kMaxK];
   const int64_t b = blockIdx.x;
@@ -144,11 +146,11 @@ void merge_topk_rows(const int32_t* ids, const float* scores, int32_t B, int64_t
 }
 
 void topk_rows_f32(const float* scores, int32_t B, int64_t n, int32_t k, int32_t* ids_out, float* val_out,
-                   cudaStream_t s) {
+                   cudaStream_t s, int* err) {
   if (B <= 0 || k <= 0) return;
   GIFT_REQUIRE(k <= kMaxK, "top-k is limited to 1024");
   GIFT_REQUIRE(n < (int64_t)INT32_MAX, "row too long for top-k");
-  launch_dep(k_topk, dim3((unsigned)B), dim3(row_threads(n, B)), 0, s, scores, n, k, ids_out, val_out);
+  launch_dep(k_topk, dim3((unsigned)B), dim3(row_threads(n, B)), 0, s, scores, n, k, ids_out, val_out, err);
   GIFT_LAUNCHED("k_topk");
 }
 
@@ -163,18 +165,19 @@ void topk_rows_u64(const uint64_t* keys, int32_t B, int64_t n, int32_t k, int32_
 }
 
 void sort_candidates(const int32_t* ids, const float* scores, int32_t B, int32_t r, int32_t k,
-                     int32_t* ids_out, float* scores_out, cudaStream_t s) {
+                     int32_t* ids_out, float* scores_out, cudaStream_t s, int* err) {
   if (B <= 0 || k <= 0) return;
   GIFT_REQUIRE(r <= kMaxK, "candidate rows are limited to 1024");
   launch_dep(k_sort_candidates, dim3((unsigned)B), dim3(row_threads(r, B)), 0, s, ids, scores, r, k, ids_out,
-             scores_out, 0);
+             scores_out, 0, err);
   GIFT_LAUNCHED("k_sort_candidates");
 }
 
 void sort_ids_rows(const int32_t* ids, int32_t B, int32_t r, int32_t* out, cudaStream_t s) {
   if (B <= 0 || r <= 0) return;
   GIFT_REQUIRE(r <= kMaxK, "candidate rows are limited to 1024");
-  launch_dep(k_sort_candidates, dim3((unsigned)B), dim3(row_threads(r, B)), 0, s, ids, nullptr, r, r, out, nullptr, 1);
+  launch_dep(k_sort_candidates, dim3((unsigned)B), dim3(row_threads(r, B)), 0, s, ids, nullptr, r, r, out, nullptr, 1,
+             nullptr);
   GIFT_LAUNCHED("k_sort_ids");
 }
 

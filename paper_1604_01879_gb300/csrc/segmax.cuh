@@ -4,9 +4,10 @@
 
 namespace gift {
 
-// S[b, p] (and argmax) from the per-(view, shape) cells of queries [b0, b0 + nq)
+// S[b, p] (and argmax) from the per-(view, shape) cells of queries [b0, b0 + nq); err: the flag of the waits behind
+// them, reported
 void segmax_reduce(const unsigned long long* cell, int64_t n_shapes, const int32_t* d_qoff, int32_t b0, int32_t nq,
-                   int32_t view0, float* S, int16_t* argmax, cudaStream_t s);
+                   int32_t view0, float* S, int16_t* argmax, int* err, cudaStream_t s);
 
 // Segmented max on the tensor cores from two-part BF16 operands (rows of A =
 // query views, rows of B = database views, nv per shape); each operand has at

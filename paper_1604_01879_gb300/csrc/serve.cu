@@ -53,6 +53,7 @@ struct Slot {
   float* h_sc = nullptr;
   std::vector<std::shared_ptr<Request>> reqs;
   bool busy = false;
+  bool doubt = false;   // a kernel's wait gave up while the batch was in flight
   size_t reserved = 0;  // admitted device bytes of the batch in flight
 };
 
@@ -105,9 +106,21 @@ struct Server {
       ++failed;
     }
     s.reqs.clear();
-    s.busy = false;
+    s.busy = s.doubt = false;
     in_flight -= s.reserved;
     s.reserved = 0;
+  }
+
+  // a wait that gave up (WaitFlag) may have been any batch's in flight: none of them is delivered
+  void doubt_all() {
+    for (auto& s : slots) s.doubt |= s.busy;
+  }
+  void look_for_waits() {
+    try {
+      ix->check_waits(slots[0].stream);
+    } catch (const Error&) {
+      doubt_all();
+    }
   }
 
   // launch the batch held by slot s (outside the lock)
@@ -184,7 +197,9 @@ struct Server {
         if (!s.busy) continue;
         const cudaError_t e = cudaEventQuery(s.ev);
         if (e == cudaSuccess) {
-          finish(s);
+          look_for_waits();
+          if (s.doubt) fail_batch(s, GIFT_ETIMEOUT, "a kernel's wait gave up while the batch was in flight");
+          else finish(s);
           progressed = true;
         } else if (e != cudaErrorNotReady) {
           cudaGetLastError();
@@ -226,6 +241,7 @@ struct Server {
         const gift_status st = launch(s, msg);
         lk.lock();
         if (st != GIFT_OK) {
+          if (st == GIFT_ETIMEOUT) doubt_all();  // (found by the call, so not by the look at a completion)
           fail_batch(s, st, msg);
           cv_done.notify_all();
         }

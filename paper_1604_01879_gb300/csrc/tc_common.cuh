@@ -1,7 +1,8 @@
 // sm_100-family (sm_103a) building blocks in inline PTX: mbarriers, TMA tile
 // loads, tcgen05 MMA with TMEM accumulators, shared-memory and instruction
 // descriptors. Every wait is bounded: on timeout it records an error code in
-// a device flag and returns false, so a kernel can unwind instead of hanging.
+// a device flag and returns false, so a kernel can unwind instead of hanging
+// (report_wait tells the host).
 #pragma once
 #include <cuda.h>  // CUtensorMap and its enums (no driver library is linked)
 

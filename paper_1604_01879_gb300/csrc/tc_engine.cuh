@@ -79,6 +79,12 @@ struct swap_cross_of : std::false_type {};
 template <class P>
 struct swap_cross_of<P, std::void_t<decltype(P::SWAP_CROSS)>> : std::integral_constant<bool, P::SWAP_CROSS> {};
 
+// REPORT: no kernel of the call follows that reports a wait that gave up; the engine's warps do
+template <class P, class = void>
+struct report_of : std::false_type {};
+template <class P>
+struct report_of<P, std::void_t<decltype(P::REPORT)>> : std::integral_constant<bool, P::REPORT> {};
+
 template <class P, class = void>
 struct accs_of : std::integral_constant<int, 1> {};
 template <class P>
@@ -477,6 +483,8 @@ __global__ void __launch_bounds__(engine_threads<P>::value, 1)
       if (!ok) break;
       p.epi_end(it, ctx, m, my);
     }
+    if constexpr (report_of<P>::value)
+      if (!ok && lane == 0) report_wait(err);  // (any role's wait that gives up ends here too)
   }
   fence_before_sync();
   __syncthreads();

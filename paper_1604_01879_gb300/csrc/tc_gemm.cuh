@@ -16,6 +16,7 @@ namespace gift {
 template <int SPLIT_>
 struct GemmPolicy {
   static constexpr int TN = 128, NBUF = 4, STAGES = SPLIT_ == 1 ? 6 : SPLIT_ == 2 ? 4 : 3, SPLIT = SPLIT_, EB = 2;
+  static constexpr bool REPORT = true;
   static constexpr int kTurn = 20;  // row pitch of a turned piece: 16-byte rows, bank groups apart
   static constexpr int kWarpSmem = 32 * kTurn * 4;
   int64_t M, N;

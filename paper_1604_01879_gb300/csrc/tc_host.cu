@@ -1,5 +1,8 @@
 // Host helpers of the tcgen05 kernels: TMA tensor maps and device queries.
 #include <atomic>
+#include <cstdlib>
+#include <cstring>
+#include <mutex>
 
 #include "tc_common.cuh"
 
@@ -78,6 +81,66 @@ CUtensorMap make_tmap_f32(const void* base, uint64_t rows, uint64_t cols, uint32
                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) fail(GIFT_ECUDA, "cuTensorMapEncodeTiled failed with " + std::to_string((int)r));
   return m;
+}
+
+// Words of bounded waits, in blocks of a page or four that are registered with CUDA and kept for the life of the process
+// (ordinary memory, so that the host's reads need no context). Words given back are taken again, so there are as many
+// blocks as the most indices at a time need, usually one; threads have 1,024 words of their own (with more threads than
+// that, one may be told of another's).
+namespace {
+constexpr int kBlockWords = 4096, kThreadWords = 1024;
+std::mutex g_words_mu;
+std::vector<int*> g_free_words;
+int* g_thread_words = nullptr;
+int* new_words(int n) {
+  void* p = aligned_alloc(4096, n * sizeof(int));
+  if (p) memset(p, 0, n * sizeof(int));
+  if (!p || cudaHostRegister(p, n * sizeof(int), cudaHostRegisterPortable | cudaHostRegisterMapped) != cudaSuccess) {
+    cudaGetLastError();
+    free(p);
+    fail(GIFT_ENOMEM, "host memory for the wait words could not be registered");
+  }
+  return static_cast<int*>(p);
+}
+}  // namespace
+
+int* take_wait_word() {
+  std::lock_guard<std::mutex> lock(g_words_mu);
+  if (g_free_words.empty()) {
+    g_free_words.reserve(kBlockWords);
+    int* w = new_words(kBlockWords);
+    for (int i = 0; i < kBlockWords; ++i) g_free_words.push_back(w + i);
+  }
+  int* w = g_free_words.back();
+  g_free_words.pop_back();
+  __atomic_store_n(w, 0, __ATOMIC_RELAXED);
+  return w;
+}
+
+void give_wait_word(int* word) {
+  if (!word) return;
+  std::lock_guard<std::mutex> lock(g_words_mu);
+  g_free_words.push_back(word);
+}
+
+int* thread_wait_word() {
+  static std::atomic<unsigned> next{0};
+  thread_local int* mine = nullptr;
+  if (!mine) {
+    std::lock_guard<std::mutex> lock(g_words_mu);
+    if (!g_thread_words) g_thread_words = new_words(kThreadWords);
+    mine = g_thread_words + next.fetch_add(1) % kThreadWords;
+  }
+  return mine;
+}
+
+void check_wait_word(int* word, int* flag, cudaStream_t s) {
+  if (__atomic_load_n(word, __ATOMIC_ACQUIRE) == 0) return;
+  const int site = __atomic_exchange_n(word, 0, __ATOMIC_ACQ_REL);
+  if (site == 0) return;
+  if (flag) GIFT_CUDA(cudaMemsetAsync(flag, 0, sizeof(int), s));
+  fail(GIFT_ETIMEOUT, "a kernel's wait gave up (site " + std::to_string(site) +
+                          "): the results of this call, or of the calls before it that were not waited for, are not valid");
 }
 
 int device_sm_count() {

@@ -303,6 +303,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
       if (!ok) break;
       p.epi_end(it, ctx, m, my);
     }
+    if constexpr (report_of<P>::value)
+      if (!ok && lane == 0) report_wait(err);
   }
   if (!ok) {  // copies and MMAs of either CTA may still be on their way: let them land (bounded)
     const long long t0 = clock64();
