@@ -319,14 +319,14 @@ __device__ __forceinline__ bool df_less(float ah, float al, int ak, float bh, fl
 }
 
 // warp-wide best entry of (value desc, position asc) strictly after the key
-// (pv, pp) in that order; positions index the row's nch * kT kept entries
+// (pv, pp) in that order; positions index the row's nch * kT kept entries, those with no codeword left out
 __device__ __forceinline__ void next_best(const float* __restrict__ v, const int32_t* __restrict__ id, int tot,
-                                          float pv, int pp, int lane, float& bv, int& bp) {
+                                          int K, float pv, int pp, int lane, float& bv, int& bp) {
   bv = -INFINITY;
   bp = 0x7fffffff;
   for (int e = lane; e < tot; e += 32) {
     const float x = v[e];
-    if (id[e] == 0x7fffffff) continue;
+    if ((unsigned)id[e] >= (unsigned)K) continue;
     const bool after = x < pv || (x == pv && e > pp);
     if (after && (x > bv || (x == bv && e < bp))) {
       bv = x;
@@ -391,7 +391,7 @@ __global__ __launch_bounds__(256, WPR == 1 ? 4 : 1) void k_assign_refine(const f
   for (int a = 0; a < ma; ++a) {
     float bv;
     int bp;
-    next_best(v, id, tot, thr, tp, lane, bv, bp);
+    next_best(v, id, tot, K, thr, tp, lane, bv, bp);
     if (bp == 0x7fffffff) break;
     thr = bv;
     tp = bp;
@@ -406,7 +406,7 @@ __global__ __launch_bounds__(256, WPR == 1 ? 4 : 1) void k_assign_refine(const f
   bool full = xi == 0.f || found < ma;  // (fewer kept scores than ma only with non-finite inputs)
   for (int c = lane; c < nch; c += 32) {
     const int e = c * kT + kT - 1;
-    if (id[e] != 0x7fffffff && v[e] >= lim && min(tn, K - c * tn) > kT) full = true;
+    if ((unsigned)id[e] < (unsigned)K && v[e] >= lim && min(tn, K - c * tn) > kT) full = true;
   }
   full = __any_sync(kFull, full);
   if (!full && ma == 1) {
@@ -416,7 +416,7 @@ __global__ __launch_bounds__(256, WPR == 1 ? 4 : 1) void k_assign_refine(const f
     for (int base = 0; base < tot; base += 32) {
       const int e = base + lane;
       const int kk = e < tot ? id[e] : 0x7fffffff;
-      const bool take = e < tot && kk != 0x7fffffff && v[e] >= lim;
+      const bool take = e < tot && (unsigned)kk < (unsigned)K && v[e] >= lim;
       const unsigned m = __ballot_sync(kFull, take);
       if (m && cnt == 0) only = __shfl_sync(kFull, kk, __ffs(m) - 1);
       cnt += __popc(m);
@@ -464,7 +464,7 @@ __global__ __launch_bounds__(256, WPR == 1 ? 4 : 1) void k_assign_refine(const f
     for (int base = 0; base < tot; base += 32) {
       const int e = base + lane;
       const int kk = e < tot ? id[e] : 0x7fffffff;
-      unsigned m = __ballot_sync(kFull, e < tot && kk != 0x7fffffff && v[e] >= lim);
+      unsigned m = __ballot_sync(kFull, e < tot && (unsigned)kk < (unsigned)K && v[e] >= lim);
       while (m) {
         const int j = __ffs(m) - 1;
         m &= m - 1;
@@ -532,7 +532,7 @@ __global__ __launch_bounds__(256, WPR == 1 ? 4 : 1) void k_assign_refine(const f
       kk = e;
     } else {
       kk = e < tot ? id[e] : 0x7fffffff;
-      take = e < tot && kk != 0x7fffffff && v[e] >= lim;
+      take = e < tot && (unsigned)kk < (unsigned)K && v[e] >= lim;
     }
     unsigned mask = __ballot_sync(kFull, take);
     while (mask) {
@@ -552,7 +552,8 @@ __global__ __launch_bounds__(256, WPR == 1 ? 4 : 1) void k_assign_refine(const f
 #pragma unroll
     for (int a = 1; a < GIFT_MAX_MA; ++a)
       if (a == lane) out = Kx[a];
-    codes[r * ma + lane] = out;
+    // (no codeword is near a row that is not finite: any code of the vocabulary, for the lists are indexed by it)
+    codes[r * ma + lane] = (unsigned)out < (unsigned)K ? out : lane;
   }
 }
 
