@@ -669,7 +669,7 @@ __global__ void k_zero_cells(uint32_t* __restrict__ t, const int64_t* __restrict
 
 void fif_zero_table(const FifPlan& P, uint32_t* table, cudaStream_t s) {
   if (P.nslots <= 0) return;
-  launch_dep(k_zero_cells, dim3(1216), dim3(256), 0, s, table, P.runbase + P.nslots);  // 8 blocks per SM of a GB300
+  launch_dep(k_zero_cells, dim3((unsigned)(8 * device_sm_count())), dim3(256), 0, s, table, P.runbase + P.nslots);
   GIFT_LAUNCHED("k_zero_cells");
 }
 

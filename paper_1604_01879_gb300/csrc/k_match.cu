@@ -833,10 +833,9 @@ struct Operand {
 };
 
 // several: matrices whose split is left to be launched together (launch_splits)
-Operand make_operand(const void* x, int dtype, int64_t rows, int cols, bool force_split, Split4s& several, Scratch& sc,
-                     cudaStream_t s) {
+Operand make_operand(const void* x, int dtype, int64_t rows, int cols, Split4s& several, Scratch& sc, cudaStream_t s) {
   Operand o;
-  if (dtype != GIFT_F32 && !force_split && rows >= tc::kTM && reinterpret_cast<uintptr_t>(x) % 16 == 0) {
+  if (dtype != GIFT_F32 && rows >= tc::kTM && reinterpret_cast<uintptr_t>(x) % 16 == 0) {
     // a BF16 input is its own one-part operand: the tensor map covers its rows
     o.hi = const_cast<__nv_bfloat16*>(static_cast<const __nv_bfloat16*>(x));
     o.rows_alloc = rows;
@@ -845,8 +844,7 @@ Operand make_operand(const void* x, int dtype, int64_t rows, int cols, bool forc
   o.rows_alloc = rows + 128;
   const int64_t n = rows * cols;
   o.hi = sc.get<__nv_bfloat16>((size_t)o.rows_alloc * cols);
-  const bool split = dtype == GIFT_F32 || force_split;
-  if (split) o.lo = sc.get<__nv_bfloat16>((size_t)o.rows_alloc * cols);
+  if (dtype == GIFT_F32) o.lo = sc.get<__nv_bfloat16>((size_t)o.rows_alloc * cols);
   const bool vec = dtype == GIFT_F32 && n % 4 == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0 &&
                    reinterpret_cast<uintptr_t>(o.hi) % 8 == 0 && reinterpret_cast<uintptr_t>(o.lo) % 8 == 0;
   if (vec) {
@@ -978,9 +976,9 @@ Proj project(const void* q, int64_t nq, const void* p, int64_t nr, const void* W
   Proj P;
   if (W) {
     Split4s several;
-    const Operand Qo = make_operand(q, dtype, nq, din, false, several, sc, s);
-    const Operand Po = make_operand(p, dtype, nr, din, false, several, sc, s);
-    const Operand Wo = make_operand(W, dtype, dout, din, false, several, sc, s);
+    const Operand Qo = make_operand(q, dtype, nq, din, several, sc, s);
+    const Operand Po = make_operand(p, dtype, nr, din, several, sc, s);
+    const Operand Wo = make_operand(W, dtype, dout, din, several, sc, s);
     launch_splits(several, s);
     P.U = sc.get<float>((size_t)nq * dout);
     P.V = sc.get<float>((size_t)nr * dout);

@@ -16,8 +16,8 @@ constexpr int kMaxK = 1024;
 
 // threads for each of B rows of n pairs: a power of two in [64, 1024]
 int row_threads(int64_t n, int B) {
-  constexpr int kSms = 152;
-  const int most = n <= sel::kCap ? 1024 : B >= 4 * kSms ? 256 : B > kSms ? 512 : 1024;
+  const int sms = device_sm_count();
+  const int most = n <= sel::kCap ? 1024 : B >= 4 * sms ? 256 : B > sms ? 512 : 1024;
   int t = 64;
   while (t < most && 2 * (int64_t)t < n) t <<= 1;
   return t;
