@@ -270,7 +270,8 @@ __device__ void dist_df_batch(const float* __restrict__ x, const float* __restri
   }
 }
 
-// the same in plain FP32: relative error below (D / 32 + 8) 2^-24, a chain of D / 32 additions per lane and a tree
+// the same in plain FP32: relative error below (D / 32 + 8) 2^-24, a chain of D / 32 additions per lane and a tree, and
+// where squares underflow 2^-150 for each of them
 template <int WPR>
 __device__ void dist_f32_batch(const float* __restrict__ x, const float* __restrict__ cb, const int (&kc)[kBatch],
                                int n, int D, int lane, int sub, DfPart* part, float (&out)[kBatch]) {
@@ -498,12 +499,12 @@ __global__ __launch_bounds__(256, WPR == 1 ? 4 : 1) void k_assign_refine(const f
             kv[c] = kv[c + 1];
             kv[c + 1] = tk;
           }
-      // twice the error bound on either side of every gap that the codes' order rests on
+      // twice the error bound on either side of every gap that the codes' order rests on (1e-40: D 2^-150 up to D = 2^16)
       const float eps = (float)(D / 32 + 16) * 1.1920929e-7f;
       bool clear = true;
 #pragma unroll
       for (int c = 0; c + 1 < kBatch; ++c)
-        if (c < ma && c + 1 < n) clear = clear && dv[c + 1] - dv[c] > eps * (dv[c + 1] + dv[c]);
+        if (c < ma && c + 1 < n) clear = clear && dv[c + 1] - dv[c] > fmaf(eps, dv[c + 1] + dv[c], 1e-40f);
       if (clear) {
         if (lane < ma && sub == 0) {
           int out = kv[0];

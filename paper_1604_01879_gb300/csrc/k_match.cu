@@ -242,23 +242,21 @@ __device__ __forceinline__ void cp_async_wait() {
 // block's columns together with the entry records of the block's query views in those
 // shapes: a row of V leaves L2 once per block instead of once per entry, and each entry
 // is one broadcast record read, one 512-byte shared-memory read and four multiply-adds.
-// The stages are a ring of up to eight, filled by one thread of a 17th warp (a TMA tile of
+// The stages are a ring of four to six, filled by one thread of a 17th warp (a TMA tile of
 // V and a bulk copy per shape's records) and freed warp by warp, so the warps drift apart
 // and none issues copies: what is left is the 512-byte reads (137 GB at full size, 16,384 x 4,096
 // entries of 512 columns: 3.4 ms at shared memory's rate), the records' and the copies' share of
-// it, and their issue: 7.41 ms with copies by every thread and a barrier per step, 6.59 now.
+// it, and their issue: 7.41 ms with copies by every thread and a barrier per step, 6.35 now.
 // A step is up to kGShapes whole shapes of at most 64 views together, or one 64-view piece of a larger shape. The
 // steps may be split into parts (blockIdx.z) whose partial sums k_tangent adds in
 // part order: the result does not depend on the launch.
-constexpr int kGWarps = 16, kGT = 32 * (kGWarps + 1), kGRows = 256, kGCols = 128, kGStages = 8, kGViews = 64, kGShapes = 8;
+constexpr int kGWarps = 16, kGT = 32 * (kGWarps + 1), kGRows = 256, kGCols = 128, kGViews = 64, kGShapes = 8;
 constexpr int kGRecOff = (kGViews + 1) * kGCols * 4;  // 33,280: V rows + one zero row, then records [shapes][kGRows]
 constexpr int kGSmem = 227 * 1024;
 static_assert(kGRecOff % 128 == 0, "stage alignment");
 // bytes of a stage and stages of the ring for steps of `shapes` record rows
 __host__ __device__ constexpr int g_stage_bytes(int shapes) { return kGRecOff + shapes * kGRows * 8; }
-__host__ __device__ constexpr int g_stages(int shapes) {
-  return (kGSmem - 1024) / g_stage_bytes(shapes) < kGStages ? (kGSmem - 1024) / g_stage_bytes(shapes) : kGStages;
-}
+__host__ __device__ constexpr int g_stages(int shapes) { return (kGSmem - 1024) / g_stage_bytes(shapes); }
 
 struct GatherSteps {
   int spc;  // whole shapes per step (N_v <= 64); 0: 64-view pieces of one shape
@@ -312,7 +310,7 @@ __global__ __launch_bounds__(kGT, 1) void k_gather_views(const __grid_constant__
   const int shapes = st.spc > 0 ? st.spc : 1;
   const int bytes = g_stage_bytes(shapes), ring = g_stages(shapes);
   uint64_t* bars = reinterpret_cast<uint64_t*>(g_sm + (size_t)ring * bytes);
-  const uint32_t full0 = tc::smem_u32(bars), empty0 = full0 + 8 * kGStages;
+  const uint32_t full0 = tc::smem_u32(bars), empty0 = full0 + 8 * ring;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int64_t i0 = (int64_t)blockIdx.x * kGRows;
   const int c0 = blockIdx.y * kGCols;

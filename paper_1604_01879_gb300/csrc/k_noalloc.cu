@@ -5,10 +5,10 @@
 // serving framework's caching pool) would see the allocation fail, and a
 // latency-critical loop must not enter the CUDA allocator at all (freeing
 // device memory can synchronise the device). For them, gift_rerank_noalloc
-// runs the same re-ranking kernels as gift_rerank on one fixed scratch
-// buffer that lives in this file as a device variable: it is created with
-// the library's module on every device that uses it and is held until the
-// process exits.
+// runs the re-rank on dense rows of all shapes, which gift_rerank takes only for
+// long walks of few queries, on one fixed scratch buffer that lives in this file
+// as a device variable: it is created with the library's module on every device
+// that uses it and is held until the process exits.
 //
 // Host code cannot use the name of a __device__ variable as an address; the
 // first call on each device asks the runtime for the variable's device

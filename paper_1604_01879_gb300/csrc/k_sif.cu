@@ -13,8 +13,8 @@
 // S' = num / (||F_q||_1 + ||F_p||_1 - num) (Eq. 14) in FP32, and the final
 // order (S' desc, S desc, id asc) is a top-k over 64-bit keys
 // (key(S') << 32 | key(S)) with ties to the lower id. One block per query does it
-// all in shared memory (k_rerank_reach); the re-rank on caller-provided scratch
-// keeps dense rows.
+// all in shared memory (k_rerank_reach), or, for long walks of few queries and on
+// caller-provided scratch, kernels over dense rows of all shapes (dense_rerank).
 //
 // Two measures (Sec. 2.4, Eqs. 9-11): a block per shape (database or query)
 // gathers the activations that make up its two contextual activations — its
