@@ -266,7 +266,7 @@ def roofline(cfg, st, scan_pairs, scan_bytes, rescore_bytes, assign_rows, peaks,
     if not table:  # no engine kernel ran (FP32 store scanned on the CUDA cores, no tensor-core quantiser)
         return None
     dom = max(table, key=lambda k: table[k]["ms"])
-    src_hash = kernel_source_hash(kernels[dom][3] + ["tc_engine.cuh", "tc_common.cuh"])
+    src_hash = kernel_source_hash(kernels[dom][3] + ["tc_engine.cuh", "tc_pair.cuh", "tc_common.cuh"])
     per_unit, unit, capture = recorded_traffic(dom, src_hash) if with_traffic else (None, None, None)
     # units of this launch: rows of the touched lists (scan, fused pass), rows the rescore reads,
     # rows quantised
