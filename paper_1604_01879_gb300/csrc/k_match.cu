@@ -257,6 +257,7 @@ static_assert(kGRecOff % 128 == 0, "stage alignment");
 // bytes of a stage and stages of the ring for steps of `shapes` record rows
 __host__ __device__ constexpr int g_stage_bytes(int shapes) { return kGRecOff + shapes * kGRows * 8; }
 __host__ __device__ constexpr int g_stages(int shapes) { return (kGSmem - 1024) / g_stage_bytes(shapes); }
+constexpr int kGStages = g_stages(1);  // the most: barriers a constant apart (a backward pass 19.6 ms, 20.2 with 8 * ring)
 
 struct GatherSteps {
   int spc;  // whole shapes per step (N_v <= 64); 0: 64-view pieces of one shape
@@ -310,7 +311,7 @@ __global__ __launch_bounds__(kGT, 1) void k_gather_views(const __grid_constant__
   const int shapes = st.spc > 0 ? st.spc : 1;
   const int bytes = g_stage_bytes(shapes), ring = g_stages(shapes);
   uint64_t* bars = reinterpret_cast<uint64_t*>(g_sm + (size_t)ring * bytes);
-  const uint32_t full0 = tc::smem_u32(bars), empty0 = full0 + 8 * ring;
+  const uint32_t full0 = tc::smem_u32(bars), empty0 = full0 + 8 * kGStages;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int64_t i0 = (int64_t)blockIdx.x * kGRows;
   const int c0 = blockIdx.y * kGCols;

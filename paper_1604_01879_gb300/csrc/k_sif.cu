@@ -634,11 +634,11 @@ constexpr int kHalf = 71680, kWhole = 188416;  // bytes of a table: two blocks s
 // shapes, or 4,480 hash slots, which the shapes a query reaches should leave a quarter empty. Heavier walks (of more
 // than twice those slots of pairs) take a whole SM's table of up to 15,680 shapes, which spares them the probing.
 //
-// One block's walk takes 0.24 to 0.6 ns a pair by its threads, however many SMs stand idle; on dense rows a query's coordinates spread over
-// the SMs, at a price in launches and in passes over all N shapes: they take over where the walks are long and the
-// queries few (both sides in microseconds, from the figures below), and where a query reaches more shapes than a table
-// holds, unless every SM has a query to walk. Measured, whole calls in us (one block, dense rows; neighbours drawn from
-// all shapes unless said):
+// One block's walk takes 0.24 to 0.6 ns a pair by its threads, however many SMs stand idle; on dense rows a query's
+// coordinates spread over the SMs, at a price in launches and in passes over all N shapes: they take over where the
+// walks are long and the queries few (both sides in microseconds, from the figures below), and where a query reaches
+// more shapes than a table holds, unless every SM has a query to walk. Measured, whole calls in us (one block, dense
+// rows; neighbours drawn from all shapes unless said):
 //   200,000 shapes, k1 =    50, 1 query     62   187        12,000 shapes, k1 = 1,000,     1 query     267    115
 //   200,000, k1 = 200 in classes, 64        61   316        12,000, k1 = 1,000,           64           278    357
 //   200,000, k1 = 1,000,          1      1,034   276        12,000, two measures, k2 = 40, 1         2,811    337
