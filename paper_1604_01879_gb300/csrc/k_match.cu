@@ -246,7 +246,7 @@ __device__ __forceinline__ void cp_async_wait() {
 // V and a bulk copy per shape's records) and freed warp by warp, so the warps drift apart
 // and none issues copies: what is left is the 512-byte reads (137 GB at full size, 16,384 x 4,096
 // entries of 512 columns: 3.4 ms at shared memory's rate), the records' and the copies' share of
-// it, and their issue: 7.41 ms with copies by every thread and a barrier per step, 6.35 now.
+// it, and their issue: 7.41 ms with copies by every thread and a barrier per step, 5.75 now.
 // A step is up to kGShapes whole shapes of at most 64 views together, or one 64-view piece of a larger shape. The
 // steps may be split into parts (blockIdx.z) whose partial sums k_tangent adds in
 // part order: the result does not depend on the launch.
@@ -257,7 +257,7 @@ static_assert(kGRecOff % 128 == 0, "stage alignment");
 // bytes of a stage and stages of the ring for steps of `shapes` record rows
 __host__ __device__ constexpr int g_stage_bytes(int shapes) { return kGRecOff + shapes * kGRows * 8; }
 __host__ __device__ constexpr int g_stages(int shapes) { return (kGSmem - 1024) / g_stage_bytes(shapes); }
-constexpr int kGStages = g_stages(1);  // the most: barriers a constant apart (a backward pass 19.6 ms, 20.2 with 8 * ring)
+constexpr int kGStages = g_stages(1);  // the most: barriers a constant apart (5.75 ms; 6.35 with 8 * ring)
 
 struct GatherSteps {
   int spc;  // whole shapes per step (N_v <= 64); 0: 64-view pieces of one shape
